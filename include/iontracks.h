@@ -67,7 +67,7 @@ extern "C" {
 #define IT_UPWIND       1
 /* it_params.kernel: which step kernel runs (all are CUDA). */
 #define IT_KERNEL_AUTO   0   /* z-march kernel where the grid allows, else simple */
-#define IT_KERNEL_SIMPLE 1   /* one thread per cell, global loads */
+#define IT_KERNEL_SIMPLE 1   /* one thread per column of cells, global loads (any grid and type) */
 #define IT_KERNEL_ZMARCH 2   /* TMA-staged z-planes in shared memory (FP32, nx % 4 == 0) */
 #define IT_KERNEL_ZMARCH2 3  /* as IT_KERNEL_ZMARCH, two time steps per launch (temporal blocking
                                 of depth 2; nx/4 must divide 256 or 512 threads); densities are
@@ -494,10 +494,9 @@ int it_mlp_destroy(it_mlp *net);
  * `stream` (a cudaStream_t, NULL = the legacy default stream).
  * The per-block tally partials live in one static device array of
  * IT_NOALLOC_MAX_BLOCKS x 10 doubles (160 KiB on each device that loads the
- * library, kept until exit); a device that would need more blocks is
- * rejected with IT_EINVAL.  The first call on a device looks up the array's
+ * library, kept until exit); a step takes at most that many blocks.  The first call on a device looks up the array's
  * address (make it before any stream capture).  All calls share the array
- * and clear the part they use, so calls that overlap on the GPU race:
+ * and overwrite the part they use, so calls that overlap on the GPU race:
  * order them on one stream.  Allocates nothing: no cudaMalloc, cudaFree or
  * allocating library call. */
 int it_step_noalloc(it_grid g, double dx_cm, double dt_s, const it_params *p,

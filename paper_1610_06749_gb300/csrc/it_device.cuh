@@ -31,6 +31,17 @@ __device__ __forceinline__ void block_sum(double (&v)[N], double *smem /* [32][N
     }
 }
 
+// Sum of quantity q of n records of `width` doubles by one warp, in a fixed
+// order: lane l adds records l, l + 32, ..., then the shuffle tree (the sum
+// is lane 0's).
+__device__ __forceinline__ double warp_strided_sum(const double *__restrict__ v, int n, int q, int width, int lane) {
+    double t = 0.0;
+    for (int b = lane; b < n; b += 32) t += v[(size_t)b * width + q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    return t;
+}
+
 // One cell of the update as an increment in flux form:
 //   n + [wd ((l + r) + (u + d) - 4 n) + wzm (zm - n) + wzp (zp - n) - adt rr]
 // (wd = wx = wy: the cells are cubes).  Every transport term is a weight

@@ -189,8 +189,9 @@ int launch_deposit(it_ctx *c, int64_t n, cudaStream_t s);   // tracks already in
 int launch_zero(void *p, size_t bytes, cudaStream_t s);
 int launch_deposit_angled(it_ctx *c, const double *d_tr, int64_t n, double *d_part, int nblocks, cudaStream_t s);
 int simple_grid(const it_ctx *c);
+int simple_grid_f32(int nx, int ny, int nz);
 int launch_step_simple_raw_f32(const float *ip, const float *im, float *op, float *om, int nx, int ny, int nz,
-                               const Coef<float> &cf, bool periodic, double *slots, int nblocks, cudaStream_t s);
+                               const Coef<float> &cf, bool periodic, double *slots, cudaStream_t s);
 int launch_monitor_raw_f32(const float *p, const float *m, size_t cells, double vol, double *mon, int nblocks,
                            cudaStream_t s);
 int validate_step_args(const it_params *p, it_grid g, double dx, double dt);

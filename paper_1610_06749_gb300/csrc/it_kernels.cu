@@ -8,6 +8,7 @@
 // diffusion on three axes, -alpha n+ n- from the old level), written in flux
 // form so the tallies of what crosses the electrode faces close the charge
 // balance.
+#include <algorithm>
 #include <cmath>
 
 #include "it_device.cuh"
@@ -16,111 +17,312 @@
 namespace itk {
 
 // ---------------------------------------------------------------------------
-// simple step: one thread per cell, neighbours read through L1/L2
+// simple step: any grid and type, neighbours read through L1/L2
 // ---------------------------------------------------------------------------
-template <typename T, bool PERIODIC>
-__global__ void __launch_bounds__(256)
-step_simple_kernel(const T *__restrict__ ip, const T *__restrict__ im, T *__restrict__ op,
-                   T *__restrict__ om, int nx, int ny, int nz, Coef<T> c,
-                   double *__restrict__ slots) {
-    __shared__ double red[32 * 9];
-    const size_t plane = (size_t)nx * ny;
-    const size_t total = plane * nz;
-    double acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(idx % nx);
-        const size_t r = idx / nx;
-        const int j = (int)(r % ny);
-        const int k = (int)(r / ny);
-        const size_t ixm = (i > 0) ? idx - 1 : idx + (nx - 1);
-        const size_t ixp = (i < nx - 1) ? idx + 1 : idx - (nx - 1);
-        const size_t iym = (j > 0) ? idx - nx : idx + (size_t)(ny - 1) * nx;
-        const size_t iyp = (j < ny - 1) ? idx + nx : idx - (size_t)(ny - 1) * nx;
-        const T p0 = ip[idx], m0 = im[idx];
-        const T rr = p0 * m0;
-        acc[0] += (double)rr;
-        const int cx = (i == 0) + (i == nx - 1);
-        const int cy = (j == 0) + (j == ny - 1);
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            const T *in = s ? im : ip;
-            const T n0 = s ? m0 : p0;
-            const T xm = (PERIODIC || i > 0) ? in[ixm] : T(0);
-            const T xp = (PERIODIC || i < nx - 1) ? in[ixp] : T(0);
-            const T ym = (PERIODIC || j > 0) ? in[iym] : T(0);
-            const T yp = (PERIODIC || j < ny - 1) ? in[iyp] : T(0);
-            const T zm = (k > 0) ? in[idx - plane] : T(0);
-            const T zp = (k < nz - 1) ? in[idx + plane] : T(0);
-            T v = upd7(n0, xm, xp, ym, yp, zm, zp, rr, c.wx[s], c.wzm[s], c.wzp[s], c.adt);
-            if (c.sc_on) {
-                v = add_sc(v, c.sc[s], n0, p0, m0);
-                acc[7 + s] += (double)(n0 * (p0 - m0));
-            }
-            (s ? om : op)[idx] = v;
-            if (k == 0) acc[1 + s] += (double)n0;
-            if (k == nz - 1) acc[3 + s] += (double)n0;
-            if (!PERIODIC && (cx | cy))
-                acc[5 + s] += (double)n0 * (cx * c.latx_f[s] + cy * c.laty_f[s]);
-        }
+// A thread owns one column of the flattened x-y plane (cell q of nx ny) and
+// marches it over a chunk of z planes, so the z neighbours stay in registers
+// and the cell's position costs one division per chunk; a block is 128
+// neighbouring columns, whatever nx is.
+//
+// What bounds it: FP64 states run at the FP64 rate of this GPU (two lanes per
+// SM and clock: 24 operations per cell are 10 us of a 48x48x100 step), FP32
+// states at the L1 wavefronts of ten scalar loads and two stores per cell.
+// The tallies therefore stay off the FP64 pipe: FP32 states sum in FP32 with
+// the rounding error of every addition carried along (CompSum), the block
+// reduction runs in the same form and one lane converts its result; faces
+// (electrodes, absorbing sides) are only reduced by blocks that touch them.
+// With one cell per thread, an FP64 addition per cell and a nine-value FP64
+// shuffle reduction per warp, the earlier form took 49 us per step on
+// 48x48x100 in FP64 and 224 us on 301x173x97 in FP32; this one takes 16.2
+// and 31 us.  Eight blocks per SM (64 registers) with the plane above loaded
+// one plane ahead: ten blocks without that took 34.6 us on 301x173x97.
+constexpr int SK_THREADS = 128;
+constexpr int SK_BLOCKS_F32 = 8, SK_BLOCKS_F64 = 6;   // resident blocks per SM
+
+// FP32 sum that carries the rounding error of each addition (Knuth's
+// two-sum), so a sum of some hundred terms keeps about 46 bits: as good as
+// FP64 for terms that are FP32 products.  A sum that overflows or meets a
+// NaN is returned as it is.
+struct CompSum {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float s = __fadd_rn(hi, x);
+        const float b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+        hi = s;
     }
-    block_sum<9>(acc, red);
-    if (threadIdx.x == 0) {
-        double *sl = slots + (size_t)blockIdx.x * NT;
-        sl[0] += acc[0] * c.rec_f;
-        sl[1] += acc[1] * c.anode_f[0];
-        sl[2] += acc[2] * c.anode_f[1];
-        sl[3] += acc[3] * c.cathode_f[0];
-        sl[4] += acc[4] * c.cathode_f[1];
-        sl[5] += acc[5];
-        sl[6] += acc[6];
-        sl[7] += acc[7] * c.sc_f[0];
-        sl[8] += acc[8] * c.sc_f[1];
+    __device__ __forceinline__ void add(const CompSum &o) {
+        const float l = o.lo;
+        add(o.hi);
+        lo = __fadd_rn(lo, l);
+    }
+    __device__ __forceinline__ void scale(float w) {   // w a small whole number
+        const float p = __fmul_rn(hi, w);
+        lo = __fmaf_rn(lo, w, __fmaf_rn(hi, w, -p));
+        hi = p;
+    }
+    __device__ __forceinline__ double value() const {
+        return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+    }
+    __device__ __forceinline__ CompSum down(int o) const {
+        CompSum r;
+        r.hi = __shfl_down_sync(0xffffffffu, hi, o);
+        r.lo = __shfl_down_sync(0xffffffffu, lo, o);
+        return r;
+    }
+};
+
+// the same for FP64 states: a plain FP64 sum
+struct PlainSum {
+    double hi = 0.0;
+    __device__ __forceinline__ void add(double x) { hi += x; }
+    __device__ __forceinline__ void add(const PlainSum &o) { hi += o.hi; }
+    __device__ __forceinline__ void scale(double w) { hi *= w; }
+    __device__ __forceinline__ double value() const { return hi; }
+    __device__ __forceinline__ PlainSum down(int o) const {
+        PlainSum r;
+        r.hi = __shfl_down_sync(0xffffffffu, hi, o);
+        return r;
+    }
+};
+
+template <typename T>
+struct SumOf { using type = PlainSum; };
+template <>
+struct SumOf<float> { using type = CompSum; };
+
+// the operations of add_sc, with the product kept for the tally
+__device__ __forceinline__ float sk_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double sk_mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float sk_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double sk_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// Block sums of N values in a fixed order, added to tot[at ..]: value v is
+// reduced by warp v mod 4 (four columns per lane, then shuffles) and
+// converted to FP64 by its lane 0.
+template <int N, typename Sum>
+__device__ __forceinline__ void sk_reduce(const Sum (&v)[N], Sum (*buf)[SK_THREADS], double *tot, int at) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < N; ++q) buf[q][tid] = v[q];
+    __syncthreads();
+#pragma unroll
+    for (int q0 = 0; q0 < N; q0 += SK_THREADS / 32) {
+        const int q = q0 + warp;
+        if (q < N) {
+            Sum s = buf[q][lane];
+#pragma unroll
+            for (int r = 1; r < SK_THREADS / 32; ++r) s.add(buf[q][lane + 32 * r]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s.add(s.down(o));
+            if (lane == 0) tot[at + q] += s.value();
+        }
     }
 }
 
-int simple_grid(const it_ctx *c) {
-    const size_t blocks = (c->g.cells() + 255) / 256;
+// Work unit u: column block u mod npb, z chunk u / npb of nchunk.  A block
+// takes units blockIdx.x, blockIdx.x + gridDim.x, ...; its tally slot is
+// added to (add = 1) or replaced (add = 0).
+template <typename T, typename Idx, bool PERIODIC, bool SC>
+__global__ void __launch_bounds__(SK_THREADS, (sizeof(T) == 4 ? SK_BLOCKS_F32 : SK_BLOCKS_F64))
+step_simple_kernel(const T *__restrict__ ip, const T *__restrict__ im, T *__restrict__ op, T *__restrict__ om, int nx,
+                   int ny, int nz, unsigned npb, unsigned nchunk, const Coef<T> c, double *__restrict__ slots,
+                   int add) {
+    using Sum = typename SumOf<T>::type;
+    constexpr int NV = 1 + (PERIODIC ? 0 : 2) + (SC ? 2 : 0);   // values reduced for every unit
+    __shared__ double raw[5 * SK_THREADS];
+    Sum(*buf)[SK_THREADS] = reinterpret_cast<Sum(*)[SK_THREADS]>(raw);
+    static_assert(sizeof(Sum) == sizeof(double), "reduction scratch");
+    __shared__ double tot[9];   // order of sk_reduce: rec, lateral +/-, space charge +/-, then anode, cathode
+    constexpr int AN = 5, CA = 7;
+    const int tid = threadIdx.x;
+    if (tid < 9) tot[tid] = 0.0;
+    const Idx plane = (Idx)nx * (Idx)ny;
+    const unsigned long long units = (unsigned long long)npb * nchunk;
+    for (unsigned long long u = blockIdx.x; u < units; u += gridDim.x) {
+        const unsigned pb = (unsigned)(u % npb), ch = (unsigned)(u / npb);
+        const int k0 = (int)((long long)nz * ch / nchunk), k1 = (int)((long long)nz * (ch + 1) / nchunk);
+        Idx q = (Idx)pb * SK_THREADS + tid;
+        const bool act = q < plane;
+        if (!act) q = plane - 1;   // columns past the plane repeat the last one and store nothing
+        const int j = (int)(q / (Idx)nx), i = (int)(q - (Idx)j * (Idx)nx);
+        // neighbour columns (wrapped; absorbing faces hold zero instead)
+        const Idx qxm = i > 0 ? q - 1 : q + (Idx)(nx - 1), qxp = i < nx - 1 ? q + 1 : q - (Idx)(nx - 1);
+        const Idx qym = j > 0 ? q - (Idx)nx : q + (Idx)(ny - 1) * (Idx)nx;
+        const Idx qyp = j < ny - 1 ? q + (Idx)nx : q - (Idx)(ny - 1) * (Idx)nx;
+        const bool hxm = PERIODIC || i > 0, hxp = PERIODIC || i < nx - 1;
+        const bool hym = PERIODIC || j > 0, hyp = PERIODIC || j < ny - 1;
+        Sum v[NV];
+        Idx base = (Idx)k0 * plane;
+        T zm[2], n[2];
+        T zp[2];   // loaded one plane ahead
+        zm[0] = k0 > 0 ? ip[base - plane + q] : T(0);
+        zm[1] = k0 > 0 ? im[base - plane + q] : T(0);
+        n[0] = ip[base + q];
+        n[1] = im[base + q];
+        zp[0] = k0 + 1 < nz ? ip[base + plane + q] : T(0);
+        zp[1] = k0 + 1 < nz ? im[base + plane + q] : T(0);
+        const int sides = (i == 0) + (i == nx - 1) + (j == 0) + (j == ny - 1);
+        const T first[2] = {n[0], n[1]};   // the chunk's first plane (anode tally)
+        T last[2] = {n[0], n[1]};
+#pragma unroll 2
+        for (int k = k0; k < k1; ++k, base += plane) {
+            const T rr = n[0] * n[1];
+            T z2[2], w[2];
+            const bool more = k + 1 < k1 && k + 2 < nz;
+            z2[0] = more ? ip[base + 2 * plane + q] : T(0);
+            z2[1] = more ? im[base + 2 * plane + q] : T(0);
+            const T d = SC ? n[0] - n[1] : T(0);
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const T *in = s ? im : ip;
+                const T xm = hxm ? in[base + qxm] : T(0), xp = hxp ? in[base + qxp] : T(0);
+                const T ym = hym ? in[base + qym] : T(0), yp = hyp ? in[base + qyp] : T(0);
+                w[s] = upd7(n[s], xm, xp, ym, yp, zm[s], zp[s], rr, c.wx[s], c.wzm[s], c.wzp[s], c.adt);
+                if constexpr (SC) {
+                    const T t = sk_mul(n[s], d);
+                    w[s] = sk_fma(c.sc[s], t, w[s]);
+                    v[NV - 2 + s].add(t);
+                }
+                if constexpr (!PERIODIC) {
+                    if (sides > 0) v[1 + s].add(n[s]);
+                }
+            }
+            v[0].add(rr);
+            if (act) {
+                op[base + q] = w[0];
+                om[base + q] = w[1];
+            }
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                last[s] = n[s];
+                zm[s] = n[s];
+                n[s] = zp[s];
+                zp[s] = z2[s];
+            }
+        }
+        // lateral faces: what leaves through the x and y sides of this column
+        if constexpr (!PERIODIC) {
+            v[1].scale((T)sides);
+            v[2].scale((T)sides);
+        }
+        if (!act) {
+#pragma unroll
+            for (int t = 0; t < NV; ++t) v[t] = Sum{};
+        }
+        sk_reduce<NV>(v, buf, tot, 0);
+        if (k0 == 0) {
+            Sum e[2];
+            if (act) { e[0].add(first[0]); e[1].add(first[1]); }
+            sk_reduce<2>(e, buf, tot, AN);
+        }
+        if (k1 == nz) {
+            Sum e[2];
+            if (act) { e[0].add(last[0]); e[1].add(last[1]); }
+            sk_reduce<2>(e, buf, tot, CA);
+        }
+    }
+    __syncthreads();
+    if (tid < 9) {   // tally tid of the slot
+        double t = 0.0;
+        if (tid == 0) t = tot[0] * c.rec_f;
+        else if (tid < 3) t = tot[AN + tid - 1] * c.anode_f[tid - 1];
+        else if (tid < 5) t = tot[CA + tid - 3] * c.cathode_f[tid - 3];
+        // x and y weights are equal for dx = dy (latx_f == laty_f)
+        else if (tid < 7) t = PERIODIC ? 0.0 : tot[1 + tid - 5] * c.latx_f[tid - 5];
+        else t = SC ? tot[NV - 2 + tid - 7] * c.sc_f[tid - 7] : 0.0;
+        double *sl = slots + (size_t)blockIdx.x * NT + tid;
+        *sl = add ? *sl + t : t;
+    }
+}
+
+// Chunks per column and blocks of a launch, by the fitted time of a split.
+// FP64: the FP64 pipe of an SM works off its units one after another, 2300
+// cycles per plane of a unit and 0.45 planes for a unit's start and
+// reduction; a single block per SM leaves it a tenth idle.  FP32: a resident
+// block takes 600 cycles per plane plus 75 for every block it shares the SM
+// with, each round of units starts with two planes of loads.  (48x48x100 in
+// FP64: 16.2 us at 25 chunks, 17.7 at 8, 116 at one; 301x173x97 in FP32
+// 30.7-33 us at 2 to 9 chunks, 37.9 at 20; 200x111x280 28.0 us at 6, 54 at
+// 2, 32 at 40.)
+struct SkShape { unsigned npb, nchunk, grid; };
+static SkShape sk_shape(int nx, int ny, int nz, bool fp64) {
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t cap = (size_t)sms * 8;
-    return (int)(blocks < cap ? (blocks > 0 ? blocks : 1) : cap);
+    const unsigned long long plane = (unsigned long long)nx * ny;
+    const unsigned long long npb = (plane + SK_THREADS - 1) / SK_THREADS;
+    const unsigned long long resident = std::min<unsigned long long>(
+        (unsigned long long)sms * (fp64 ? SK_BLOCKS_F64 : SK_BLOCKS_F32), IT_NOALLOC_MAX_BLOCKS);
+    unsigned best = 1;
+    double best_cost = 1e300;
+    for (unsigned c = 1; c <= (unsigned)nz; c += std::max(1u, c / 16)) {   // a few hundred splits at most
+        const unsigned long long units = npb * c;
+        if (c > 1 && units > 8 * resident) break;
+        const double kc = (nz + c - 1) / c;
+        double cost;
+        if (fp64) {
+            const double per_sm = (double)((units + sms - 1) / sms);
+            cost = per_sm * (kc + 0.45) * 2300.0 * (per_sm == 1.0 ? 1.1 : 1.0) + (kc + 2.0) * 300.0;
+        } else {
+            const unsigned long long rem = units % resident;
+            cost = (double)(units / resident) * (kc + 2.0) * (600.0 + 75.0 * SK_BLOCKS_F32);
+            if (rem) cost += (kc + 2.0) * (600.0 + 75.0 * (double)((rem + sms - 1) / sms));
+        }
+        if (cost < 0.99 * best_cost) {
+            best_cost = cost;
+            best = c;
+        }
+    }
+    const unsigned long long units = npb * best;
+    return SkShape{(unsigned)npb, best, (unsigned)std::min(units, resident)};
+}
+
+int simple_grid(const it_ctx *c) { return (int)sk_shape(c->g.nx, c->g.ny, c->g.nz, c->prec == IT_FP64).grid; }
+
+int simple_grid_f32(int nx, int ny, int nz) { return (int)sk_shape(nx, ny, nz, false).grid; }
+
+template <typename T>
+static int sk_launch(const T *ip, const T *im, T *op, T *om, int nx, int ny, int nz, const Coef<T> &cf, bool periodic,
+                     double *slots, int add, cudaStream_t s) {
+    const SkShape h = sk_shape(nx, ny, nz, sizeof(T) == 8);
+    // 32-bit element offsets where they reach (a neighbour plane beyond the
+    // last is never formed: its load is predicated off, its offset may wrap)
+    const bool small = (unsigned long long)nx * ny * nz <= 0xffffffffull - 2 * SK_THREADS;
+    const bool sc = cf.sc_on != 0;
+    auto go = [&](auto *k) { k<<<h.grid, SK_THREADS, 0, s>>>(ip, im, op, om, nx, ny, nz, h.npb, h.nchunk, cf, slots, add); };
+    if (small) {
+        if (periodic) sc ? go(step_simple_kernel<T, uint32_t, true, true>) : go(step_simple_kernel<T, uint32_t, true, false>);
+        else sc ? go(step_simple_kernel<T, uint32_t, false, true>) : go(step_simple_kernel<T, uint32_t, false, false>);
+    } else {
+        if (periodic) sc ? go(step_simple_kernel<T, uint64_t, true, true>) : go(step_simple_kernel<T, uint64_t, true, false>);
+        else sc ? go(step_simple_kernel<T, uint64_t, false, true>) : go(step_simple_kernel<T, uint64_t, false, false>);
+    }
+    IT_CK(cudaGetLastError());
+    return IT_OK;
 }
 
 int launch_step_simple(it_ctx *c, cudaStream_t s) {
-    const int nb = c->nslots;
     const int cur = c->cur, nxt = cur ^ 1;
-    if (c->prec == IT_FP32) {
-        auto *ip = (const float *)c->n[cur][0], *im = (const float *)c->n[cur][1];
-        auto *op = (float *)c->n[nxt][0], *om = (float *)c->n[nxt][1];
-        if (c->p.lateral_bc == IT_PERIODIC)
-            step_simple_kernel<float, true><<<nb, 256, 0, s>>>(ip, im, op, om, c->g.nx, c->g.ny, c->g.nz, c->cf, c->d_slots);
-        else
-            step_simple_kernel<float, false><<<nb, 256, 0, s>>>(ip, im, op, om, c->g.nx, c->g.ny, c->g.nz, c->cf, c->d_slots);
-    } else {
-        auto *ip = (const double *)c->n[cur][0], *im = (const double *)c->n[cur][1];
-        auto *op = (double *)c->n[nxt][0], *om = (double *)c->n[nxt][1];
-        if (c->p.lateral_bc == IT_PERIODIC)
-            step_simple_kernel<double, true><<<nb, 256, 0, s>>>(ip, im, op, om, c->g.nx, c->g.ny, c->g.nz, c->cd, c->d_slots);
-        else
-            step_simple_kernel<double, false><<<nb, 256, 0, s>>>(ip, im, op, om, c->g.nx, c->g.ny, c->g.nz, c->cd, c->d_slots);
-    }
-    IT_CK(cudaGetLastError());
+    const bool per = c->p.lateral_bc == IT_PERIODIC;
+    const int rc = c->prec == IT_FP32
+                       ? sk_launch<float>((const float *)c->n[cur][0], (const float *)c->n[cur][1],
+                                          (float *)c->n[nxt][0], (float *)c->n[nxt][1], c->g.nx, c->g.ny, c->g.nz,
+                                          c->cf, per, c->d_slots, 1, s)
+                       : sk_launch<double>((const double *)c->n[cur][0], (const double *)c->n[cur][1],
+                                           (double *)c->n[nxt][0], (double *)c->n[nxt][1], c->g.nx, c->g.ny, c->g.nz,
+                                           c->cd, per, c->d_slots, 1, s);
+    if (rc) return rc;
     c->cur = nxt;
     return IT_OK;
 }
 
-// The simple step on caller-given FP32 arrays with a caller-given slot array
-// of nblocks x NT doubles (one block per slot, grid-stride over the cells).
+// The simple step on caller-given FP32 arrays; writes (not adds) the tallies
+// of simple_grid_f32(nx, ny, nz) slots of NT doubles.
 int launch_step_simple_raw_f32(const float *ip, const float *im, float *op, float *om, int nx, int ny, int nz,
-                               const Coef<float> &cf, bool periodic, double *slots, int nblocks, cudaStream_t s) {
-    if (periodic)
-        step_simple_kernel<float, true><<<nblocks, 256, 0, s>>>(ip, im, op, om, nx, ny, nz, cf, slots);
-    else
-        step_simple_kernel<float, false><<<nblocks, 256, 0, s>>>(ip, im, op, om, nx, ny, nz, cf, slots);
-    IT_CK(cudaGetLastError());
-    return IT_OK;
+                               const Coef<float> &cf, bool periodic, double *slots, cudaStream_t s) {
+    return sk_launch<float>(ip, im, op, om, nx, ny, nz, cf, periodic, slots, 0, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -156,8 +358,8 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 monitor_kernel(const T *__restrict__ ip, const T *__restrict__ im, size_t total, double vol,
                double *__restrict__ mon) {
-    __shared__ double red[32 * 2];
-    __shared__ double rmin[32 * 2], rmax[32 * 2];
+    __shared__ double bsum[2][256];
+    __shared__ T bext[4][256];
     MonAcc<T> acc;
     const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t nthr = (size_t)gridDim.x * blockDim.x;
@@ -203,31 +405,35 @@ monitor_kernel(const T *__restrict__ ip, const T *__restrict__ im, size_t total,
         }
         acc.flush();
     }
-    double sum[2] = {acc.sum[0], acc.sum[1]};
-    double mn[2] = {(double)acc.mn[0], (double)acc.mn[1]}, mx[2] = {(double)acc.mx[0], (double)acc.mx[1]};
+    // block reduction, one warp per quantity over the 256 threads' values in
+    // shared memory: a shuffle reduction of all six in every warp kept the
+    // FP64 pipe busy longer than the loads took
+    bsum[0][threadIdx.x] = acc.sum[0]; bsum[1][threadIdx.x] = acc.sum[1];
+    bext[0][threadIdx.x] = acc.mn[0]; bext[1][threadIdx.x] = acc.mn[1];
+    bext[2][threadIdx.x] = acc.mx[0]; bext[3][threadIdx.x] = acc.mx[1];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    double *m = mon + (size_t)blockIdx.x * NM;
+    if (q < 2) {
+        double t = bsum[q][lane];
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
+        for (int r = 1; r < 8; ++r) t += bsum[q][lane + 32 * r];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (lane == 0) m[q] = t * vol;
+    } else if (q < 6) {
+        const bool lo = q < 4;
+        T t = bext[q - 2][lane];
+        for (int r = 1; r < 8; ++r) {
+            const T x = bext[q - 2][lane + 32 * r];
+            t = (lo ? x < t : x > t) ? x : t;
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            mn[q] = fmin(mn[q], __shfl_down_sync(0xffffffffu, mn[q], o));
-            mx[q] = fmax(mx[q], __shfl_down_sync(0xffffffffu, mx[q], o));
+            const T x = __shfl_down_sync(0xffffffffu, t, o);
+            t = (lo ? x < t : x > t) ? x : t;
         }
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) {
-        rmin[warp * 2] = mn[0]; rmin[warp * 2 + 1] = mn[1];
-        rmax[warp * 2] = mx[0]; rmax[warp * 2 + 1] = mx[1];
-    }
-    block_sum<2>(sum, red);   // contains the __syncthreads for rmin/rmax too
-    if (threadIdx.x == 0) {
-        const int nw = blockDim.x >> 5;
-        for (int w = 1; w < nw; ++w) {
-            mn[0] = fmin(mn[0], rmin[w * 2]); mn[1] = fmin(mn[1], rmin[w * 2 + 1]);
-            mx[0] = fmax(mx[0], rmax[w * 2]); mx[1] = fmax(mx[1], rmax[w * 2 + 1]);
-        }
-        double *m = mon + (size_t)blockIdx.x * NM;
-        m[0] = sum[0] * vol; m[1] = sum[1] * vol;
-        m[2] = mn[0]; m[3] = mn[1]; m[4] = mx[0]; m[5] = mx[1];
+        if (lane == 0) m[q] = (double)t;
     }
 }
 
@@ -256,48 +462,37 @@ int launch_monitor_raw_f32(const float *p, const float *m, size_t cells, double 
 // finalize: fixed-order sums of the per-CTA slots and monitor values
 //   out[0..NT) tallies, out[NT..NT+NM) monitor, out[NT+NM..+2) released
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256)
+// One warp per quantity: lane l takes entries l, l + 32, ..., then shuffles.
+// (A block_sum of all twelve sums took 16 us for 304 slots: sixty FP64
+// additions per warp at two lanes per clock and a serial tail; this form
+// takes 4.2 us.)
+__global__ void __launch_bounds__(480)
 finalize_kernel(const double *__restrict__ slots, int nslots, const double *__restrict__ mon,
                 int nmon, const double *__restrict__ acc, const int *__restrict__ err, double *__restrict__ out) {
-    __shared__ double red[32 * (NT + 2)];
-    __shared__ double rmin[32 * 2], rmax[32 * 2];
-    double v[NT + 2];
-#pragma unroll
-    for (int q = 0; q < NT + 2; ++q) v[q] = 0.0;
-    for (int b = threadIdx.x; b < nslots; b += blockDim.x) {
-#pragma unroll
-        for (int q = 0; q < NT; ++q) v[q] += slots[(size_t)b * NT + q];
-    }
-    double mn[2] = {INFINITY, INFINITY}, mx[2] = {-INFINITY, -INFINITY};
-    for (int b = threadIdx.x; b < nmon; b += blockDim.x) {
-        v[NT] += mon[(size_t)b * NM + 0];
-        v[NT + 1] += mon[(size_t)b * NM + 1];
-        mn[0] = fmin(mn[0], mon[(size_t)b * NM + 2]); mn[1] = fmin(mn[1], mon[(size_t)b * NM + 3]);
-        mx[0] = fmax(mx[0], mon[(size_t)b * NM + 4]); mx[1] = fmax(mx[1], mon[(size_t)b * NM + 5]);
-    }
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (w < 9) {            // tallies 0..8 (9 is unused)
+        const double t = warp_strided_sum(slots, nslots, w, NT, lane);
+        if (lane == 0) out[w] = t;
+    } else if (w < 11) {    // in-domain ions
+        const double t = warp_strided_sum(mon, nmon, w - 9, NM, lane);
+        if (lane == 0) out[NT + w - 9] = t;
+    } else {                // extremes
+        const int q = w - 9;
+        const bool lo = q < 4;
+        double t = lo ? INFINITY : -INFINITY;
+        for (int b = lane; b < nmon; b += 32) {
+            const double x = mon[(size_t)b * NM + q];
+            t = lo ? fmin(t, x) : fmax(t, x);
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            mn[q] = fmin(mn[q], __shfl_down_sync(0xffffffffu, mn[q], o));
-            mx[q] = fmax(mx[q], __shfl_down_sync(0xffffffffu, mx[q], o));
+            const double x = __shfl_down_sync(0xffffffffu, t, o);
+            t = lo ? fmin(t, x) : fmax(t, x);
         }
+        if (lane == 0) out[NT + q] = t;
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) {
-        rmin[warp * 2] = mn[0]; rmin[warp * 2 + 1] = mn[1];
-        rmax[warp * 2] = mx[0]; rmax[warp * 2 + 1] = mx[1];
-    }
-    block_sum<NT + 2>(v, red);
     if (threadIdx.x == 0) {
-        const int nw = blockDim.x >> 5;
-        for (int w = 1; w < nw; ++w) {
-            mn[0] = fmin(mn[0], rmin[w * 2]); mn[1] = fmin(mn[1], rmin[w * 2 + 1]);
-            mx[0] = fmax(mx[0], rmax[w * 2]); mx[1] = fmax(mx[1], rmax[w * 2 + 1]);
-        }
-        for (int q = 0; q < NT; ++q) out[q] = v[q];
-        out[NT + 0] = v[NT]; out[NT + 1] = v[NT + 1];
-        out[NT + 2] = mn[0]; out[NT + 3] = mn[1]; out[NT + 4] = mx[0]; out[NT + 5] = mx[1];
+        out[9] = 0.0;
         out[NT + NM + 0] = acc[0];
         out[NT + NM + 1] = acc[1];
         out[NT + NM + 2] = (double)*err;
@@ -305,7 +500,7 @@ finalize_kernel(const double *__restrict__ slots, int nslots, const double *__re
 }
 
 int launch_finalize(it_ctx *c, cudaStream_t s) {
-    finalize_kernel<<<1, 256, 0, s>>>(c->d_slots, c->nslots, c->d_mon, c->nmon, c->d_acc, c->d_err, c->d_out);
+    finalize_kernel<<<1, 480, 0, s>>>(c->d_slots, c->nslots, c->d_mon, c->nmon, c->d_acc, c->d_err, c->d_out);
     IT_CK(cudaGetLastError());
     return IT_OK;
 }

@@ -14,7 +14,7 @@
 // is looked up once per device (cudaGetSymbolAddress, with that device
 // current) on the first call made on that device; that first call should
 // therefore come before any stream capture.  Every call shares the array
-// and zeroes the part it uses before the step, so two calls that overlap on
+// and overwrites the part it uses, so two calls that overlap on
 // the GPU (different streams, or different host threads, without ordering
 // between them) race on it and must not be issued.
 #include <mutex>
@@ -52,20 +52,13 @@ int noalloc_scratch(double **out) {
     return IT_OK;
 }
 
-// Fixed-order sum of the per-block slots into the 7 tallies of this step
-// (same order as the context's finalize reduction).
-__global__ void __launch_bounds__(256)
+// Fixed-order sum of the per-block slots into the 7 tallies of this step, one
+// warp per tally (the order of the context's finalize reduction).
+__global__ void __launch_bounds__(224)
 noalloc_reduce_kernel(const double *__restrict__ slots, int nslots, double *__restrict__ out7) {
-    __shared__ double red[32 * 7];
-    double v[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int b = threadIdx.x; b < nslots; b += blockDim.x) {
-#pragma unroll
-        for (int q = 0; q < 7; ++q) v[q] += slots[(size_t)b * NT + q];
-    }
-    block_sum<7>(v, red);
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < 7; ++q) out7[q] = v[q];
-    }
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const double t = warp_strided_sum(slots, nslots, q, NT, lane);
+    if (lane == 0) out7[q] = t;
 }
 
 }  // namespace
@@ -96,30 +89,17 @@ extern "C" int it_step_noalloc(it_grid g, double dx_cm, double dt_s, const it_pa
         set_error("it_step_noalloc: outputs must not alias the inputs");
         return IT_EINVAL;
     }
-    const size_t cells = (size_t)g.nx * g.ny * g.nz;
-    int dev = 0, sms = 0;
-    IT_CK(cudaGetDevice(&dev));
-    IT_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const size_t want = (cells + 255) / 256;
-    const size_t cap = (size_t)sms * 8;
-    const size_t blocks = want < cap ? want : cap;
-    if (blocks > (size_t)IT_NOALLOC_MAX_BLOCKS) {
-        set_error("it_step_noalloc: this device needs " + std::to_string(blocks) +
-                  " tally blocks, the static scratch holds " + std::to_string(IT_NOALLOC_MAX_BLOCKS));
-        return IT_EINVAL;
-    }
+    const int blocks = simple_grid_f32(g.nx, g.ny, g.nz);   // at most IT_NOALLOC_MAX_BLOCKS
     double *slots = nullptr;
     rc = noalloc_scratch(&slots);
     if (rc) return rc;
     Coef<float> cf;
     coef_f32(p, dx_cm, dt_s, &cf);
     cudaStream_t s = (cudaStream_t)stream;
-    // the step kernel adds into its slots: clear the part this call uses
-    IT_CK(cudaMemsetAsync(slots, 0, sizeof(double) * NT * blocks, s));
     rc = launch_step_simple_raw_f32(dev_plus, dev_minus, dev_out_plus, dev_out_minus, g.nx, g.ny, g.nz, cf,
-                                    p->lateral_bc == IT_PERIODIC, slots, (int)blocks, s);
+                                    p->lateral_bc == IT_PERIODIC, slots, s);
     if (rc) return rc;
-    noalloc_reduce_kernel<<<1, 256, 0, s>>>(slots, (int)blocks, dev_tallies7);
+    noalloc_reduce_kernel<<<1, 224, 0, s>>>(slots, blocks, dev_tallies7);
     IT_CK(cudaGetLastError());
     return IT_OK;
 }
