@@ -61,10 +61,10 @@ struct ZmConf {
     int nzc;          // CTAs in the grid (each takes a contiguous range of tile-planes)
     int ntile;        // ny / TY
     int S;            // ring depth (>= 3)
-    int bx;           // row width a block holds (nx; 256 for the 3-D maps of nx > 256)
+    int bx;           // row width a block holds (nx)
     int nbx;          // nx / bx
-    int xs;           // 1: 3-D maps; nx / 256 > 1: 4-D maps that split a row into xs
-                      // 256-float pieces, so one box carries whole rows (bx = nx)
+    int xs;           // 1: 3-D maps; > 1: 4-D maps that split a row of nx > 256 into xs
+                      // equal pieces (row_piece), so one box carries whole rows (bx = nx)
     int reg_top, reg_main, reg_bot;   // float offsets of the halo/main rows in a block
     int blk;          // floats per (species, x-box) block, 128-byte multiple
     int slot;         // floats per slot = 2 * nbx * blk
@@ -145,8 +145,8 @@ struct it_ctx {
     // z-march kernel configuration (it_zmarch.cu)
     itk::ZmConf zm;
     int zm_grid;
-    CUtensorMap tm_main[2][2];   // [set][species], box {bx, TY, 1} (4-D {256, nx/256, TY, 1} for nx > 256)
-    CUtensorMap tm_halo[2][2];   // [set][species], box {bx, 1, 1} (4-D {256, nx/256, 1, 1} for nx > 256)
+    CUtensorMap tm_main[2][2];   // [set][species], box {bx, TY, 1} (4-D for nx > 256: pieces of a row)
+    CUtensorMap tm_halo[2][2];   // [set][species], box {bx, 1, 1} (4-D for nx > 256)
     itk::Zm2Conf zm2;            // two steps per launch (IT_KERNEL_ZMARCH2)
     CUtensorMap tm_main2[2][2];  // [set][species], box {bx, TY, 1}
     CUtensorMap tm_halo2[2][2];  // [set][species], box {bx, 2, 1}
@@ -176,6 +176,7 @@ int zmarch_configure(it_ctx *c);
 int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid);
 // FP32 3-D tensor map over [nz][ny][nx] with a box of bx x rows x 1 (it_zmarch.cu)
 int encode_map(CUtensorMap *m, void *base, int nx, int ny, int nz, int bx, int rows);
+int row_piece(int nx);
 int encode_map_rows(CUtensorMap *m, void *base, int nx, int ny, int nz, int rows);
 int encode_bf16_sw128(CUtensorMap *m, const void *base, long long K, long long rows, long long members,
                       long long row_bytes, long long member_bytes);

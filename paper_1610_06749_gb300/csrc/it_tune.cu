@@ -31,7 +31,7 @@ std::vector<Shape> candidates(const it_ctx *c) {
     std::vector<Shape> v;
     v.push_back({IT_KERNEL_SIMPLE, 0, 0, 0, 0});
     const int nx = c->g.nx, ny = c->g.ny;
-    if (c->prec != IT_FP32 || nx % 4 != 0 || (nx > 256 && nx % 256 != 0)) return v;
+    if (c->prec != IT_FP32 || nx % 4 != 0 || (nx > 256 && !row_piece(nx))) return v;
     const int ncol4 = nx / 4;
     for (int cps = 1; cps <= 2; ++cps) {
         const int threads = cps == 1 ? 512 : 256;
@@ -47,7 +47,7 @@ std::vector<Shape> candidates(const it_ctx *c) {
     // threads / (nx/4)
     for (int cps = 1; cps <= 2; ++cps) {
         const int threads = cps == 1 ? 512 : 256;
-        if (threads % ncol4 != 0 || 2 * ncol4 > threads) continue;
+        if (threads % ncol4 != 0 || 2 * ncol4 > threads || (nx > 256 && nx % 256 != 0)) continue;
         const int ty = threads / ncol4;
         if (ny % ty != 0 || ny < 4) continue;
         for (int s : {3, 4, 5, 6})

@@ -414,20 +414,30 @@ int encode_map(CUtensorMap *m, void *base, int nx, int ny, int nz, int bx, int r
     return IT_OK;
 }
 
-// Wide rows (nx > 256, nx % 256 == 0): a 4-D view {256, nx / 256, ny, nz} of
-// the same array (byte strides 1 KiB, one row, one plane), boxes of
-// {256, nx / 256, rows, 1}, which land in shared memory as `rows` whole rows
-// of nx floats: one copy per box where the 3-D view needs nx / 256.
+// Width of the pieces a row of nx > 256 floats is split into: its largest
+// divisor that is a multiple of 4 floats (16-byte strides) and fits a box
+// dimension (256).  0: no divisor of at least 128 bytes, whose boxes would
+// crawl in 16-byte pieces, or too many pieces for a box dimension.
+int row_piece(int nx) {
+    for (int d = 256; d >= 32; d -= 4)
+        if (nx % d == 0) return nx / d <= 256 ? d : 0;
+    return 0;
+}
+
+// Wide rows (nx > 256): a 4-D view {d, nx / d, ny, nz} of the same array with
+// d = row_piece(nx) (byte strides of a piece, a row, a plane), boxes of
+// {d, nx / d, rows, 1}, which land in shared memory as `rows` whole rows of
+// nx floats: one copy per box where the 3-D view needs nx / d.
 int encode_map_rows(CUtensorMap *m, void *base, int nx, int ny, int nz, int rows) {
     auto fn = encode_fn();
     if (!fn) {
         set_error("cuTensorMapEncodeTiled is not available");
         return IT_ECUDA;
     }
-    const int xs = nx / 256;
-    cuuint64_t dims[4] = {256, (cuuint64_t)xs, (cuuint64_t)ny, (cuuint64_t)nz};
-    cuuint64_t strides[3] = {256 * 4, (cuuint64_t)nx * 4, (cuuint64_t)nx * ny * 4};
-    cuuint32_t box[4] = {256, (cuuint32_t)xs, (cuuint32_t)rows, 1};
+    const int d = row_piece(nx), xs = nx / d;
+    cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)xs, (cuuint64_t)ny, (cuuint64_t)nz};
+    cuuint64_t strides[3] = {(cuuint64_t)d * 4, (cuuint64_t)nx * 4, (cuuint64_t)nx * ny * 4};
+    cuuint32_t box[4] = {(cuuint32_t)d, (cuuint32_t)xs, (cuuint32_t)rows, 1};
     cuuint32_t es[4] = {1, 1, 1, 1};
     CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, dims, strides, box, es,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -500,7 +510,10 @@ int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid
     const int nx = c->g.nx, ny = c->g.ny, nz = c->g.nz;
     if (c->prec != IT_FP32) { set_error("z-march kernel needs FP32 densities"); return IT_EINVAL; }
     if (nx % 4 != 0) { set_error("z-march kernel needs nx % 4 == 0"); return IT_EINVAL; }
-    if (nx > 256 && nx % 256 != 0) { set_error("z-march kernel needs nx <= 256 or nx % 256 == 0"); return IT_EINVAL; }
+    if (nx > 256 && !row_piece(nx)) {
+        set_error("z-march kernel: nx > 256 needs a divisor of 32 to 256 that is a multiple of 4");
+        return IT_EINVAL;
+    }
     if ((unsigned long long)nx * ny * nz > 0xFFFFFFFFull) {
         set_error("z-march kernel indexes a species array with 32 bits: needs nx*ny*nz < 2^32");
         return IT_EINVAL;
@@ -511,8 +524,8 @@ int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid
     ZmConf z{};
     z.threads = nw * 32;
     // a ring block holds whole rows; rows wider than a TMA box dimension (256
-    // floats) come through the 4-D view (nx / 256 pieces per row, one box)
-    z.xs = nx > 256 ? nx / 256 : 1;
+    // floats) come through the 4-D view (one box of several pieces per row)
+    z.xs = nx > 256 ? nx / row_piece(nx) : 1;
     z.bx = nx;
     z.nbx = 1;
     // rows per tile: the smallest divisor of ny that gives every thread two
