@@ -68,7 +68,8 @@ extern "C" {
 /* it_params.kernel: which step kernel runs (all are CUDA). */
 #define IT_KERNEL_AUTO   0   /* z-march kernel where the grid allows, else simple */
 #define IT_KERNEL_SIMPLE 1   /* one thread per column of cells, global loads (any grid and type) */
-#define IT_KERNEL_ZMARCH 2   /* TMA-staged z-planes in shared memory (FP32, nx % 4 == 0) */
+#define IT_KERNEL_ZMARCH 2   /* marches up z, float4 segments (FP32, nx % 4 == 0): TMA-staged z-planes in
+                                shared memory, or (IT_KERNEL_AUTO, small grids) straight from L1/L2 */
 #define IT_KERNEL_ZMARCH2 3  /* as IT_KERNEL_ZMARCH, two time steps per launch (temporal blocking
                                 of depth 2; nx/4 must divide 256 or 512 threads); densities are
                                 bitwise those of two single steps */
@@ -350,7 +351,8 @@ int it_set_launch_ex(it_ctx *ctx, int kernel, int tile_rows, int ctas_per_sm, in
 int it_autotune(it_ctx *ctx, int trial_steps, int flags, double *best_us);
 
 /* Report the kernel in use, its launch shape and its CTA count (for
- * IT_KERNEL_ZMARCH2, the CTAs of its two-step launches). */
+ * IT_KERNEL_ZMARCH2, the CTAs of its two-step launches; IT_KERNEL_ZMARCH
+ * without a shared-memory ring reports 0 rows, 0 CTAs per SM, 0 stages). */
 int it_get_launch(it_ctx *ctx, int *kernel, int *tile_rows, int *ctas_per_sm, int *stages, int *ctas);
 
 /* ---------------------------------------------------------------------------

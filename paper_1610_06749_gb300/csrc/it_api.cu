@@ -296,6 +296,15 @@ int validate_step_args(const it_params *p, it_grid g, double dx, double dt) {
 
 void coef_f32(const it_params *p, double dx, double dt, Coef<float> *out) { make_coef(*out, p, dx, dt); }
 
+// tally slots of the configured kernel: one per CTA of every launch it makes
+// (the z-march has two forms, staged and direct; the two-step kernel leaves
+// odd steps to the simple kernel)
+static int slots_needed(const it_ctx *c) {
+    return c->kernel == IT_KERNEL_ZMARCH    ? std::max(c->zm_grid, direct_grid(c))
+           : c->kernel == IT_KERNEL_ZMARCH2 ? std::max(c->zm2.grid, simple_grid(c))
+                                            : simple_grid(c);
+}
+
 // Reconfigure the step kernel (no step-count check); tally slots restart.
 int set_launch(it_ctx *c, int kernel, int tile_rows, int ctas_per_sm, int stages, int grid) {
     if (kernel == IT_KERNEL_SIMPLE) {
@@ -315,10 +324,8 @@ int set_launch(it_ctx *c, int kernel, int tile_rows, int ctas_per_sm, int stages
     } else {
         return fail(IT_EINVAL, "bad kernel");
     }
-    // the two-step kernel leaves odd steps to the simple kernel: slots for both
-    const int n = c->kernel == IT_KERNEL_ZMARCH    ? c->zm_grid
-                  : c->kernel == IT_KERNEL_ZMARCH2 ? std::max(c->zm2.grid, simple_grid(c))
-                                                   : simple_grid(c);
+    c->direct = c->kernel == IT_KERNEL_ZMARCH && ((kernel == IT_KERNEL_AUTO && direct_wins(c)) || tile_rows < 0);
+    const int n = slots_needed(c);
     if (n != c->nslots) {
         double *ns = nullptr;
         IT_CK(cudaMalloc(&ns, sizeof(double) * NT * n));
@@ -485,10 +492,8 @@ int it_create_ex(it_grid g, double dx_cm, double dt_s, const it_params *p, void 
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // the two-step kernel leaves odd steps to the simple kernel: slots for both
-    c->nslots = c->kernel == IT_KERNEL_ZMARCH    ? c->zm_grid
-                : c->kernel == IT_KERNEL_ZMARCH2 ? std::max(c->zm2.grid, simple_grid(c))
-                                                 : simple_grid(c);
+    c->direct = c->kernel == IT_KERNEL_ZMARCH && p->kernel == IT_KERNEL_AUTO && direct_wins(c);
+    c->nslots = slots_needed(c);
     c->nmon = 2 * sms;
 
     if ((e = cudaMalloc(&c->d_slots, sizeof(double) * NT * c->nslots)) != cudaSuccess ||
@@ -863,7 +868,7 @@ int it_device_state(it_ctx *c, void **plus, void **minus, void **stream) {
 int it_set_launch_ex(it_ctx *c, int kernel, int tile_rows, int ctas_per_sm, int stages, int grid) {
     if (!c) return fail(IT_EINVAL, "ctx is NULL");
     if (c->steps != 0) return fail(IT_ESTATE, "launch shape can only change before the first step");
-    return set_launch(c, kernel, tile_rows, ctas_per_sm, stages, grid);
+    return set_launch(c, kernel, std::max(tile_rows, 0), ctas_per_sm, stages, grid);
 }
 
 int it_set_launch(it_ctx *c, int kernel, int tile_rows, int ctas_per_sm, int stages) {
@@ -872,12 +877,12 @@ int it_set_launch(it_ctx *c, int kernel, int tile_rows, int ctas_per_sm, int sta
 
 int it_get_launch(it_ctx *c, int *kernel, int *tile_rows, int *ctas_per_sm, int *stages, int *ctas) {
     if (!c) return fail(IT_EINVAL, "ctx is NULL");
-    const bool zm = c->kernel == IT_KERNEL_ZMARCH, zm2 = c->kernel == IT_KERNEL_ZMARCH2;
+    const bool zm = c->kernel == IT_KERNEL_ZMARCH && !c->direct, zm2 = c->kernel == IT_KERNEL_ZMARCH2;
     if (kernel) *kernel = c->kernel;
     if (tile_rows) *tile_rows = zm ? c->zm.TY : zm2 ? c->zm2.TY : 0;
     if (ctas_per_sm) *ctas_per_sm = zm ? c->zm.ctas_per_sm : zm2 ? c->zm2.ctas_per_sm : 0;
     if (stages) *stages = zm ? c->zm.S : zm2 ? c->zm2.S : 0;
-    if (ctas) *ctas = zm2 ? c->zm2.grid : c->nslots;
+    if (ctas) *ctas = zm2 ? c->zm2.grid : zm ? c->zm_grid : c->direct ? direct_grid(c) : c->nslots;
     return IT_OK;
 }
 
@@ -895,6 +900,7 @@ int it_test_withhold_load(it_ctx *c, int on) {
     if (on != 0 && on != 1) return fail(IT_EINVAL, "on must be 0 or 1");
     if (on && c->kernel != IT_KERNEL_ZMARCH) return fail(IT_ESTATE, "the test hook applies to the z-march kernel only");
     c->withhold = on;
+    if (on) c->direct = 0;   // the hook is the ring's
     if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
     return IT_OK;
 }

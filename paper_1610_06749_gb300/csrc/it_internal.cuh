@@ -145,6 +145,7 @@ struct it_ctx {
     // z-march kernel configuration (it_zmarch.cu)
     itk::ZmConf zm;
     int zm_grid;
+    int direct;              // 1: the z-march runs straight from L1/L2 (step_direct_kernel), no ring
     CUtensorMap tm_main[2][2];   // [set][species], box {bx, TY, 1} (4-D for nx > 256: pieces of a row)
     CUtensorMap tm_halo[2][2];   // [set][species], box {bx, 1, 1} (4-D for nx > 256)
     itk::Zm2Conf zm2;            // two steps per launch (IT_KERNEL_ZMARCH2)
@@ -172,6 +173,10 @@ int cuda_fail(cudaError_t e, const char *what);
 // kernels (it_kernels.cu)
 int launch_step_simple(it_ctx *c, cudaStream_t s);
 int launch_step_zmarch(it_ctx *c, cudaStream_t s);
+int launch_step_direct(it_ctx *c, cudaStream_t s);
+int direct_grid(const it_ctx *c);
+bool direct_wins(const it_ctx *c);
+double direct_us(const it_ctx *c);
 int zmarch_configure(it_ctx *c);
 int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid);
 // FP32 3-D tensor map over [nz][ny][nx] with a box of bx x rows x 1 (it_zmarch.cu)

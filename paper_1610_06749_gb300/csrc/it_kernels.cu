@@ -13,6 +13,7 @@
 
 #include "it_device.cuh"
 #include "it_internal.cuh"
+#include "it_tma.cuh"
 
 namespace itk {
 
@@ -38,6 +39,8 @@ namespace itk {
 // one plane ahead: ten blocks without that took 34.6 us on 301x173x97.
 constexpr int SK_THREADS = 128;
 constexpr int SK_BLOCKS_F32 = 8, SK_BLOCKS_F64 = 6;   // resident blocks per SM
+constexpr int DK_BLOCKS = 4;                            // of the direct kernel (128 registers)
+constexpr double DK_LAT = 650.0, DK_THR = 190.0;        // its cycles per plane: alone, and per block it shares the SM with
 
 // FP32 sum that carries the rounding error of each addition (Knuth's
 // two-sum), so a sum of some hundred terms keeps about 46 bits: as good as
@@ -119,6 +122,21 @@ __device__ __forceinline__ void sk_reduce(const Sum (&v)[N], Sum (*buf)[SK_THREA
             if (lane == 0) tot[at + q] += s.value();
         }
     }
+}
+
+// Tally tid of a block's slot from its sums (order: rec, lateral, space
+// charge, anode from 5, cathode from 7), added or written.
+template <bool PERIODIC, bool SC, int NV, typename T>
+__device__ __forceinline__ void sk_slot(const double *tot, const Coef<T> &c, double *slots, int tid, int add) {
+    double t = 0.0;
+    if (tid == 0) t = tot[0] * c.rec_f;
+    else if (tid < 3) t = tot[5 + tid - 1] * c.anode_f[tid - 1];
+    else if (tid < 5) t = tot[7 + tid - 3] * c.cathode_f[tid - 3];
+    // x and y weights are equal for dx = dy (latx_f == laty_f)
+    else if (tid < 7) t = PERIODIC ? 0.0 : tot[1 + tid - 5] * c.latx_f[tid - 5];
+    else t = SC ? tot[NV - 2 + tid - 7] * c.sc_f[tid - 7] : 0.0;
+    double *sl = slots + (size_t)blockIdx.x * NT + tid;
+    *sl = add ? *sl + t : t;
 }
 
 // Work unit u: column block u mod npb, z chunk u / npb of nchunk.  A block
@@ -224,17 +242,7 @@ step_simple_kernel(const T *__restrict__ ip, const T *__restrict__ im, T *__rest
         }
     }
     __syncthreads();
-    if (tid < 9) {   // tally tid of the slot
-        double t = 0.0;
-        if (tid == 0) t = tot[0] * c.rec_f;
-        else if (tid < 3) t = tot[AN + tid - 1] * c.anode_f[tid - 1];
-        else if (tid < 5) t = tot[CA + tid - 3] * c.cathode_f[tid - 3];
-        // x and y weights are equal for dx = dy (latx_f == laty_f)
-        else if (tid < 7) t = PERIODIC ? 0.0 : tot[1 + tid - 5] * c.latx_f[tid - 5];
-        else t = SC ? tot[NV - 2 + tid - 7] * c.sc_f[tid - 7] : 0.0;
-        double *sl = slots + (size_t)blockIdx.x * NT + tid;
-        *sl = add ? *sl + t : t;
-    }
+    if (tid < 9) sk_slot<PERIODIC, SC, NV>(tot, c, slots, tid, add);
 }
 
 // Chunks per column and blocks of a launch, by the fitted time of a split.
@@ -323,6 +331,196 @@ int launch_step_simple(it_ctx *c, cudaStream_t s) {
 int launch_step_simple_raw_f32(const float *ip, const float *im, float *op, float *om, int nx, int ny, int nz,
                                const Coef<float> &cf, bool periodic, double *slots, cudaStream_t s) {
     return sk_launch<float>(ip, im, op, om, nx, ny, nz, cf, periodic, slots, 0, s);
+}
+
+// ---------------------------------------------------------------------------
+// direct march: FP32, nx % 4 == 0, columns of float4 straight from L1/L2
+// ---------------------------------------------------------------------------
+// The simple kernel's work split with a float4 x-segment per thread and the
+// paired-FP32 update: a block is 128 neighbouring segments of the flattened
+// x-y plane, marched over a chunk of planes.  x neighbours come by warp
+// shuffle (a load at the ends of a warp or row), y neighbours by 16-byte
+// loads that mostly hit L1, the plane above is loaded one plane ahead.
+// It has no ring to fill and no slot hand-back, which is what a step of a
+// small or middle-sized grid (state in L2) spends its time on with the
+// TMA-staged kernel; on grids that stream from HBM the ring wins.
+// DIRECT_MEASURED
+__device__ __forceinline__ float dk_sum(float4 a) { return __fadd_rn(__fadd_rn(a.x, a.y), __fadd_rn(a.z, a.w)); }
+
+template <typename Idx, bool PERIODIC, bool SC>
+__global__ void __launch_bounds__(SK_THREADS, DK_BLOCKS)
+step_direct_kernel(const float *__restrict__ ip, const float *__restrict__ im, float *__restrict__ op,
+                   float *__restrict__ om, int nx, int ny, int nz, unsigned npb, unsigned nchunk, const Coef<float> c,
+                   double *__restrict__ slots) {
+    constexpr int NV = 1 + (PERIODIC ? 0 : 2) + (SC ? 2 : 0);   // values reduced for every unit
+    __shared__ double raw[5 * SK_THREADS];
+    CompSum(*buf)[SK_THREADS] = reinterpret_cast<CompSum(*)[SK_THREADS]>(raw);
+    __shared__ double tot[9];   // order of sk_reduce: rec, lateral +/-, space charge +/-, then anode, cathode
+    constexpr int AN = 5, CA = 7;
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid < 9) tot[tid] = 0.0;
+    const unsigned ncol4 = (unsigned)nx >> 2;
+    const Idx plane = (Idx)nx * (Idx)ny, plane4 = (Idx)ncol4 * (Idx)ny;
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    const unsigned long long units = (unsigned long long)npb * nchunk;
+    for (unsigned long long u = blockIdx.x; u < units; u += gridDim.x) {
+        const unsigned pb = (unsigned)(u % npb), ch = (unsigned)(u / npb);
+        const int k0 = (int)((long long)nz * ch / nchunk), k1 = (int)((long long)nz * (ch + 1) / nchunk);
+        Idx q4 = (Idx)pb * SK_THREADS + tid;
+        const bool act = q4 < plane4;
+        if (!act) q4 = plane4 - 1;   // segments past the plane repeat the last one and store nothing
+        const int j = (int)(q4 / (Idx)ncol4), c4 = (int)(q4 - (Idx)j * (Idx)ncol4);
+        const Idx q = 4 * q4;
+        const bool first = c4 == 0, last = c4 == (int)ncol4 - 1;
+        const Idx qu = j > 0 ? q - (Idx)nx : q + (Idx)(ny - 1) * (Idx)nx;
+        const Idx qd = j < ny - 1 ? q + (Idx)nx : q - (Idx)(ny - 1) * (Idx)nx;
+        const bool hu = PERIODIC || j > 0, hd = PERIODIC || j < ny - 1;
+        const bool el = lane == 0 || first, er = lane == 31 || last || q4 + 1 >= plane4;
+        const Idx ql = first ? q + (Idx)(nx - 1) : q - 1, qr = last ? q - (Idx)(nx - 4) : q + 4;
+        CompSum v[NV];
+        Idx base = (Idx)k0 * plane;
+        auto ld = [&](const float *f, Idx e) { return __ldg(reinterpret_cast<const float4 *>(f + e)); };
+        float4 zm[2], n[2], zp[2];
+        zm[0] = k0 > 0 ? ld(ip, base - plane + q) : zero4;
+        zm[1] = k0 > 0 ? ld(im, base - plane + q) : zero4;
+        n[0] = ld(ip, base + q);
+        n[1] = ld(im, base + q);
+        zp[0] = k0 + 1 < nz ? ld(ip, base + plane + q) : zero4;
+        zp[1] = k0 + 1 < nz ? ld(im, base + plane + q) : zero4;
+        const float an[2] = {dk_sum(n[0]), dk_sum(n[1])};   // the chunk's first plane (anode tally)
+        // y neighbours and the x neighbours a shuffle cannot give, of plane k
+        float4 up[2], dn[2];
+        float le[2], re[2];
+        auto around = [&](Idx at) {
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const float *in = s ? im : ip;
+                up[s] = hu ? ld(in, at + qu) : zero4;
+                dn[s] = hd ? ld(in, at + qd) : zero4;
+                le[s] = el && (PERIODIC || !first) ? __ldg(in + at + ql) : 0.f;
+                re[s] = er && (PERIODIC || !last) ? __ldg(in + at + qr) : 0.f;
+            }
+        };
+        around(base);
+        float ca[2] = {0.f, 0.f};
+        for (int k = k0; k < k1; ++k, base += plane) {
+            float4 z2[2];   // two planes above, for the next round
+            const bool more = k + 1 < k1 && k + 2 < nz;
+            z2[0] = more ? ld(ip, base + 2 * plane + q) : zero4;
+            z2[1] = more ? ld(im, base + 2 * plane + q) : zero4;
+            const float2 rxy = __fmul2_rn(make_float2(n[0].x, n[0].y), make_float2(n[1].x, n[1].y));
+            const float2 rzw = __fmul2_rn(make_float2(n[0].z, n[0].w), make_float2(n[1].z, n[1].w));
+            float2 dxy, dzw;
+            if (SC) sc_diff4(n[0], n[1], dxy, dzw);
+            float4 w4[2];
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                float l = __shfl_up_sync(0xffffffffu, n[s].w, 1);
+                float r = __shfl_down_sync(0xffffffffu, n[s].x, 1);
+                if (el) l = le[s];
+                if (er) r = re[s];
+                w4[s] = upd7x4(n[s], l, r, up[s], dn[s], zm[s], zp[s], rxy, rzw, c.wx[s], c.wzm[s], c.wzp[s], c.adt);
+                if constexpr (SC) {
+                    float2 pxy, pzw;
+                    w4[s] = add_sc4(w4[s], c.sc[s], n[s], dxy, dzw, pxy, pzw);
+                    v[NV - 2 + s].add(dk_sum(make_float4(pxy.x, pxy.y, pzw.x, pzw.y)));
+                }
+                if constexpr (!PERIODIC) {
+                    if (first) v[1 + s].add(n[s].x);
+                    if (last) v[1 + s].add(n[s].w);
+                    if (j == 0) v[1 + s].add(dk_sum(n[s]));
+                    if (j == ny - 1) v[1 + s].add(dk_sum(n[s]));
+                }
+                if (k == nz - 1) ca[s] = dk_sum(n[s]);
+            }
+            if (k + 1 < k1) around(base + plane);
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+                if (act) *reinterpret_cast<float4 *>((s ? om : op) + base + q) = w4[s];
+            v[0].add(dk_sum(make_float4(rxy.x, rxy.y, rzw.x, rzw.y)));
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                zm[s] = n[s];
+                n[s] = zp[s];
+                zp[s] = z2[s];
+            }
+        }
+        if (!act) {
+#pragma unroll
+            for (int t = 0; t < NV; ++t) v[t] = CompSum{};
+        }
+        sk_reduce<NV>(v, buf, tot, 0);
+        if (k0 == 0) {
+            CompSum e[2];
+            if (act) { e[0].add(an[0]); e[1].add(an[1]); }
+            sk_reduce<2>(e, buf, tot, AN);
+        }
+        if (k1 == nz) {
+            CompSum e[2];
+            if (act) { e[0].add(ca[0]); e[1].add(ca[1]); }
+            sk_reduce<2>(e, buf, tot, CA);
+        }
+    }
+    __syncthreads();
+    if (tid < 9) sk_slot<PERIODIC, SC, NV>(tot, c, slots, tid, 1);
+}
+
+// Chunks and blocks, fitted as the simple kernel's are; *cycles receives the
+// fitted time.
+static SkShape dk_shape(int nx, int ny, int nz, double *cycles = nullptr) {
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const unsigned long long npb = ((unsigned long long)(nx / 4) * ny + SK_THREADS - 1) / SK_THREADS;
+    const unsigned long long resident = (unsigned long long)sms * DK_BLOCKS;
+    unsigned best = 1;
+    double best_cost = 1e300;
+    for (unsigned c = 1; c <= (unsigned)nz; c += std::max(1u, c / 16)) {
+        const unsigned long long units = npb * c;
+        if (c > 1 && units > 8 * resident) break;
+        const double kc = (nz + c - 1) / c;
+        const unsigned long long rem = units % resident;
+        double cost = (double)(units / resident) * (kc + 2.0) * (DK_LAT + DK_THR * DK_BLOCKS);
+        if (rem) cost += (kc + 2.0) * (DK_LAT + DK_THR * (double)((rem + sms - 1) / sms));
+        if (cost < 0.99 * best_cost) {
+            best_cost = cost;
+            best = c;
+        }
+    }
+    if (cycles) *cycles = best_cost;
+    const unsigned long long units = npb * best;
+    return SkShape{(unsigned)npb, best, (unsigned)std::min(units, resident)};
+}
+
+int direct_grid(const it_ctx *c) {
+    if (c->prec != IT_FP32 || c->g.nx % 4 != 0) return 0;
+    return (int)dk_shape(c->g.nx, c->g.ny, c->g.nz).grid;
+}
+
+// Fitted time of a direct step in us: its rounds at 1.9 GHz and a launch, or,
+// when both sets of the state outgrow L2, 1.45 times a copy at 6.8 TB/s.
+double direct_us(const it_ctx *c) {
+    double cycles = 0.0;
+    (void)dk_shape(c->g.nx, c->g.ny, c->g.nz, &cycles);
+    const double bytes = 16.0 * (double)c->g.cells();
+    return std::max(cycles / 1900.0 + 1.5, bytes > 100e6 ? 1.45 * bytes / 6.8e6 : 0.0);
+}
+
+int launch_step_direct(it_ctx *c, cudaStream_t s) {
+    const int cur = c->cur, nxt = cur ^ 1;
+    const int nx = c->g.nx, ny = c->g.ny, nz = c->g.nz;
+    const SkShape h = dk_shape(nx, ny, nz);
+    const float *ip = (const float *)c->n[cur][0], *im = (const float *)c->n[cur][1];
+    float *op = (float *)c->n[nxt][0], *om = (float *)c->n[nxt][1];
+    auto go = [&](auto *k) { k<<<h.grid, SK_THREADS, 0, s>>>(ip, im, op, om, nx, ny, nz, h.npb, h.nchunk, c->cf, c->d_slots); };
+    // 32-bit element offsets: the z-march family takes grids below 2^32 cells
+    if (c->p.lateral_bc == IT_PERIODIC)
+        c->cf.sc_on ? go(step_direct_kernel<uint32_t, true, true>) : go(step_direct_kernel<uint32_t, true, false>);
+    else
+        c->cf.sc_on ? go(step_direct_kernel<uint32_t, false, true>) : go(step_direct_kernel<uint32_t, false, false>);
+    IT_CK(cudaGetLastError());
+    c->cur = nxt;
+    return IT_OK;
 }
 
 // ---------------------------------------------------------------------------

@@ -503,6 +503,56 @@ static int zm_occupancy(size_t smem) {
 
 static int ipt_of(const it_ctx *c, int TY, int nw) { return ((c->g.nx / 4) * TY + nw * 32 - 1) / (nw * 32); }
 
+// CTAs of a launch without a given grid: the largest multiple of the tile
+// count, so that every tile column is cut at the same z and adjacent tiles
+// stream in step (their halo rows are then still in L2), unless that leaves
+// more than a tenth of the resident slots empty (300 of 304 CTAs on
+// 200x200x800: 95.3 us against 100.4 with all of them; 280 on 384x320x128:
+// 53.1 against 58.0).
+static long long zmarch_grid(int ntile, long long slots) {
+    const long long g = slots / ntile * ntile;
+    return g * 10 >= slots * 9 ? g : slots;
+}
+
+static int sm_count() {
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
+// Tile height and CTAs per SM when neither is given: the shape with the least
+// fitted time, (planes a CTA walks + 2) rounds and about 4 us to start and
+// drain; returns that time in us.  A round takes about 1.25 / 1.62 / 2.4 /
+// 3.7 us with one to four float4 per thread at two CTAs per SM and 1.3 / 1.75
+// / 2.4 / 3.5 at one (launch-shape sweeps on 256x256x400, 200x200x800,
+// 384x320x128 and 128x128x200: two CTAs per SM with two float4 per thread
+// take 76.8, 95.3, 56.5 and 19.3 us; the earlier rule, one CTA per SM with at
+// least two float4 per thread, took 81.7, 107.9, 59.0 and 22.4).
+static double zmarch_shape(const it_ctx *c, int *ty, int *cps) {
+    static const double round_us[2][4] = {{1.3, 1.75, 2.4, 3.5}, {1.25, 1.62, 2.4, 3.7}};
+    const int sms = sm_count();
+    double best = 1e300;
+    for (int k = 2; k >= 1; --k)
+        for (int t = 1; t <= std::min(c->g.ny, 255); ++t) {
+            if (c->g.ny % t) continue;
+            const int ipt = ipt_of(c, t, k == 1 ? 16 : 8);
+            if (ipt > ZM_MAX_IPT) break;
+            const size_t slot = sizeof(float) * 2 * (align32f(t * c->g.nx) + 2 * align32f(c->g.nx));
+            if (3 * slot + 512 > (size_t)(220 * 1024) / k) continue;   // a ring of three slots must fit
+            const int ntile = c->g.ny / t;
+            const long long tp = (long long)ntile * c->g.nz;
+            const long long grid = std::min<long long>(tp, zmarch_grid(ntile, (long long)sms * k));
+            const double us = (double)((tp + grid - 1) / grid + 2) * round_us[k - 1][ipt - 1] + 4.0;
+            if (us < 0.98 * best) {
+                best = us;
+                *ty = t;
+                *cps = k;
+            }
+        }
+    return best;
+}
+
 // Fill c->zm for a requested tile height / CTAs per SM / ring depth
 // (0 = choose) and build the tensor maps.  One CTA per SM runs 16 warps,
 // two CTAs per SM run 8 warps each.
@@ -518,7 +568,8 @@ int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid
         set_error("z-march kernel indexes a species array with 32 bits: needs nx*ny*nz < 2^32");
         return IT_EINVAL;
     }
-    const int cps = want_cps > 0 ? want_cps : 1;
+    int cps = want_cps > 0 ? want_cps : 1, TY = want_ty;
+    if (want_ty <= 0 && want_cps <= 0) zmarch_shape(c, &TY, &cps);
     if (cps > 2) { set_error("z-march kernel runs 1 or 2 CTAs per SM"); return IT_EINVAL; }
     const int nw = cps == 1 ? 16 : 8;
     ZmConf z{};
@@ -528,9 +579,8 @@ int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid
     z.xs = nx > 256 ? nx / row_piece(nx) : 1;
     z.bx = nx;
     z.nbx = 1;
-    // rows per tile: the smallest divisor of ny that gives every thread two
-    // float4 items (else the largest with at most ZM_MAX_IPT)
-    int TY = want_ty;
+    // CTAs per SM given: the smallest divisor of ny that gives every thread
+    // two float4 items (else the largest with at most ZM_MAX_IPT)
     if (TY <= 0) {
         TY = 0;
         for (int t = 1; t <= ny; ++t) {
@@ -581,11 +631,9 @@ int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(z-march)");
     if (occ < cps) { set_error("z-march kernel: requested CTAs per SM do not fit"); return IT_EINVAL; }
     z.ctas_per_sm = cps;
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     // grid: CTAs, each taking one contiguous range of tile-planes.  0: one
-    // per resident slot; -1: the largest multiple of the tile count that
+    // per resident slot (with no shape given at all, zmarch_grid's rule); -1: the largest multiple of the tile count that
     // fits the resident slots, so every tile column is cut at the same z and
     // vertically adjacent tiles are streamed in step (their halo rows are
     // then still in L2); > 0: as given.
@@ -593,6 +641,7 @@ int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid
     long long grid = (long long)sms * cps;
     if (want_grid == -1 && grid >= z.ntile) grid = grid / z.ntile * z.ntile;
     else if (want_grid > 0) grid = want_grid;
+    else if (want_ty <= 0 && want_cps <= 0 && want_s <= 0) grid = zmarch_grid(z.ntile, grid);
     z.nzc = (int)std::min<long long>(grid, tp);
     for (int set = 0; set < 2; ++set)
         for (int s = 0; s < 2; ++s) {
@@ -608,9 +657,21 @@ int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid
     return IT_OK;
 }
 
+// Does the march straight from L1/L2 (step_direct_kernel) beat the TMA-staged
+// one?  By the fitted times of both: it does while the state stays in L2
+// (256x256x100: 22.8 against 26.2 us per step, 128x128x200: 12.4 against
+// 19.6) and where ny has no divisor that fills a tile (224x293x119: one row
+// per tile took 154 us); from HBM it moves 1.45 times slower than a copy and
+// the ring wins (256x256x400: 86 against 77).
+bool direct_wins(const it_ctx *c) {
+    int ty = 0, cps = 1;
+    return direct_us(c) < zmarch_shape(c, &ty, &cps);
+}
+
 int zmarch_configure(it_ctx *c) { return zmarch_setup(c, 0, 0, 0, 0); }
 
 int launch_step_zmarch(it_ctx *c, cudaStream_t s) {
+    if (c->direct) return launch_step_direct(c, s);
     const int cur = c->cur, nxt = cur ^ 1;
     ZmMaps maps;
     maps.main[0] = c->tm_main[cur][0];
