@@ -150,7 +150,7 @@ static int ensure_tracks(it_ctx *c, int64_t n) {
     cudaFree(c->d_tracks); cudaFree(c->d_wx); cudaFree(c->d_wy);
     c->d_tracks = c->d_wx = c->d_wy = nullptr;
     c->track_cap = 0;
-    IT_CK(cudaMalloc(&c->d_tracks, sizeof(double) * 4 * n));
+    IT_CK(cudaMalloc(&c->d_tracks, kTrackScratch * n));
     IT_CK(cudaMalloc(&c->d_wx, sizeof(double) * c->g.nx * n));
     IT_CK(cudaMalloc(&c->d_wy, sizeof(double) * c->g.ny * n));
     c->track_cap = n;

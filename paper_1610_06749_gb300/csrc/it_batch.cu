@@ -1117,7 +1117,7 @@ int deposit_sim(it_batch *b, int sim, const double *packed, int64_t n) {
         b->d_tracks = b->d_wx = b->d_wy = nullptr;
         b->track_cap = 0;
         cudaError_t e;
-        if ((e = cudaMalloc(&b->d_tracks, sizeof(double) * 4 * n)) != cudaSuccess ||
+        if ((e = cudaMalloc(&b->d_tracks, kTrackScratch * n)) != cudaSuccess ||
             (e = cudaMalloc(&b->d_wx, sizeof(double) * b->max_nx * n)) != cudaSuccess ||
             (e = cudaMalloc(&b->d_wy, sizeof(double) * b->max_ny * n)) != cudaSuccess) {
             delete v;

@@ -90,6 +90,9 @@ struct Zm2Conf {
     int threads, ctas_per_sm, grid;
 };
 
+// device bytes per track of a deposit: its record and its window of cells
+constexpr size_t kTrackScratch = 4 * sizeof(double) + 4 * sizeof(int);
+
 // tallies of one context kept on the device
 struct DevAcc {
     double released[2];
@@ -120,7 +123,7 @@ struct it_ctx {
     double *h_out;        // pinned mirror
     // deposition scratch
     double *d_plane;      // [ny][nx] plane, then the per-tile sums of the deposit
-    double *d_tracks;     // [cap][4]: x, y, LET, b
+    double *d_tracks;     // [n][4]: x, y, LET, b, then the n tracks' windows (kTrackScratch bytes per track)
     double *d_angled;     // [angled_cap][5] tilted tracks (x, y, N0, b, theta), then per-block sums
     int64_t angled_cap;
     double *d_wx, *d_wy;  // [cap][nx], [cap][ny]

@@ -710,112 +710,150 @@ __device__ __forceinline__ long long floor_div(long long a, long long n) {
     return (a >= 0) ? a / n : -((-a + n - 1) / n);
 }
 
+// A track's window of cells on each axis (+-ceil(6 b/dx) around its cell):
+// the first cell (wrapped into the axis when periodic, clipped when
+// absorbing) and the number of cells, at most the axis.
+struct DepWindow { int x, nx, y, ny; };
+
 // Per track and axis: the fraction of the 1D Gaussian factor
 // exp(-u^2/b^2)/(sqrt(pi) b) that falls in each cell, summed over the
 // periodic images of the cell inside the window +-ceil(6 b/dx) around the
-// centre cell (absorbing faces: only the cell itself, if inside).
-__global__ void deposit_tables_kernel(const double *__restrict__ tr, double dx, int nx, int ny,
-                                      int periodic, double *__restrict__ wx, double *__restrict__ wy) {
-    const long long t = blockIdx.x;
-    const int axis = blockIdx.y;
+// centre cell (absorbing faces: only the cell itself, if inside); the x table
+// carries the track's ions per cm.  One warp per track and axis walks the
+// cells from the window's start, so that a cell edge's error function is
+// evaluated once, by the lane that owns it, and the next lane takes it by
+// shuffle.  (A block per track and axis with two error functions per cell
+// took 74 us for 2000 tracks on 256x256, this takes 28.)
+__global__ void __launch_bounds__(128)
+deposit_tables_kernel(const double *__restrict__ tr, long long nt, double dx, int nx, int ny, int periodic,
+                      double inv_W, double *__restrict__ wx, double *__restrict__ wy, DepWindow *__restrict__ win) {
+    const long long unit = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (unit >= 2 * nt) return;
+    const long long t = unit >> 1;
+    const int axis = (int)(unit & 1);
     const int n = axis ? ny : nx;
     const double ctr = tr[t * 4 + axis];
     const double b = tr[t * 4 + 3];
+    const double f = axis ? 1.0 : tr[t * 4 + 2] * 1e7 * inv_W;   // ions per cm, on the x table
     const long long w = (long long)ceil(6.0 * b / dx);
     const long long ic = (long long)floor(ctr / dx);
     const long long lo = ic - w, hi = ic + w;
     double *out = axis ? (wy + t * ny) : (wx + t * nx);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        double sum = 0.0;
-        if (periodic) {
+    int start, count;   // the window on the axis
+    if (periodic) {
+        start = (int)(lo - n * floor_div(lo, n));
+        count = (int)min((long long)n, 2 * w + 1);
+    } else {
+        const long long c0 = lo > 0 ? lo : 0, c1 = hi < n - 1 ? hi : n - 1;
+        start = c1 >= c0 ? (int)c0 : 0;
+        count = c1 >= c0 ? (int)(c1 - c0 + 1) : 0;
+    }
+    if (lane == 0) {
+        int *o = reinterpret_cast<int *>(win + t) + 2 * axis;
+        o[0] = start;
+        o[1] = count;
+    }
+    if (periodic && 2 * w + 1 > n) {   // a cell has several images: sum them, lowest first
+        for (int i = lane; i < n; i += 32) {
+            double sum = 0.0;
             long long ii = i + n * (-floor_div(-(lo - i), n));   // first image >= lo
             for (; ii <= hi; ii += n)
                 sum += 0.5 * (erf(((double)(ii + 1) * dx - ctr) / b) - erf(((double)ii * dx - ctr) / b));
-        } else if (i >= lo && i <= hi) {
-            sum = 0.5 * (erf(((double)(i + 1) * dx - ctr) / b) - erf(((double)i * dx - ctr) / b));
+            out[i] = f * sum;
         }
-        out[i] = sum;
+        return;
+    }
+    // cell m of the walk is cell (start + m) mod n; its unwrapped index is
+    // first + m, and 31 cells a round share 32 edges
+    const long long first = periodic ? lo : start;
+    for (int m0 = 0; m0 < n; m0 += 31) {
+        const int m = m0 + lane;
+        double e = 0.0;
+        if (m0 < count) e = m <= count ? erf(((double)(first + m) * dx - ctr) / b) : 0.0;
+        const double up = __shfl_down_sync(0xffffffffu, e, 1);
+        if (lane < 31 && m < n) {
+            int i = start + m;
+            if (i >= n) i -= n;
+            out[i] = m < count ? f * (0.5 * (up - e)) : 0.0;
+        }
     }
 }
 
-// Does the deposit window of a track (+-w cells around cell ic, wrapped on a
-// periodic axis of n cells) reach the cells [t0, t0 + tn)?  Conservative: a
-// track that only touches zero weights is harmless (it adds exact zeros).
-__device__ __forceinline__ bool window_hits(long long ic, long long w, int t0, int tn, int n, bool periodic) {
-    if (periodic) {
-        if (2 * w + 1 >= n) return true;
-        long long d = ((long long)t0 - (ic - w)) % n;
-        if (d < 0) d += n;
-        return d <= 2 * w || d + tn - 1 >= n;
-    }
-    return ic + w >= t0 && ic - w <= t0 + tn - 1;
+// Does a window reach the cells [t0, t0 + tn) of an axis of n cells?
+__device__ __forceinline__ bool window_hits(int start, int count, int t0, int tn, int n, bool periodic) {
+    if (!periodic) return start < t0 + tn && start + count > t0;
+    int d = t0 - start;
+    if (d < 0) d += n;
+    return d < count || d + tn - 1 >= n;
 }
 
-constexpr int DEP_TILE = 16;      // 16 x 16 cells per CTA
-constexpr int DEP_LIST = 1024;    // tracks gathered per pass
+constexpr int DEP_TILE = 8;       // 8 x 8 cells per CTA
+constexpr int DEP_LIST = 512;     // tracks gathered per pass
 
 // plane[j][i] = sum_t N0_t wx[t][i] wy[t][j] / dx^2, tracks in index order.
 // Each CTA first lists (in index order) the tracks whose window reaches its
 // tile, then every cell sums over that list; tracks that miss the tile only
 // contribute zeros, so the per-cell sum is the same as over all tracks.
-// part[blockIdx] receives the tile's sum of the plane (FP64).
+// part[blockIdx] receives the tile's sum of the plane (FP64).  Bound by the
+// chain of additions per cell and by the scan; small tiles keep the lists
+// short and give a 48x48 section 36 CTAs (16x16 tiles with 64-bit window
+// arithmetic in every scan: 93 us on 256x256 with 2000 tracks and 120 us on
+// 48x48 with up to 500; this: 23 and 30).
 __global__ void __launch_bounds__(DEP_TILE *DEP_TILE)
-deposit_plane_kernel(const double *__restrict__ tr, const double *__restrict__ wx, const double *__restrict__ wy,
-                     long long nt, int nx, int ny, double dx, int periodic, double inv_dx2, double inv_W,
-                     double *__restrict__ plane, double *__restrict__ part) {
+deposit_plane_kernel(const DepWindow *__restrict__ win, const double *__restrict__ wx, const double *__restrict__ wy,
+                     long long nt, int nx, int ny, int periodic, double inv_dx2, double *__restrict__ plane,
+                     double *__restrict__ part) {
+    constexpr int NTH = DEP_TILE * DEP_TILE, NWARP = NTH / 32;
     __shared__ int list[DEP_LIST];
-    __shared__ int wcount[DEP_TILE * DEP_TILE / 32];
-    __shared__ int nlist;
+    __shared__ int wcount[NWARP];
     __shared__ double red[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int i0 = blockIdx.x * DEP_TILE, j0 = blockIdx.y * DEP_TILE;
     const int tnx = min(DEP_TILE, nx - i0), tny = min(DEP_TILE, ny - j0);
-    const int i = i0 + (tid % DEP_TILE), j = j0 + (tid / DEP_TILE);
     const bool inside = (tid % DEP_TILE) < tnx && (tid / DEP_TILE) < tny;
+    const int i = inside ? i0 + (tid % DEP_TILE) : i0, j = inside ? j0 + (tid / DEP_TILE) : j0;
     double sum = 0.0;
     for (long long base = 0; base < nt;) {
-        if (tid == 0) nlist = 0;
-        __syncthreads();
-        // gather up to DEP_LIST candidates in index order, 256 tracks per round
+        // gather up to DEP_LIST candidates in index order, NTH tracks per round
+        int n = 0;
         long long t0 = base;
-        for (; t0 < nt; t0 += blockDim.x) {
+        for (; t0 < nt && n + NTH <= DEP_LIST; t0 += NTH) {
             const long long t = t0 + tid;
             bool hit = false;
             if (t < nt) {
-                const double b = tr[t * 4 + 3];
-                const long long w = (long long)ceil(6.0 * b / dx);
-                hit = window_hits((long long)floor(tr[t * 4] / dx), w, i0, tnx, nx, periodic != 0) &&
-                      window_hits((long long)floor(tr[t * 4 + 1] / dx), w, j0, tny, ny, periodic != 0);
+                const DepWindow w = win[t];
+                hit = window_hits(w.x, w.nx, i0, tnx, nx, periodic != 0) &&
+                      window_hits(w.y, w.ny, j0, tny, ny, periodic != 0);
             }
             const unsigned bal = __ballot_sync(0xffffffffu, hit);
             if (lane == 0) wcount[warp] = __popc(bal);
             __syncthreads();
             int before = 0, total = 0;
-            for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
+#pragma unroll
+            for (int q = 0; q < NWARP; ++q) {
                 if (q < warp) before += wcount[q];
                 total += wcount[q];
             }
-            const int start = nlist;
-            if (total > DEP_LIST - start) {   // list full: stop before this round, take it next pass
-                __syncthreads();
-                break;
-            }
-            if (hit) list[start + before + __popc(bal & ((1u << lane) - 1u))] = (int)t;
-            __syncthreads();
-            if (tid == 0) nlist = start + total;
+            if (hit) list[n + before + __popc(bal & ((1u << lane) - 1u))] = (int)t;
+            n += total;
             __syncthreads();
         }
-        const int n = nlist;
-        if (inside) {
-            for (int q = 0; q < n; ++q) {
-                const long long t = list[q];
-                const double a = wx[t * nx + i];
-                if (a == 0.0) continue;
-                const double bb = wy[t * ny + j];
-                if (bb == 0.0) continue;
-                const double N0 = tr[t * 4 + 2] * 1e7 * inv_W;   // ions per cm
-                sum += N0 * a * bb;
+        int q = 0;
+        for (; q + 4 <= n; q += 4) {   // four tracks' loads in flight, added in order
+            double a[4], c[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const long long t = list[q + r];
+                a[r] = wx[t * nx + i];
+                c[r] = wy[t * ny + j];
             }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) sum = fma(a[r], c[r], sum);
+        }
+        for (; q < n; ++q) {
+            const long long t = list[q];
+            sum = fma(wx[t * nx + i], wy[t * ny + j], sum);
         }
         base = t0;
         __syncthreads();
@@ -894,17 +932,17 @@ int launch_deposit(it_ctx *c, int64_t n, cudaStream_t s) {
     if (n <= 0) return IT_OK;
     const int nx = c->g.nx, ny = c->g.ny;
     const bool periodic = c->p.lateral_bc == IT_PERIODIC;
-    dim3 gt((unsigned)n, 2);
-    deposit_tables_kernel<<<gt, 128, 0, s>>>(c->d_tracks, c->dx, nx, ny, periodic, c->d_wx, c->d_wy);
+    DepWindow *win = reinterpret_cast<DepWindow *>(c->d_tracks + 4 * n);   // after the track records
+    deposit_tables_kernel<<<(unsigned)((2 * n + 3) / 4), 128, 0, s>>>(c->d_tracks, n, c->dx, nx, ny, periodic,
+                                                                     1.0 / c->p.W_eV, c->d_wx, c->d_wy, win);
     IT_CK(cudaGetLastError());
     const long long pn = (long long)nx * ny;
     dim3 gp((nx + DEP_TILE - 1) / DEP_TILE, (ny + DEP_TILE - 1) / DEP_TILE);
     const size_t nparts = (size_t)gp.x * gp.y;
     // the tile sums go after the plane in the same scratch buffer
     double *part = c->d_plane + pn;
-    deposit_plane_kernel<<<gp, DEP_TILE * DEP_TILE, 0, s>>>(c->d_tracks, c->d_wx, c->d_wy, n, nx, ny, c->dx,
-                                                            periodic ? 1 : 0, 1.0 / (c->dx * c->dx),
-                                                            1.0 / c->p.W_eV, c->d_plane, part);
+    deposit_plane_kernel<<<gp, DEP_TILE * DEP_TILE, 0, s>>>(win, c->d_wx, c->d_wy, n, nx, ny, periodic ? 1 : 0,
+                                                            1.0 / (c->dx * c->dx), c->d_plane, part);
     IT_CK(cudaGetLastError());
     const unsigned kchunks = (unsigned)((c->g.nz + DEP_KCHUNK - 1) / DEP_KCHUNK);
     if (c->prec == IT_FP32 && nx % 4 == 0)
