@@ -543,14 +543,23 @@ int it_deposit_tracks_angled(it_ctx *c, int64_t n, const double *xy, const doubl
         if (!(theta[t] >= 0.0 && theta[t] <= 1.5707963267948966))
             return fail(IT_EINVAL, "theta must lie in [0, pi/2]");
     if (n > (1 << 20)) return fail(IT_EINVAL, "at most 2^20 tilted tracks per call");
-    // track records, then one FP64 partial sum per block of the kernel
+    // track records, one FP64 partial sum per block of the kernel without
+    // tables, then the tables
     constexpr int kBlocks = 1216;   // 8 per SM on 152 SMs; fixed, so the sums are deterministic
-    const int64_t need = 5 * n + kBlocks;
+    int64_t tab = angled_table_doubles(c, n);
+    int64_t need = 5 * n + kBlocks + tab;
     if (need > c->angled_cap) {
         cudaFree(c->d_angled);
         c->d_angled = nullptr;
         c->angled_cap = 0;
-        IT_CK(cudaMalloc(&c->d_angled, sizeof(double) * need));
+        cudaError_t e = cudaMalloc(&c->d_angled, sizeof(double) * need);
+        if (e == cudaErrorMemoryAllocation && tab > 0) {   // no room for the tables: the kernel without them
+            (void)cudaGetLastError();
+            tab = 0;
+            need = 5 * n + kBlocks;
+            e = cudaMalloc(&c->d_angled, sizeof(double) * need);
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(tilted tracks)");
         c->angled_cap = need;
     }
     std::vector<double> h((size_t)5 * n);
@@ -562,7 +571,8 @@ int it_deposit_tracks_angled(it_ctx *c, int64_t n, const double *xy, const doubl
         h[5 * t + 4] = theta[t];
     }
     IT_CK(cudaMemcpyAsync(c->d_angled, h.data(), sizeof(double) * 5 * n, cudaMemcpyHostToDevice, c->stream));
-    rc = launch_deposit_angled(c, c->d_angled, n, c->d_angled + 5 * n, kBlocks, c->stream);
+    rc = launch_deposit_angled(c, c->d_angled, n, c->d_angled + 5 * n, kBlocks,
+                               tab > 0 ? c->d_angled + 5 * n + kBlocks : nullptr, c->stream);
     if (rc) return rc;
     IT_CK(cudaStreamSynchronize(c->stream));   // the host records are released on return
     return IT_OK;

@@ -124,7 +124,7 @@ struct it_ctx {
     // deposition scratch
     double *d_plane;      // [ny][nx] plane, then the per-tile sums of the deposit
     double *d_tracks;     // [n][4]: x, y, LET, b, then the n tracks' windows (kTrackScratch bytes per track)
-    double *d_angled;     // [angled_cap][5] tilted tracks (x, y, N0, b, theta), then per-block sums
+    double *d_angled;     // [angled_cap][5] tilted tracks (x, y, N0, b, theta), then per-block sums, then the tables
     int64_t angled_cap;
     double *d_wx, *d_wy;  // [cap][nx], [cap][ny]
     int64_t track_cap;
@@ -196,7 +196,9 @@ int launch_finalize(it_ctx *c, cudaStream_t s);
 int launch_monitor(it_ctx *c, cudaStream_t s);
 int launch_deposit(it_ctx *c, int64_t n, cudaStream_t s);   // tracks already in d_tracks
 int launch_zero(void *p, size_t bytes, cudaStream_t s);
-int launch_deposit_angled(it_ctx *c, const double *d_tr, int64_t n, double *d_part, int nblocks, cudaStream_t s);
+int launch_deposit_angled(it_ctx *c, const double *d_tr, int64_t n, double *d_part, int nblocks, double *d_tab,
+                          cudaStream_t s);
+int64_t angled_table_doubles(const it_ctx *c, int64_t n);
 int simple_grid(const it_ctx *c);
 int simple_grid_f32(int nx, int ny, int nz);
 int launch_step_simple_raw_f32(const float *ip, const float *im, float *op, float *om, int nx, int ny, int nz,

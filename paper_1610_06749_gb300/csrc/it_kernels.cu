@@ -1048,10 +1048,164 @@ deposit_angled_kernel(const double *__restrict__ tr, int n, int nx, int ny, int 
     if (threadIdx.x == 0) part[blockIdx.x] = bsum[0];
 }
 
-int launch_deposit_angled(it_ctx *c, const double *d_tr, int64_t n, double *d_part, int nblocks, cudaStream_t s) {
+// The same deposit from tables, for the few tracks it is meant for: in every
+// plane a tilted column is an x profile times a y profile, so the error
+// functions (and, parallel to the electrodes, the exponential) are evaluated
+// once per (track, plane, column) and once per (track, row), not once per
+// cell and track.  ay[t][j] holds wy; ax[t][k][i] holds wx with the track's
+// ions per cm and 1/dx^2, so a cell adds one product per track.
+// One warp per row of a table; lane 0 writes the row's sum: rows [0, n) are
+// the y rows, row n + t nz + k the x row of track t and plane k.
+__global__ void __launch_bounds__(128)
+angled_tables_kernel(const double *__restrict__ tr, int n, int nx, int ny, int nz, double dx, int periodic,
+                     double *__restrict__ ax, double *__restrict__ ay, double *__restrict__ rowsum) {
+    const long long row = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (row >= (long long)n * (nz + 1)) return;
+    const double zmid = 0.5 * nz * dx;
+    const double sqrt_pi = 1.7724538509055160272981674833411;
+    double sum = 0.0;
+    if (row < n) {
+        const double y0 = tr[5 * row + 1], b = tr[5 * row + 3];
+        const int w = (int)ceil(6.0 * b / dx), jc = (int)floor(y0 / dx);
+        for (int j = lane; j < ny; j += 32) {
+            const double v = image_weights(j, ny, jc - w, jc + w, y0, b, dx, periodic);
+            ay[row * ny + j] = v;
+            sum += v;
+        }
+    } else {
+        const long long q = row - n;
+        const int t = (int)(q / nz), k = (int)(q - (long long)t * nz);
+        const double x0 = tr[5 * t], N0 = tr[5 * t + 2], b = tr[5 * t + 3], th = tr[5 * t + 4];
+        const double zk = (k + 0.5) * dx;
+        double *out = ax + q * nx;
+        const double c = cos(th), sn = sin(th);
+        if (c * dx / b < 1e-3) {
+            for (int i = lane; i < nx; i += 32) {
+                const double u = ((i + 0.5) * dx - x0) * c - (zk - zmid) * sn;
+                const double v = N0 / (sqrt_pi * b) * exp(-(u * u) / (b * b)) / dx;
+                out[i] = v;
+                sum += v;
+            }
+        } else {
+            const double xc = x0 + (zk - zmid) * sn / c;
+            const int w = (int)ceil(6.0 * b / (dx * c)), ic = (int)floor(xc / dx);
+            const double f = N0 / c / (dx * dx);
+            for (int i = lane; i < nx; i += 32) {
+                const double v = f * image_weights(i, nx, ic - w, ic + w, xc, b / c, dx, periodic);
+                out[i] = v;
+                sum += v;
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+    if (lane == 0) rowsum[row] = sum;
+}
+
+// n += sum over the tracks of ax[t][k][i] ay[t][j].  Thread = V adjacent
+// cells of a row (float4 when the state is FP32 and nx % 4 == 0); cells no
+// track reaches are neither read nor written.  FP32 states add the FP64 sum
+// rounded once, as the other deposits do.
+template <typename T, int V, typename Idx>
+__global__ void __launch_bounds__(256)
+angled_apply_kernel(const double *__restrict__ ax, const double *__restrict__ ay, int n, int nx, int ny, int nz,
+                    T *__restrict__ p, T *__restrict__ m) {
+    const Idx nxv = (Idx)(nx / V);
+    const Idx total = nxv * (Idx)ny * (Idx)nz;
+    for (Idx e = (Idx)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (Idx)gridDim.x * blockDim.x) {
+        const Idx r = e / nxv;
+        const int i = (int)(e - r * nxv) * V, k = (int)(r / (Idx)ny), j = (int)(r - (Idx)k * (Idx)ny);
+        double v[V] = {};
+        bool any = false;
+        for (int t = 0; t < n; ++t) {
+            const double y = ay[(long long)t * ny + j];
+            if (y == 0.0) continue;
+            const double *x = ax + ((long long)t * nz + k) * nx + i;
+#pragma unroll
+            for (int q = 0; q < V; ++q) {
+                const double xv = x[q];
+                v[q] = fma(xv, y, v[q]);
+                any |= xv != 0.0;
+            }
+        }
+        if (!any) continue;
+        const size_t idx = (size_t)r * nx + i;
+        if constexpr (V == 4) {
+            float4 a = *reinterpret_cast<float4 *>(p + idx), b = *reinterpret_cast<float4 *>(m + idx);
+            const float4 f = make_float4(__double2float_rn(v[0]), __double2float_rn(v[1]), __double2float_rn(v[2]),
+                                         __double2float_rn(v[3]));
+            a.x = __fadd_rn(a.x, f.x); a.y = __fadd_rn(a.y, f.y); a.z = __fadd_rn(a.z, f.z); a.w = __fadd_rn(a.w, f.w);
+            b.x = __fadd_rn(b.x, f.x); b.y = __fadd_rn(b.y, f.y); b.z = __fadd_rn(b.z, f.z); b.w = __fadd_rn(b.w, f.w);
+            *reinterpret_cast<float4 *>(p + idx) = a;
+            *reinterpret_cast<float4 *>(m + idx) = b;
+        } else if constexpr (sizeof(T) == 4) {
+            const float f = __double2float_rn(v[0]);
+            p[idx] = __fadd_rn(p[idx], f);
+            m[idx] = __fadd_rn(m[idx], f);
+        } else {
+            p[idx] += v[0];
+            m[idx] += v[0];
+        }
+    }
+}
+
+// released += sum over tracks and planes of (x row sum) (y row sum) * vol
+__global__ void __launch_bounds__(256)
+angled_released_kernel(const double *__restrict__ rowsum, int n, int nz, double vol, double *__restrict__ acc) {
+    __shared__ double red[32];
+    double v[1] = {0.0};
+    const long long rows = (long long)n * nz;
+    for (long long q = threadIdx.x; q < rows; q += blockDim.x) v[0] = fma(rowsum[n + q], rowsum[q / nz], v[0]);
+    block_sum<1>(v, red);
+    if (threadIdx.x == 0) {
+        acc[0] += v[0] * vol;
+        acc[1] += v[0] * vol;
+    }
+}
+
+// Doubles of scratch the tables of n tracks take, 0 where the kernel without
+// tables is used: the x tables hold nz nx doubles per track, so many tracks
+// on a large section would outgrow the section's own state.  Up to 256 MB
+// (26 tracks on 200x200x800) the tables win by far: one iron track there
+// takes 0.25 ms against 19.5 (0.19 of it adds 32M cells, bound by the FP64
+// product and conversion per cell).
+int64_t angled_table_doubles(const it_ctx *c, int64_t n) {
+    const double need = (double)n * ((double)c->g.nz * c->g.nx + c->g.ny + c->g.nz + 1);
+    if (need * sizeof(double) > 256.0 * 1024 * 1024) return 0;
+    return (int64_t)need;
+}
+
+int launch_deposit_angled(it_ctx *c, const double *d_tr, int64_t n, double *d_part, int nblocks, double *d_tab,
+                          cudaStream_t s) {
     if (n <= 0) return IT_OK;
     const int nx = c->g.nx, ny = c->g.ny, nz = c->g.nz;
     const int per = c->p.lateral_bc == IT_PERIODIC ? 1 : 0;
+    const double vol = c->dx * c->dx * c->dx;
+    if (d_tab) {
+        double *ax = d_tab, *ay = ax + n * nz * (int64_t)nx, *rowsum = ay + n * ny;
+        const long long rows = n * (nz + 1);
+        angled_tables_kernel<<<(unsigned)((rows + 3) / 4), 128, 0, s>>>(d_tr, (int)n, nx, ny, nz, c->dx, per, ax, ay,
+                                                                       rowsum);
+        IT_CK(cudaGetLastError());
+        const int cur = c->cur;
+        const size_t cells = c->g.cells();
+        const bool small = cells <= 0xf0000000ull;
+        const bool v4 = c->prec == IT_FP32 && nx % 4 == 0;
+        const size_t items = v4 ? cells / 4 : cells;
+        // a few rounds per thread on large grids
+        const unsigned grid = (unsigned)std::min<size_t>((items + 255) / 256, 152 * 64);
+        auto go = [&](auto *k, auto *pp, auto *mm) { k<<<grid, 256, 0, s>>>(ax, ay, (int)n, nx, ny, nz, pp, mm); };
+        float *pf = (float *)c->n[cur][0], *mf = (float *)c->n[cur][1];
+        double *pd = (double *)c->n[cur][0], *md = (double *)c->n[cur][1];
+        if (v4) small ? go(angled_apply_kernel<float, 4, uint32_t>, pf, mf) : go(angled_apply_kernel<float, 4, uint64_t>, pf, mf);
+        else if (c->prec == IT_FP32) small ? go(angled_apply_kernel<float, 1, uint32_t>, pf, mf) : go(angled_apply_kernel<float, 1, uint64_t>, pf, mf);
+        else small ? go(angled_apply_kernel<double, 1, uint32_t>, pd, md) : go(angled_apply_kernel<double, 1, uint64_t>, pd, md);
+        IT_CK(cudaGetLastError());
+        angled_released_kernel<<<1, 256, 0, s>>>(rowsum, (int)n, nz, vol, c->d_acc);
+        IT_CK(cudaGetLastError());
+        return IT_OK;
+    }
     if (c->prec == IT_FP32)
         deposit_angled_kernel<float><<<nblocks, 256, 0, s>>>(d_tr, (int)n, nx, ny, nz, c->dx, per,
                                                              (float *)c->n[c->cur][0], (float *)c->n[c->cur][1],
@@ -1061,7 +1215,6 @@ int launch_deposit_angled(it_ctx *c, const double *d_tr, int64_t n, double *d_pa
                                                               (double *)c->n[c->cur][0],
                                                               (double *)c->n[c->cur][1], d_part);
     IT_CK(cudaGetLastError());
-    const double vol = c->dx * c->dx * c->dx;
     deposit_released_kernel<<<1, 256, 0, s>>>(d_part, (size_t)nblocks, vol, c->d_acc);
     IT_CK(cudaGetLastError());
     return IT_OK;
