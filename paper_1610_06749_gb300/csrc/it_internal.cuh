@@ -187,7 +187,7 @@ int encode_map(CUtensorMap *m, void *base, int nx, int ny, int nz, int bx, int r
 int row_piece(int nx);
 int encode_map_rows(CUtensorMap *m, void *base, int nx, int ny, int nz, int rows);
 int encode_bf16_sw128(CUtensorMap *m, const void *base, long long K, long long rows, long long members,
-                      long long row_bytes, long long member_bytes);
+                      long long row_bytes, long long member_bytes, int box_rows);
 // two steps per launch (it_zmarch2.cu)
 int zmarch2_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid);
 int launch_step_zmarch2(it_ctx *c, cudaStream_t s);

@@ -3,21 +3,27 @@
 //
 //   D[m][n] = sum_k A[m][k] B[n][k]        (A, B bf16, K contiguous; D FP32)
 //
-// One CTA of 128 threads computes a 128 x 128 tile of D for one ensemble
-// member (blockIdx.z):
+// One CTA of 256 threads computes a 128 x 32 tile of D for one ensemble
+// member (blockIdx.z).  At the network's sizes (256 x 256 outputs, a few
+// hundred samples) the epilogue on the CUDA cores is the long part of a tile,
+// so tiles are narrow and eight warps share one: a 256-sample product of five
+// members spreads over 80 CTAs, each warp with one 32 x 16 block (128 x 128
+// tiles on four warps: 20 CTAs, 22-26 us a product; 128 x 32 on four warps 7.4
+// (backward) and 8.7 (forward); this 6.1 and 7.4):
 //   * warp 0, one thread: TMA producer.  K is walked in chunks of 64
-//     elements (128 bytes), each chunk of A (128 rows) and B (128 rows)
-//     lands in one of four shared-memory stages with the 128-byte swizzle;
-//   * warp 1, one thread: issues tcgen05.mma (M = 128, N = 128, K = 16,
+//     elements (128 bytes), each chunk of A (128 rows) and B (32 rows)
+//     lands in one of three shared-memory stages with the 128-byte swizzle;
+//   * warp 1, one thread: issues tcgen05.mma (M = 128, N = 32, K = 16,
 //     kind::f16 with bf16 inputs and FP32 accumulation) from shared-memory
 //     descriptors, accumulating in tensor memory, and hands each stage back
 //     with tcgen05.commit once the MMAs reading it are done;
-//   * warp 2 allocates (and at the end frees) 128 columns of tensor memory;
-//   * all four warps then read the accumulator back with tcgen05.ld (warp w
-//     owns TMEM lanes 32w .. 32w+31, i.e. rows 32w .. 32w+31 of the tile) and
-//     run the epilogue functor on 32 x 32 blocks, each warp with a slice of
-//     the (by then idle) stage memory to reorder its block for coalesced
-//     stores.
+//   * warp 2 allocates (and at the end frees) 32 columns of tensor memory;
+//   * all eight warps then read the accumulator back with tcgen05.ld (warp w
+//     reaches TMEM lanes 32 (w mod 4) .., i.e. those rows of the tile, and
+//     takes columns 16 (w / 4) ..) and run the epilogue functor on their
+//     32 x 16 block, each warp with a slice
+//     of the (by then idle) stage memory to reorder its block for coalesced
+//     stores; what the epilogue reads is loaded before the wait.
 // Every mbarrier wait is bounded (about 2^31 SM cycles); a wait that runs
 // out raises the error flag, no further copy or MMA is issued, the copies
 // already issued are waited for, and tensor memory is freed before return.
@@ -34,11 +40,14 @@
 namespace itk {
 namespace tc {
 
-constexpr int TM = 128, TN = 128, TK = 64, STAGES = 4;
+constexpr int TM = 128, TN = 32, TK = 64, STAGES = 3;
+constexpr int THREADS = 256, NC = 16;   // columns of a warp's block
 constexpr int A_BYTES = TM * TK * 2, B_BYTES = TN * TK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
 // dynamic shared memory: the stages (1024-byte aligned for the 128-byte
 // swizzle) plus the alignment slack
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
+constexpr int SCRATCH = 32 * 20;   // floats of reordering scratch per warp
+static_assert(THREADS / 32 * SCRATCH * 4 <= STAGES * STAGE_BYTES, "scratch lies in the stages");
 constexpr long long WAIT_CYCLES = 1LL << 31;
 
 // shared-memory matrix descriptor of a K-major tile with the 128-byte
@@ -92,29 +101,29 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar) {
                  : "memory");
 }
 
-// 32 consecutive FP32 columns of this thread's TMEM lane
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32]) {
-    uint32_t r[32];
+// 16 consecutive FP32 columns of this thread's TMEM lane
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int q = 0; q < 32; ++q) v[q] = __uint_as_float(r[q]);
+    for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(r[q]);
 }
 
 // D = A B^T for the tile (blockIdx.y, blockIdx.x) of member blockIdx.z; M,
 // N: rows of D (TMA zero-fills the rows and the K tail outside the tensors;
 // the epilogue masks rows >= M).  The whole warp calls
-// epi(z, mw, lane, M, n0, v, scratch): lane holds D[mw + lane][n0 .. n0+31]
-// in v, scratch is 32 x 33 floats of shared memory of this warp alone.
+// epi.done(z, mw, lane, M, n0, v, scratch, pre): lane holds
+// D[mw + lane][n0 .. n0+15] in v, scratch is 32 x 20 floats of shared memory of
+// this warp alone (16-byte aligned), pre what epi.load(z, mw, lane, M, n0)
+// returned before the accumulator was waited for.
 template <class Epi>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(THREADS, 3)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, int M, int N, int K,
                Epi epi, int *__restrict__ err) {
     extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
@@ -181,6 +190,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ C
         tc_commit(&done);
     }
     __syncwarp();
+    // this warp's block of the tile
+    const int mw = m0 + (warp & 3) * 32, nw = (warp >> 2) * NC;
+    const auto pre = epi.load(z, mw, lane, M, n0 + nw);
     // every thread: the accumulator is complete (or the run was abandoned)
     const bool ok = tc_wait(&done, 0u);
     tc_fence_after();
@@ -189,14 +201,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ C
     if (!failed) {
         // every copy has landed and every MMA has read its operands: the
         // stage memory is free for the epilogue's reordering
-        float *scratch = reinterpret_cast<float *>(base) + warp * (32 * 33);
-        const uint32_t row = tmem + ((uint32_t)(warp * 32) << 16);
-#pragma unroll 1
-        for (int c = 0; c < TN; c += 32) {
-            float v[32];
-            tc_ld32(row + (uint32_t)c, v);
-            if (n0 + c < N) epi(z, m0 + warp * 32, lane, M, n0 + c, v, scratch);
-        }
+        float *scratch = reinterpret_cast<float *>(base) + warp * SCRATCH;
+        float v[NC];
+        tc_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)nw, v);
+        epi.done(z, mw, lane, M, n0 + nw, v, scratch, pre);
     }
     tc_fence_before();
     __syncthreads();
