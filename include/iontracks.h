@@ -380,7 +380,8 @@ typedef struct {
 int it_batch_create(int32_t nsim, const it_sim_desc *descs, const it_params *common, it_batch **out);
 
 /* Deposit n tracks into simulation `sim` (arrays as in it_deposit_tracks);
- * only before the first step (IT_ESTATE otherwise).  Synchronous. */
+ * only before the first step (IT_ESTATE otherwise).  Asynchronous on the
+ * batch's stream; the host arrays are read before the call returns. */
 int it_batch_deposit_tracks(it_batch *b, int32_t sim, int64_t n, const double *xy_cm,
                             const double *let_keV_um, const double *b_cm);
 
@@ -403,11 +404,12 @@ int it_batch_set_chunk(it_batch *b, int64_t cells_per_block);
 /* Native autotuner of the batched launch shape: after the deposits (and
  * it_batch_retime), before the first step.  Times trial_steps (>= 2, rounded
  * up to even) batched steps of the deposited state for each candidate --
- * the TMA-staged kernel with one or two float4 per thread or the register
- * float4 kernel, times z splits aiming at 1..32 CTAs per SM, times 4096 /
- * 16384 / 65536 cells per scalar-kernel entry when a simulation runs on the
- * scalar kernel (nx % 4 != 0) -- with CUDA events on the batch
- * stream, restores the deposited state after every trial (it allocates a
+ * the march straight from L1/L2 with two chunk lengths, the TMA-staged
+ * kernel with one or two float4 per thread times z splits aiming at 1..32
+ * CTAs per SM, times 4096 / 16384 / 65536 cells per single-cell entry when a
+ * simulation needs it (nx % 4 != 0) -- with CUDA events on the batch stream
+ * (a candidate whose first two steps are a twentieth slower than the best is
+ * not timed further), restores the deposited state after every trial (it allocates a
  * temporary copy of one state set, freed before return), keeps the fastest
  * and stores its microseconds per step in *best_us (may be NULL).  No tally
  * changes.  IT_ESTATE after the first step.  The paper has no batching; the

@@ -5,9 +5,9 @@
 // Gaussian / created, electrode tallies and f of Eq. collection_efficiency)
 // on its own grid, dx, voltage and time step.  All simulations live in four
 // shared FP32 arrays (two ping-pong sets of n+ and n-), each simulation
-// aligned to 256 bytes.  A work table lists (simulation, row range) entries;
-// one launch of step_batched_kernel advances every active simulation by one
-// of its own steps, and segments of launches are replayed from a CUDA graph.
+// aligned to 256 bytes.  Work tables list (simulation, tile or columns, planes)
+// entries; one step's launches advance every active simulation by one of its
+// own steps, and segments of launches are replayed from a CUDA graph.
 // At segment ends the per-entry tally slots are folded into per-simulation
 // FP64 accumulators in a fixed order, in-domain charge is measured, and
 // finished simulations leave the table.
@@ -20,6 +20,7 @@
 
 #include "it_device.cuh"
 #include "it_internal.cuh"
+#include "it_march.cuh"
 #include "it_tma.cuh"
 
 namespace itk {
@@ -35,237 +36,58 @@ struct BatchEntry {
     long long begin, end;   // row range inside the simulation (row = k * ny + j)
 };
 
-// One explicit step of the rows [begin, end) of one simulation; the same
-// per-cell operation sequence as the single-simulation kernels.  Thread t
-// owns x = t mod nx of every (256 / nx)-th row, so there is no division per
-// cell.
-template <bool PERIODIC, bool SC>
-__global__ void __launch_bounds__(256)
-step_batched_kernel(const BatchSim *__restrict__ sims, const BatchEntry *__restrict__ tab,
-                    const float *__restrict__ ip_all, const float *__restrict__ im_all, float *__restrict__ op_all,
-                    float *__restrict__ om_all, double *__restrict__ slots) {
-    constexpr int NQ = SC ? 9 : 7;   // tallies: 7, 9 with space charge
-    __shared__ double red[32 * NQ];
-    __shared__ BatchSim S;
-    __shared__ BatchEntry E;
-    if (threadIdx.x == 0) {
-        E = tab[blockIdx.x];
-        S = sims[E.sim];
-    }
+// Entry of the marches without a ring: 128 columns (x-segments of four cells,
+// or cells) from q0 of one simulation's flattened x-y plane, planes [k0, k1).
+struct MarchEntry {
+    int sim;
+    unsigned q0;
+    int k0, k1;
+};
+
+// the update weights of a simulation, in registers for the march
+struct RegCoef {
+    float wx[2], wzm[2], wzp[2], adt, sc[2];
+    __device__ __forceinline__ explicit RegCoef(const Coef<float> &c)
+        : wx{c.wx[0], c.wx[1]}, wzm{c.wzm[0], c.wzm[1]}, wzp{c.wzp[0], c.wzp[1]}, adt(c.adt), sc{c.sc[0], c.sc[1]} {}
+};
+
+// One step of an entry straight from L1/L2 (direct_march with V = 4: the
+// simulation's nx % 4 == 0; simple_march with V = 1: any nx): the same
+// marches as the single-grid kernels', one unit per block.  Against the
+// TMA-staged kernel it has no ring to fill and no tile that is mostly empty:
+// per step of surrogate simulations (48 x 48 cells) 256 of them take 136, 64
+// 40, 16 12.1 and four 6.3 us, against 166, 60, 20.7 and 16.5 with the ring
+// (85, 21, 5.6 and 1.1 at the copy rate); the 256 larger ones of the batched
+// workload, which stream from HBM, take 624 against 576.
+template <bool PERIODIC, bool SC, int V>
+__global__ void __launch_bounds__(SK_THREADS, (V == 4 ? DK_BLOCKS : SK_BLOCKS_F32))
+step_batched_march_kernel(const BatchSim *__restrict__ sims, const MarchEntry *__restrict__ tab,
+                          const float *__restrict__ ip_all, const float *__restrict__ im_all,
+                          float *__restrict__ op_all, float *__restrict__ om_all, double *__restrict__ slots) {
+    constexpr int NV = MarchValues<PERIODIC, SC>::N;
+    __shared__ double raw[5 * SK_THREADS];
+    CompSum(*buf)[SK_THREADS] = reinterpret_cast<CompSum(*)[SK_THREADS]>(raw);
+    __shared__ double tot[9];
+    const MarchEntry E = tab[blockIdx.x];
+    const BatchSim &S = sims[E.sim];
+    const RegCoef c(S.cf);
+    const long long off = S.off;
+    if (threadIdx.x < 9) tot[threadIdx.x] = 0.0;
+    if constexpr (V == 4)
+        direct_march<uint32_t, PERIODIC, SC>(ip_all + off, im_all + off, op_all + off, om_all + off, S.nx, S.ny, S.nz,
+                                             E.q0, E.k0, E.k1, c, buf, tot);
+    else
+        simple_march<float, uint32_t, PERIODIC, SC>(ip_all + off, im_all + off, op_all + off, om_all + off, S.nx, S.ny,
+                                                    S.nz, E.q0, E.k0, E.k1, c, buf, tot);
     __syncthreads();
-    const int nx = S.nx, ny = S.ny, nz = S.nz;
-    const Coef<float> &c = S.cf;
-    const float *ip = ip_all + S.off, *im = im_all + S.off;
-    float *op = op_all + S.off, *om = om_all + S.off;
-    const int plane = nx * ny;
-    const int R = nx <= (int)blockDim.x ? (int)blockDim.x / nx : 1;   // rows per pass
-    const int lane_row = nx <= (int)blockDim.x ? (int)threadIdx.x / nx : 0;
-    double acc[NQ] = {};
-    if (lane_row < R) {
-        const int i0 = nx <= (int)blockDim.x ? (int)threadIdx.x - lane_row * nx : (int)threadIdx.x;
-        long long row = E.begin + lane_row;
-        int k = (int)(row / ny), j = (int)(row - (long long)k * ny);
-        for (; row < E.end; row += R) {
-            for (int i = i0; i < nx; i += (nx <= (int)blockDim.x ? nx : (int)blockDim.x)) {
-                const int idx = (k * ny + j) * nx + i;
-                const int ixm = (i > 0) ? idx - 1 : idx + (nx - 1);
-                const int ixp = (i < nx - 1) ? idx + 1 : idx - (nx - 1);
-                const int iym = (j > 0) ? idx - nx : idx + (ny - 1) * nx;
-                const int iyp = (j < ny - 1) ? idx + nx : idx - (ny - 1) * nx;
-                const float p0 = ip[idx], m0 = im[idx];
-                const float rr = p0 * m0;
-                acc[0] += (double)rr;
-                const int cx = (i == 0) + (i == nx - 1);
-                const int cy = (j == 0) + (j == ny - 1);
-#pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    const float *in = s ? im : ip;
-                    const float n0 = s ? m0 : p0;
-                    const float xm = (PERIODIC || i > 0) ? in[ixm] : 0.f;
-                    const float xp = (PERIODIC || i < nx - 1) ? in[ixp] : 0.f;
-                    const float ym = (PERIODIC || j > 0) ? in[iym] : 0.f;
-                    const float yp = (PERIODIC || j < ny - 1) ? in[iyp] : 0.f;
-                    const float zm = (k > 0) ? in[idx - plane] : 0.f;
-                    const float zp = (k < nz - 1) ? in[idx + plane] : 0.f;
-                    float v =
-                        upd7(n0, xm, xp, ym, yp, zm, zp, rr, c.wx[s], c.wzm[s], c.wzp[s], c.adt);
-                    if constexpr (SC) {
-                        v = add_sc(v, c.sc[s], n0, p0, m0);
-                        acc[NQ - 2 + s] += (double)__fmul_rn(n0, __fsub_rn(p0, m0));
-                    }
-                    (s ? om : op)[idx] = v;
-                    if (k == 0) acc[1 + s] += (double)n0;
-                    if (k == nz - 1) acc[3 + s] += (double)n0;
-                    if (!PERIODIC && (cx | cy)) acc[5 + s] += (double)n0 * (cx * c.latx_f[s] + cy * c.laty_f[s]);
-                }
-            }
-            j += R;
-            while (j >= ny) { j -= ny; ++k; }
-        }
-    }
-    block_sum<NQ>(acc, red);
-    if (threadIdx.x == 0) {
-        double *sl = slots + (size_t)blockIdx.x * NT;
-        sl[0] += acc[0] * c.rec_f;
-        sl[1] += acc[1] * c.anode_f[0];
-        sl[2] += acc[2] * c.anode_f[1];
-        sl[3] += acc[3] * c.cathode_f[0];
-        sl[4] += acc[4] * c.cathode_f[1];
-        sl[5] += acc[5];
-        sl[6] += acc[6];
-        if constexpr (SC) {
-            sl[7] += acc[NQ - 2] * c.sc_f[0];
-            sl[8] += acc[NQ - 1] * c.sc_f[1];
-        }
-    }
+    if (threadIdx.x < 9) sk_slot<PERIODIC, SC, NV>(tot, S.cf, slots, threadIdx.x, 1);
 }
 
-// Entry of the float4 kernel: rows [y0, y0 + rows) of one simulation,
+// Entry of the TMA-staged kernel: rows [y0, y0 + rows) of one simulation,
 // planes [z0, z1).
 struct VecEntry {
     int sim, y0, rows, z0, z1, pad;
 };
-
-__device__ __forceinline__ float4 ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
-
-// Float4 z-march for simulations with nx % 4 == 0: thread t owns x-segment
-// 4 (t mod nx/4) of row t div (nx/4), keeps planes k-1, k, k+1 of it in
-// registers, reads the y-neighbour rows with 16-byte loads (mostly L1/L2
-// hits: they are other threads' centres), and takes x-neighbours by warp
-// shuffle.  Same per-cell operation sequence as every other kernel.
-template <bool PERIODIC, bool SC>
-__global__ void __launch_bounds__(256, 3)
-step_batched_vec_kernel(const BatchSim *__restrict__ sims, const VecEntry *__restrict__ tab,
-                        const float *__restrict__ ip_all, const float *__restrict__ im_all,
-                        float *__restrict__ op_all, float *__restrict__ om_all, double *__restrict__ slots) {
-    // per-warp FP64 tallies (tally q of warp w at w*WQ+q): 7 tallies, 9 with
-    // space charge; a power-of-two row keeps the index a shift
-    constexpr int WQ = SC ? 16 : 8, NQ = SC ? 9 : 7;
-    __shared__ double wacc[8 * WQ];
-    __shared__ BatchSim S;
-    __shared__ VecEntry E;
-    if (threadIdx.x == 0) {
-        E = tab[blockIdx.x];
-        S = sims[E.sim];
-    }
-    if (threadIdx.x < 8 * WQ) wacc[threadIdx.x] = 0.0;
-    __syncthreads();
-    const int nx = S.nx, ny = S.ny, nz = S.nz;
-    const Coef<float> &c = S.cf;
-    const float *in_[2] = {ip_all + S.off, im_all + S.off};
-    float *out_[2] = {op_all + S.off, om_all + S.off};
-    const int plane = nx * ny;
-    const int ncol4 = nx >> 2;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int ty = t / ncol4, c4 = t - (t / ncol4) * ncol4;
-    const bool valid = ty < E.rows;
-    const int yg = E.y0 + (valid ? ty : E.rows - 1);
-    const int x0 = 4 * c4;
-    const int row = yg * nx + x0;
-    const bool edge_u = yg == 0, edge_d = yg == ny - 1;
-    const int row_u = (edge_u ? ny - 1 : yg - 1) * nx + x0;
-    const int row_d = (edge_d ? 0 : yg + 1) * nx + x0;
-    const bool zero_u = !PERIODIC && edge_u, zero_d = !PERIODIC && edge_d;
-    const bool need_l = lane == 0 || c4 == 0, need_r = lane == 31 || c4 == ncol4 - 1;
-    const int row_l = yg * nx + (c4 == 0 ? nx - 1 : x0 - 1);
-    const int row_r = yg * nx + (c4 == ncol4 - 1 ? 0 : x0 + 4);
-    const bool zero_l = !PERIODIC && c4 == 0, zero_r = !PERIODIC && c4 == ncol4 - 1;
-    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    // warp-uniform: one FP32 partial per lane, reduced in FP64 (fixed order)
-    // into the warp's tally q
-    auto flush = [&](int q, float part) {
-        double v = (double)part;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) wacc[warp * WQ + q] += v;
-    };
-    float4 prev[2], cur[2], nxt[2];
-    for (int s = 0; s < 2; ++s) {
-        prev[s] = E.z0 > 0 ? ldg4(in_[s] + (E.z0 - 1) * plane + row) : zero4;
-        cur[s] = ldg4(in_[s] + E.z0 * plane + row);
-        nxt[s] = E.z0 + 1 < nz ? ldg4(in_[s] + (E.z0 + 1) * plane + row) : zero4;
-    }
-    float rsum = 0.f, lsum0 = 0.f, lsum1 = 0.f, ssum0 = 0.f, ssum1 = 0.f;
-    int nacc = 0;
-    for (int k = E.z0; k < E.z1; ++k) {
-        const int pk = k * plane;
-        float4 nn[2];   // two planes ahead: more loads in flight per thread
-#pragma unroll
-        for (int s = 0; s < 2; ++s) nn[s] = k + 2 < nz ? ldg4(in_[s] + pk + 2 * plane + row) : zero4;
-        const float2 rxy = __fmul2_rn(make_float2(cur[0].x, cur[0].y), make_float2(cur[1].x, cur[1].y));
-        const float2 rzw = __fmul2_rn(make_float2(cur[0].z, cur[0].w), make_float2(cur[1].z, cur[1].w));
-        float an[2] = {0.f, 0.f}, lat[2] = {0.f, 0.f};
-        float2 dxy, dzw;
-        if (SC) sc_diff4(cur[0], cur[1], dxy, dzw);
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            const float4 n = cur[s];
-            const float4 u = zero_u ? zero4 : ldg4(in_[s] + pk + row_u);
-            const float4 d = zero_d ? zero4 : ldg4(in_[s] + pk + row_d);
-            float l = __shfl_up_sync(0xffffffffu, n.w, 1);
-            float r = __shfl_down_sync(0xffffffffu, n.x, 1);
-            if (need_l) l = zero_l ? 0.f : __ldg(in_[s] + pk + row_l);
-            if (need_r) r = zero_r ? 0.f : __ldg(in_[s] + pk + row_r);
-            float4 v = upd7x4(n, l, r, u, d, prev[s], nxt[s], rxy, rzw, c.wx[s], c.wzm[s],
-                              c.wzp[s], c.adt);
-            if (SC) {
-                float2 pxy, pzw;
-                v = add_sc4(v, c.sc[s], n, dxy, dzw, pxy, pzw);
-                if (valid) (s ? ssum1 : ssum0) += (pxy.x + pxy.y) + (pzw.x + pzw.y);
-            }
-            if (valid) {
-                *reinterpret_cast<float4 *>(out_[s] + pk + row) = v;
-                if (k == 0 || k == nz - 1) an[s] += (n.x + n.y) + (n.z + n.w);
-                if (!PERIODIC) {
-                    if (c4 == 0) lat[s] += n.x;
-                    if (c4 == ncol4 - 1) lat[s] += n.w;
-                    if (edge_u) lat[s] += (n.x + n.y) + (n.z + n.w);
-                    if (edge_d) lat[s] += (n.x + n.y) + (n.z + n.w);
-                }
-            }
-            prev[s] = n;
-            cur[s] = nxt[s];
-            nxt[s] = nn[s];
-        }
-        if (valid) rsum += (rxy.x + rxy.y) + (rzw.x + rzw.y);
-        if (!PERIODIC) { lsum0 += lat[0]; lsum1 += lat[1]; }
-        // FP32 partials over at most 32 planes, then FP64
-        if (++nacc == 32) {
-            flush(0, rsum);
-            rsum = 0.f;
-            if (!PERIODIC) { flush(5, lsum0); flush(6, lsum1); lsum0 = lsum1 = 0.f; }
-            if (SC) { flush(7, ssum0); flush(8, ssum1); ssum0 = ssum1 = 0.f; }
-            nacc = 0;
-        }
-        if (k == 0) { flush(1, an[0]); flush(2, an[1]); }
-        if (k == nz - 1) { flush(3, an[0]); flush(4, an[1]); }
-    }
-    flush(0, rsum);
-    if (!PERIODIC) { flush(5, lsum0); flush(6, lsum1); }
-    if (SC) { flush(7, ssum0); flush(8, ssum1); }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double acc[NQ];
-        for (int q = 0; q < NQ; ++q) {
-            double v = 0.0;
-            for (int w = 0; w < 8; ++w) v += wacc[w * WQ + q];
-            acc[q] = v;
-        }
-        double *sl = slots + (size_t)blockIdx.x * NT;
-        sl[0] += acc[0] * c.rec_f;
-        sl[1] += acc[1] * c.anode_f[0];
-        sl[2] += acc[2] * c.anode_f[1];
-        sl[3] += acc[3] * c.cathode_f[0];
-        sl[4] += acc[4] * c.cathode_f[1];
-        // lateral faces: x and y weights are equal for dx = dy (latx_f == laty_f)
-        sl[5] += acc[5] * c.latx_f[0];
-        sl[6] += acc[6] * c.latx_f[1];
-        if (SC) {
-            sl[7] += acc[NQ - 2] * c.sc_f[0];
-            sl[8] += acc[NQ - 1] * c.sc_f[1];
-        }
-    }
-}
 
 // TMA-staged float4 z-march over the entries of simulations with nx % 4 == 0
 // and nx <= 256: the batched counterpart of the single-context step kernel.
@@ -552,48 +374,85 @@ step_batched_tma_kernel(const BatchSim *__restrict__ sims, const VecEntry *__res
 }
 
 // Fold the slots of each active simulation's entries (contiguous in the
-// table, in order) into its FP64 accumulators and clear them.  One block
-// per active simulation, one thread per tally.
-__global__ void batch_fold_kernel(const int *__restrict__ first, const int *__restrict__ count,
-                                  const int *__restrict__ sim_of, double *__restrict__ slots,
-                                  double *__restrict__ acc) {
-    const int a = blockIdx.x, q = threadIdx.x;
-    if (q >= NT) return;
-    double s = 0.0;
-    for (int e = first[a]; e < first[a] + count[a]; ++e) {
-        s += slots[(size_t)e * NT + q];
-        slots[(size_t)e * NT + q] = 0.0;
-    }
-    acc[(size_t)sim_of[a] * NT + q] += s;
+// table, in order) into its FP64 accumulators and clear them.  One block per
+// active simulation, one warp per tally.
+__global__ void __launch_bounds__(NT * 32)
+batch_fold_kernel(const int *__restrict__ first, const int *__restrict__ count, const int *__restrict__ sim_of,
+                  double *__restrict__ slots, double *__restrict__ acc) {
+    const int a = blockIdx.x, lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    double *sl = slots + (size_t)first[a] * NT;
+    const int n = count[a];
+    const double s = warp_strided_sum(sl, n, q, NT, lane);
+    for (int e = lane; e < n; e += 32) sl[(size_t)e * NT + q] = 0.0;
+    if (lane == 0) acc[(size_t)sim_of[a] * NT + q] += s;
 }
 
-// Per-entry sums of n+ and n- for the in-domain charge: FP32 partials over
-// at most 32 cells per thread, then FP64 (once per 32 cells, outside the
-// per-cell loop: FP64 arithmetic is slow on this GPU).
+// Per-entry sums of n+ and n- for the in-domain charge, and their largest
+// value for the dt ladder: FP32 partials over at most 32 cells per thread,
+// then FP64 (once per 32 cells, outside the per-cell loop: FP64 arithmetic is
+// slow on this GPU).
 __global__ void __launch_bounds__(256)
 batch_monitor_kernel(const BatchSim *__restrict__ sims, const BatchEntry *__restrict__ tab,
                      const float *__restrict__ ip_all, const float *__restrict__ im_all, double *__restrict__ mon) {
     __shared__ double red[32 * 2];
+    __shared__ float rmax[8];
     const BatchEntry E = tab[blockIdx.x];
     const long long off = sims[E.sim].off;
     const long long nxs = sims[E.sim].nx;
     double v[2] = {0.0, 0.0};
+    float mx = -INFINITY;
     const size_t end = (size_t)(E.end * nxs);
     size_t idx = (size_t)(E.begin * nxs) + threadIdx.x;
     while (idx < end) {
         float a = 0.f, b = 0.f;
         for (int j = 0; j < 32 && idx < end; ++j, idx += blockDim.x) {
-            a += ip_all[off + idx];
-            b += im_all[off + idx];
+            const float p = ip_all[off + idx], m = im_all[off + idx];
+            a += p;
+            b += m;
+            mx = fmaxf(mx, fmaxf(p, m));
         }
         v[0] += (double)a;
         v[1] += (double)b;
     }
-    block_sum<2>(v, red);
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_down_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0) rmax[threadIdx.x >> 5] = mx;
+    block_sum<2>(v, red);   // contains the __syncthreads for rmax too
     if (threadIdx.x == 0) {
-        mon[2 * blockIdx.x] = v[0];
-        mon[2 * blockIdx.x + 1] = v[1];
+        for (int w = 1; w < 8; ++w) mx = fmaxf(mx, rmax[w]);
+        mon[3 * blockIdx.x] = v[0];
+        mon[3 * blockIdx.x + 1] = v[1];
+        mon[3 * blockIdx.x + 2] = (double)mx;
     }
+}
+
+// One simulation's results in one place: out[0 .. NT) tallies, two released
+// charges, two in-domain sums, two smallest and two largest densities.  One
+// warp per value.
+constexpr int TAL_BLOCKS = 64, TAL_OUT = NT + 8;
+__global__ void __launch_bounds__(TAL_OUT * 32)
+batch_tally_kernel(const double *__restrict__ acc, const double *__restrict__ rel, const double *__restrict__ mon,
+                   double *__restrict__ out) {
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    double v = 0.0;
+    if (q < NT) {
+        v = acc[q];
+    } else if (q < NT + 2) {
+        v = rel[q - NT];
+    } else if (q < NT + 4) {
+        v = warp_strided_sum(mon, TAL_BLOCKS, q - NT - 2, NM, lane);
+    } else {
+        const int e = q - NT - 2;   // 2, 3 smallest, 4, 5 largest
+        v = e < 4 ? INFINITY : -INFINITY;
+        for (int m = lane; m < TAL_BLOCKS; m += 32) {
+            const double x = mon[(size_t)m * NM + e];
+            v = e < 4 ? fmin(v, x) : fmax(v, x);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const double x = __shfl_down_sync(0xffffffffu, v, o);
+            v = e < 4 ? fmin(v, x) : fmax(v, x);
+        }
+    }
+    if (lane == 0) out[q] = v;
 }
 
 // Per-entry maximum of n+ and n-.
@@ -616,6 +475,12 @@ batch_max_kernel(const BatchSim *__restrict__ sims, const BatchEntry *__restrict
     }
 }
 
+// Launch shape of a step for the simulations with nx % 4 == 0.
+struct BatchShape {
+    int tma;   // 2 / 1: TMA-staged kernel with two / one float4 per thread; 0: direct march
+    int cps;   // TMA: CTAs per SM its z splits aim for; direct: divisor of the fitted chunk length
+};
+
 }  // namespace itk
 
 using namespace itk;
@@ -637,17 +502,24 @@ struct it_batch {
     std::vector<BatchEntry> tab;      // row ranges of every active simulation (monitors)
     std::vector<int> mfirst, mcount;  // per active simulation, into tab
     std::vector<int> morder;          // the active simulation of each mfirst/mcount entry
-    std::vector<VecEntry> vtab;       // step entries of the float4 kernel
-    std::vector<BatchEntry> stab;     // step entries of the scalar kernel
+    std::vector<VecEntry> vtab;       // step entries of the TMA-staged kernel
+    std::vector<MarchEntry> dtab;     // of the direct march (float4 segments)
+    std::vector<MarchEntry> stab;     // of the march over single cells (nx % 4 != 0)
     std::vector<int> first, count, sim_of;   // per active simulation, into the step slots
-    BatchEntry *d_tab, *d_stab;
+    BatchEntry *d_tab;
     VecEntry *d_vtab;
+    MarchEntry *d_dtab, *d_stab;
     int *d_first, *d_count, *d_simof;
     double *d_slots, *d_mon;
-    float *d_max;                     // per-entry peak density (the dt ladder)
-    size_t tab_cap, stab_cap, vtab_cap, slot_cap, act_cap, max_cap;
-    long long chunk;                  // cells per entry
-    int vec_cps;                      // CTAs per SM the float4 launch aims for (sets its z split)
+    std::vector<double> nmax;         // per simulation: largest density at the last check
+    size_t tab_cap, stab_cap, dtab_cap, vtab_cap, slot_cap, act_cap;
+    long long chunk;                  // cells per entry (monitors, single-cell march)
+    BatchShape shape;                 // launch shape of the current table
+    bool tuned;                       // the autotuner's choice, for the simulations it was made for
+    BatchShape tuned_shape;
+    int tuned_active;
+    double cal[3];                    // measured over fitted time of the direct march and the TMA kernels
+    double *d_tal;                    // one simulation's monitor blocks, then its gathered tallies
     // per simulation
     std::vector<int64_t> steps;
     std::vector<double> t_s;          // simulated time: the sum of every step's dt
@@ -667,14 +539,10 @@ struct it_batch {
     int64_t track_cap;
     int max_nx, max_ny;
     // TMA-staged float4 kernel: per simulation [set][species][main, halo]
-    // tensor maps (zero for simulations it does not take), its use, the
-    // number of leading float4 entries it runs, and the device error flag of
-    // its bounded waits
+    // tensor maps (zero for simulations it does not take) and the device error
+    // flag of its bounded waits
     CUtensorMap *d_maps;
     std::vector<char> tma_ok;
-    int use_tma;
-    int tma_ipt;                      // float4 per thread of the TMA kernel (1 or 2)
-    int nvt;
     int *d_err;
 };
 
@@ -685,39 +553,148 @@ int bfail(int code, const std::string &m) {
     return code;
 }
 
-// Rebuild the work tables for the active simulations.  Step entries: the
-// float4 kernel takes simulations with nx % 4 == 0 (tiles of 256/(nx/4)
-// rows, split in z when few cells are active), the scalar kernel the rest.
-// All entries of one simulation are contiguous, so the fold is in order.
-int build_table(it_batch *b) {
-    b->tab.clear(); b->mfirst.clear(); b->mcount.clear(); b->morder.clear();
-    b->vtab.clear(); b->stab.clear();
-    b->first.clear(); b->count.clear(); b->sim_of.clear();
-    long long active_cells = 0, vec_tiles = 0;
-    for (int s = 0; s < b->nsim; ++s) {
-        if (!b->active[s]) continue;
-        const BatchSim &h = b->hs[s];
-        active_cells += (long long)h.nx * h.ny * h.nz;
-        if (h.nx % 4 == 0 && h.nx <= 1024) {
-            const int rows = std::max(1, 256 / (h.nx / 4));
-            vec_tiles += (h.ny + rows - 1) / rows;
-        }
-    }
+int sm_count() {
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
+int tma_rows(const BatchSim &h, int ipt) { return std::max(1, std::min(256 * ipt / (h.nx / 4), 256)); }
+long long march_blocks(const BatchSim &h, int v) {
+    return ((long long)(h.nx / v) * h.ny + SK_THREADS - 1) / SK_THREADS;
+}
+
+// z splits of the TMA entries: about cps CTAs per SM, at least eight planes each
+int tma_split(const it_batch *b, const BatchShape &sh, int sms) {
+    long long tiles = 0;
+    for (int s = 0; s < b->nsim; ++s)
+        if (b->active[s] && b->tma_ok[s]) {
+            const int rows = tma_rows(b->hs[s], sh.tma);
+            tiles += (b->hs[s].ny + rows - 1) / rows;
+        }
+    return tiles > 0 ? (int)std::max(1LL, ((long long)sh.cps * sms + tiles - 1) / tiles) : 1;
+}
+
+// Planes per entry of the direct march and its fitted time in us: the blocks
+// resident at a time walk their planes in 650 cycles plus 190 per block they
+// share the SM with (the single-grid march's figures), an entry starting with
+// two planes of loads; a state beyond L2 moves 1.42 times slower than a copy.
+int direct_chunk(const it_batch *b, int sms, double *us) {
+    const double resident = (double)sms * DK_BLOCKS;
+    int best = 1;
+    double best_cost = 1e300, bytes = 0.0;
+    for (int kc : {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 48, 64, 96, 128, 256, 512}) {
+        double entries = 0.0, work = 0.0;
+        int longest = 0;
+        bytes = 0.0;
+        for (int s = 0; s < b->nsim; ++s) {
+            const BatchSim &h = b->hs[s];
+            if (!b->active[s] || h.nx % 4 != 0) continue;
+            const int c = (h.nz + kc - 1) / kc;
+            const double nb = (double)march_blocks(h, 4);
+            entries += nb * c;
+            work += nb * (h.nz + 2.0 * c);
+            longest = std::max(longest, (h.nz + c - 1) / c);
+            bytes += 16.0 * h.nx * h.ny * h.nz;
+        }
+        const double full = DK_LAT + DK_THR * DK_BLOCKS;
+        const double cost = entries <= resident
+                                ? (longest + 2.0) * (DK_LAT + DK_THR * std::ceil(entries / sms))
+                                : work / resident * full + 0.5 * (longest + 2.0) * full;
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = kc;
+        }
+    }
+    *us = std::max(best_cost / 1900.0 + 1.5, bytes > 100e6 ? 1.42 * bytes / 6.8e6 : 0.0);
+    return best;
+}
+
+// Fitted time of a step of the active simulations in us, TMA-staged: a plane's
+// round takes 1.5 us with two float4 per thread and two CTAs per SM, 1.32 with
+// one and three, the last entries leave the chip a fifth of the longest one
+// idle, and starting takes about 6 us (256 uneven simulations of the batched
+// workload at one, two, three and six z splits: 614, 576, 579 and 602 us,
+// fitted 610, 590, 589 and 605).
+double tma_us(const it_batch *b, const BatchShape &sh, int sms) {
+    const int split = tma_split(b, sh, sms);
+    const double round = sh.tma == 2 ? 1.5 : 1.32;
+    double rounds = 0.0;
+    int longest = 0;
+    for (int s = 0; s < b->nsim; ++s) {
+        const BatchSim &h = b->hs[s];
+        if (!b->active[s] || !b->tma_ok[s]) continue;
+        const int rows = tma_rows(h, sh.tma), zc = std::min(split, std::max(1, h.nz / 8));
+        rounds += (double)((h.ny + rows - 1) / rows) * (h.nz + 2.0 * zc);
+        longest = std::max(longest, (h.nz + zc - 1) / zc);
+    }
+    return rounds * round / ((sh.tma == 2 ? 2.0 : 3.0) * sms) + 0.2 * (longest + 2) * round + 6.0;
+}
+
+double shape_us(const it_batch *b, const BatchShape &sh, int sms) {
+    double us = 0.0;
+    if (sh.tma == 0) (void)direct_chunk(b, sms, &us);
+    else us = tma_us(b, sh, sms);
+    return us;
+}
+
+// The launch shape for the simulations now active: the autotuner's while they
+// are the ones it timed, else the least fitted time, scaled by what the
+// autotuner measured against the fit (batches shrink as simulations finish,
+// and small ones are faster without the ring).
+BatchShape choose_shape(const it_batch *b, int sms) {
+    int active = 0;
+    bool any_tma = false;
+    for (int s = 0; s < b->nsim; ++s)
+        if (b->active[s]) {
+            ++active;
+            any_tma = any_tma || b->tma_ok[s];
+        }
+    if (b->tuned && active == b->tuned_active) return b->tuned_shape;
+    BatchShape best{0, 1};
+    double best_us = shape_us(b, best, sms) * b->cal[0];
+    if (any_tma)
+        for (int tma : {2, 1})
+            for (int cps : {1, 2, 4, 8, 16, 32}) {
+                const BatchShape sh{tma, cps};
+                const double us = tma_us(b, sh, sms) * b->cal[tma];
+                if (us < best_us) {
+                    best_us = us;
+                    best = sh;
+                }
+            }
+    return best;
+}
+
+// Rebuild the work tables for the active simulations in launch shape b->shape.
+// All step entries of one simulation are contiguous, so the fold is in order.
+int build_table(it_batch *b) {
+    b->tab.clear(); b->mfirst.clear(); b->mcount.clear(); b->morder.clear();
+    b->vtab.clear(); b->dtab.clear(); b->stab.clear();
+    b->first.clear(); b->count.clear(); b->sim_of.clear();
+    long long active_cells = 0;
+    for (int s = 0; s < b->nsim; ++s)
+        if (b->active[s]) active_cells += (long long)b->hs[s].nx * b->hs[s].ny * b->hs[s].nz;
+    const int sms = sm_count();
     const long long chunk = std::max(1024LL, std::min(b->chunk, active_cells / (4LL * sms)));
-    // z splits so that the float4 launch keeps about vec_cps CTAs per SM busy
-    const long long zsplit =
-        vec_tiles > 0 ? std::max(1LL, ((long long)b->vec_cps * sms + vec_tiles - 1) / vec_tiles) : 1;
-    std::vector<int> vfirst, vcount, sfirst, scount, vsim, ssim;
-    // float4 entries of the simulations the TMA kernel takes come first
-    b->nvt = 0;
-    std::vector<int> order;
-    for (int pass = 0; pass < 2; ++pass)
-        for (int s = 0; s < b->nsim; ++s)
-            if (b->active[s] && ((b->use_tma && b->tma_ok[s]) == (pass == 0))) order.push_back(s);
-    for (int s : order) {
+    const BatchShape sh = b->shape;
+    const int split = sh.tma ? tma_split(b, sh, sms) : 1;
+    double us = 0.0;
+    const int kc4 = std::max(1, direct_chunk(b, sms, &us) / (sh.tma ? 1 : sh.cps));
+    const int kc1 = (int)std::max(1LL, chunk / SK_THREADS);
+    std::vector<int> part[3], pfirst[3], pcount[3];   // simulations on the TMA, direct and single-cell kernels
+    auto march = [&](std::vector<MarchEntry> &tab, int s, int v, int kc) {
+        const BatchSim &h = b->hs[s];
+        const int c = (h.nz + kc - 1) / kc;
+        const long long nb = march_blocks(h, v);
+        for (int q = 0; q < c; ++q)
+            for (long long p = 0; p < nb; ++p)
+                tab.push_back(MarchEntry{s, (unsigned)(p * SK_THREADS), (int)((long long)h.nz * q / c),
+                                         (int)((long long)h.nz * (q + 1) / c)});
+    };
+    for (int s = 0; s < b->nsim; ++s) {
+        if (!b->active[s]) continue;
         const BatchSim &h = b->hs[s];
         const long long rows = (long long)h.ny * h.nz;
         const long long rpe = std::max(1LL, chunk / h.nx);
@@ -726,35 +703,36 @@ int build_table(it_batch *b) {
         for (long long r0 = 0; r0 < rows; r0 += rpe, ++n) b->tab.push_back(BatchEntry{s, 0, r0, std::min(rows, r0 + rpe)});
         b->mcount.push_back(n);
         b->morder.push_back(s);
-        if (h.nx % 4 == 0 && h.nx <= 1024) {
-            // rows per entry: a 256-thread tile of float4 (times the TMA
-            // kernel's float4 per thread for the simulations it takes)
-            const int ipt = (b->use_tma && b->tma_ok[s]) ? b->tma_ipt : 1;
-            const int rpt = std::max(1, std::min(256 * ipt / (h.nx / 4), 256));
-            const int zc = (int)std::min<long long>(zsplit, std::max(1, h.nz / 8));
-            vsim.push_back(s);
-            vfirst.push_back((int)b->vtab.size());
-            int m = 0;
+        const int on = h.nx % 4 != 0 ? 2 : sh.tma && b->tma_ok[s] ? 0 : 1;
+        const size_t before = on == 0 ? b->vtab.size() : on == 1 ? b->dtab.size() : b->stab.size();
+        if (on == 0) {
+            // rows per entry: a 256-thread tile of float4 times those per thread
+            const int rpt = tma_rows(h, sh.tma);
+            const int zc = std::min(split, std::max(1, h.nz / 8));
             for (int y0 = 0; y0 < h.ny; y0 += rpt)
-                for (int q = 0; q < zc; ++q, ++m)
+                for (int q = 0; q < zc; ++q)
                     b->vtab.push_back(VecEntry{s, y0, std::min(rpt, h.ny - y0), (int)((long long)h.nz * q / zc),
                                                (int)((long long)h.nz * (q + 1) / zc), 0});
-            vcount.push_back(m);
-            if (b->use_tma && b->tma_ok[s]) b->nvt += m;
+        } else if (on == 1) {
+            march(b->dtab, s, 4, kc4);
         } else {
-            ssim.push_back(s);
-            sfirst.push_back((int)b->stab.size());
-            int m = 0;
-            for (long long r0 = 0; r0 < rows; r0 += rpe, ++m) b->stab.push_back(BatchEntry{s, 0, r0, std::min(rows, r0 + rpe)});
-            scount.push_back(m);
+            march(b->stab, s, 1, kc1);
         }
+        const size_t after = on == 0 ? b->vtab.size() : on == 1 ? b->dtab.size() : b->stab.size();
+        part[on].push_back(s);
+        pfirst[on].push_back((int)before);
+        pcount[on].push_back((int)(after - before));
     }
-    // step slots: [float4 entries][scalar entries]
-    const int nv = (int)b->vtab.size();
-    for (size_t q = 0; q < vsim.size(); ++q) { b->sim_of.push_back(vsim[q]); b->first.push_back(vfirst[q]); b->count.push_back(vcount[q]); }
-    for (size_t q = 0; q < ssim.size(); ++q) { b->sim_of.push_back(ssim[q]); b->first.push_back(nv + sfirst[q]); b->count.push_back(scount[q]); }
-    const size_t ne = b->tab.size(), nvs = b->vtab.size(), nss = b->stab.size(), na = b->sim_of.size();
-    const size_t nslot = nvs + nss;
+    // step slots: [TMA entries][direct entries][single-cell entries]
+    const int base[3] = {0, (int)b->vtab.size(), (int)(b->vtab.size() + b->dtab.size())};
+    for (int on = 0; on < 3; ++on)
+        for (size_t q = 0; q < part[on].size(); ++q) {
+            b->sim_of.push_back(part[on][q]);
+            b->first.push_back(base[on] + pfirst[on][q]);
+            b->count.push_back(pcount[on][q]);
+        }
+    const size_t ne = b->tab.size(), nvs = b->vtab.size(), nds = b->dtab.size(), nss = b->stab.size(), na = b->sim_of.size();
+    const size_t nslot = nvs + nds + nss;
     auto grow = [&](void **p, size_t &cap, size_t need, size_t esz) -> cudaError_t {
         if (need <= cap) return cudaSuccess;
         cudaFree(*p);
@@ -769,10 +747,11 @@ int build_table(it_batch *b) {
     if (b->tab_cap != mon_cap || !b->d_mon) {
         cudaFree(b->d_mon);
         b->d_mon = nullptr;
-        IT_CK(cudaMalloc(&b->d_mon, sizeof(double) * 2 * std::max<size_t>(b->tab_cap, 1)));
+        IT_CK(cudaMalloc(&b->d_mon, sizeof(double) * 3 * std::max<size_t>(b->tab_cap, 1)));
     }
     IT_CK(grow((void **)&b->d_vtab, b->vtab_cap, nvs, sizeof(VecEntry)));
-    IT_CK(grow((void **)&b->d_stab, b->stab_cap, nss, sizeof(BatchEntry)));
+    IT_CK(grow((void **)&b->d_dtab, b->dtab_cap, nds, sizeof(MarchEntry)));
+    IT_CK(grow((void **)&b->d_stab, b->stab_cap, nss, sizeof(MarchEntry)));
     IT_CK(grow((void **)&b->d_slots, b->slot_cap, nslot, sizeof(double) * NT));
     if (na > b->act_cap) {
         cudaFree(b->d_first); cudaFree(b->d_count); cudaFree(b->d_simof);
@@ -783,7 +762,8 @@ int build_table(it_batch *b) {
     }
     if (ne) IT_CK(cudaMemcpyAsync(b->d_tab, b->tab.data(), sizeof(BatchEntry) * ne, cudaMemcpyHostToDevice, b->stream));
     if (nvs) IT_CK(cudaMemcpyAsync(b->d_vtab, b->vtab.data(), sizeof(VecEntry) * nvs, cudaMemcpyHostToDevice, b->stream));
-    if (nss) IT_CK(cudaMemcpyAsync(b->d_stab, b->stab.data(), sizeof(BatchEntry) * nss, cudaMemcpyHostToDevice, b->stream));
+    if (nds) IT_CK(cudaMemcpyAsync(b->d_dtab, b->dtab.data(), sizeof(MarchEntry) * nds, cudaMemcpyHostToDevice, b->stream));
+    if (nss) IT_CK(cudaMemcpyAsync(b->d_stab, b->stab.data(), sizeof(MarchEntry) * nss, cudaMemcpyHostToDevice, b->stream));
     if (nslot) IT_CK(cudaMemsetAsync(b->d_slots, 0, sizeof(double) * NT * nslot, b->stream));
     if (na) {
         IT_CK(cudaMemcpyAsync(b->d_first, b->first.data(), sizeof(int) * na, cudaMemcpyHostToDevice, b->stream));
@@ -796,14 +776,20 @@ int build_table(it_batch *b) {
     return IT_OK;
 }
 
+// the tables in the launch shape chosen for the active simulations
+int rebuild(it_batch *b) {
+    b->shape = choose_shape(b, sm_count());
+    return build_table(b);
+}
+
 int launch_batched_step(it_batch *b, int parity) {
-    const int nv = (int)b->vtab.size(), ns = (int)b->stab.size(), nt = b->nvt;
+    const int nt = (int)b->vtab.size(), nd = (int)b->dtab.size(), ns = (int)b->stab.size();
     const float *ip = b->state[parity][0], *im = b->state[parity][1];
     float *op = b->state[parity ^ 1][0], *om = b->state[parity ^ 1][1];
     const bool per = b->p.lateral_bc == IT_PERIODIC;
     const bool sc = b->p.space_charge != 0;
     if (nt) {
-        const bool two = b->tma_ipt == 2;
+        const bool two = b->shape.tma == 2;
         auto *kt = two ? (per ? (sc ? step_batched_tma_kernel<true, true, 2> : step_batched_tma_kernel<true, false, 2>)
                               : (sc ? step_batched_tma_kernel<false, true, 2> : step_batched_tma_kernel<false, false, 2>))
                        : (per ? (sc ? step_batched_tma_kernel<true, true, 1> : step_batched_tma_kernel<true, false, 1>)
@@ -813,17 +799,16 @@ int launch_batched_step(it_batch *b, int parity) {
                                                                        two ? kBtSmemFloats2 : kBtSmemFloats, b->d_err);
         IT_CK(cudaGetLastError());
     }
-    if (nv > nt) {
-        auto *kv = per ? (sc ? step_batched_vec_kernel<true, true> : step_batched_vec_kernel<true, false>)
-                       : (sc ? step_batched_vec_kernel<false, true> : step_batched_vec_kernel<false, false>);
-        kv<<<nv - nt, 256, 0, b->stream>>>(b->d_sims, b->d_vtab + nt, ip, im, op, om, b->d_slots + (size_t)NT * nt);
+    if (nd) {
+        auto *kd = per ? (sc ? step_batched_march_kernel<true, true, 4> : step_batched_march_kernel<true, false, 4>)
+                       : (sc ? step_batched_march_kernel<false, true, 4> : step_batched_march_kernel<false, false, 4>);
+        kd<<<nd, SK_THREADS, 0, b->stream>>>(b->d_sims, b->d_dtab, ip, im, op, om, b->d_slots + (size_t)NT * nt);
         IT_CK(cudaGetLastError());
     }
     if (ns) {
-        double *sl = b->d_slots + (size_t)NT * nv;
-        auto *ks = per ? (sc ? step_batched_kernel<true, true> : step_batched_kernel<true, false>)
-                       : (sc ? step_batched_kernel<false, true> : step_batched_kernel<false, false>);
-        ks<<<ns, 256, 0, b->stream>>>(b->d_sims, b->d_stab, ip, im, op, om, sl);
+        auto *ks = per ? (sc ? step_batched_march_kernel<true, true, 1> : step_batched_march_kernel<true, false, 1>)
+                       : (sc ? step_batched_march_kernel<false, true, 1> : step_batched_march_kernel<false, false, 1>);
+        ks<<<ns, SK_THREADS, 0, b->stream>>>(b->d_sims, b->d_stab, ip, im, op, om, b->d_slots + (size_t)NT * (nt + nd));
         IT_CK(cudaGetLastError());
     }
     return IT_OK;
@@ -858,30 +843,13 @@ int run_segment(it_batch *b, int K) {
 }
 
 // The doubling ladder of it_run_to_completion, per active simulation with no
-// pulse still to come: one pass for the peak density of every table entry,
-// then each simulation's dt rises to its largest admissible rung.  The step
-// graph reads the descriptors from device memory, so only they change.
+// pulse still to come: its dt rises to the largest rung admissible at the
+// peak density the check has just measured.  The step graph reads the
+// descriptors from device memory, so only they change.
 static int ladder_batch(it_batch *b) {
-    const int ne = (int)b->tab.size();
-    if (!ne) return IT_OK;
-    if ((size_t)ne > b->max_cap) {
-        cudaFree(b->d_max);
-        b->d_max = nullptr;
-        b->max_cap = 0;
-        IT_CK(cudaMalloc(&b->d_max, sizeof(float) * ne));
-        b->max_cap = ne;
-    }
-    const int parity = (int)(b->bstep & 1);
-    batch_max_kernel<<<ne, 256, 0, b->stream>>>(b->d_sims, b->d_tab, b->state[parity][0], b->state[parity][1],
-                                                b->d_max);
-    IT_CK(cudaGetLastError());
-    std::vector<float> mx(ne);
-    IT_CK(cudaMemcpyAsync(mx.data(), b->d_max, sizeof(float) * ne, cudaMemcpyDeviceToHost, b->stream));
-    IT_CK(cudaStreamSynchronize(b->stream));
     for (size_t a = 0; a < b->morder.size(); ++a) {
         const int s = b->morder[a];
-        double nmax = -INFINITY;
-        for (int q = b->mfirst[a]; q < b->mfirst[a] + b->mcount[a]; ++q) nmax = std::max(nmax, (double)mx[q]);
+        const double nmax = b->nmax[s];
         // as in a single context, whose check runs before the deposits of its
         // step: a check at the step of the last pulse still counts that pulse
         // as to come
@@ -907,12 +875,12 @@ static int ladder_batch(it_batch *b) {
 int fold(it_batch *b) {
     const int na = (int)b->sim_of.size();
     if (!na) return IT_OK;
-    batch_fold_kernel<<<na, 32, 0, b->stream>>>(b->d_first, b->d_count, b->d_simof, b->d_slots, b->d_acc);
+    batch_fold_kernel<<<na, NT * 32, 0, b->stream>>>(b->d_first, b->d_count, b->d_simof, b->d_slots, b->d_acc);
     IT_CK(cudaGetLastError());
     return IT_OK;
 }
 
-// in-domain ions of every simulation in the current table
+// in-domain ions of every simulation in the current table, and its largest density
 int in_domain(it_batch *b, std::vector<double> &ind2) {
     ind2.assign(2 * (size_t)b->nsim, 0.0);
     const int ne = (int)b->tab.size();
@@ -921,17 +889,22 @@ int in_domain(it_batch *b, std::vector<double> &ind2) {
     batch_monitor_kernel<<<ne, 256, 0, b->stream>>>(b->d_sims, b->d_tab, b->state[parity][0], b->state[parity][1],
                                                     b->d_mon);
     IT_CK(cudaGetLastError());
-    std::vector<double> mon(2 * (size_t)ne);
+    std::vector<double> mon(3 * (size_t)ne);
     int err = 0;
-    IT_CK(cudaMemcpyAsync(mon.data(), b->d_mon, sizeof(double) * 2 * ne, cudaMemcpyDeviceToHost, b->stream));
+    IT_CK(cudaMemcpyAsync(mon.data(), b->d_mon, sizeof(double) * 3 * ne, cudaMemcpyDeviceToHost, b->stream));
     IT_CK(cudaMemcpyAsync(&err, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
     IT_CK(cudaStreamSynchronize(b->stream));
     if (err) return bfail(IT_ETIMEOUT, "a bounded device wait ran out in the batched step kernel");
     for (size_t a = 0; a < b->morder.size(); ++a) {
         const int s = b->morder[a];
         const double vol = b->dx[s] * b->dx[s] * b->dx[s];
-        double p = 0, m = 0;
-        for (int e = b->mfirst[a]; e < b->mfirst[a] + b->mcount[a]; ++e) { p += mon[2 * e]; m += mon[2 * e + 1]; }
+        double p = 0, m = 0, mx = -INFINITY;
+        for (int e = b->mfirst[a]; e < b->mfirst[a] + b->mcount[a]; ++e) {
+            p += mon[3 * e];
+            m += mon[3 * e + 1];
+            mx = std::max(mx, mon[3 * e + 2]);
+        }
+        b->nmax[s] = mx;
         ind2[2 * s] = p * vol;
         ind2[2 * s + 1] = m * vol;
     }
@@ -944,8 +917,8 @@ void batch_free(it_batch *b) {
     if (b->graph) cudaGraphExecDestroy(b->graph);
     cudaFree(b->state_base);
     cudaFree(b->d_sims); cudaFree(b->d_acc); cudaFree(b->d_rel);
-    cudaFree(b->d_tab); cudaFree(b->d_slots); cudaFree(b->d_mon); cudaFree(b->d_max);
-    cudaFree(b->d_vtab); cudaFree(b->d_stab);
+    cudaFree(b->d_tab); cudaFree(b->d_slots); cudaFree(b->d_mon); cudaFree(b->d_tal);
+    cudaFree(b->d_vtab); cudaFree(b->d_dtab); cudaFree(b->d_stab);
     cudaFree(b->d_first); cudaFree(b->d_count); cudaFree(b->d_simof);
     cudaFree(b->d_plane); cudaFree(b->d_tracks); cudaFree(b->d_wx); cudaFree(b->d_wy);
     cudaFree(b->d_maps); cudaFree(b->d_err);
@@ -980,7 +953,8 @@ int it_batch_create(int32_t nsim, const it_sim_desc *descs, const it_params *com
     b->pulse_done.assign(nsim, 0);
     b->pulse_period.assign(nsim, 0);
     b->chunk = 16384;
-    b->vec_cps = 4;
+    b->cal[0] = b->cal[1] = b->cal[2] = 1.0;
+    b->nmax.assign(nsim, 0.0);
     b->graph_parity = -1;
     size_t off = 0;
     for (int s = 0; s < nsim; ++s) {
@@ -1031,6 +1005,7 @@ int it_batch_create(int32_t nsim, const it_sim_desc *descs, const it_params *com
     if ((e = cudaMalloc(&b->d_sims, sizeof(BatchSim) * nsim)) != cudaSuccess ||
         (e = cudaMalloc(&b->d_acc, sizeof(double) * NT * nsim)) != cudaSuccess ||
         (e = cudaMalloc(&b->d_rel, sizeof(double) * 8 * nsim)) != cudaSuccess ||
+        (e = cudaMalloc(&b->d_tal, sizeof(double) * (NM * TAL_BLOCKS + TAL_OUT))) != cudaSuccess ||
         (e = cudaMalloc(&b->d_plane, sizeof(double) * 2 * b->max_nx * b->max_ny)) != cudaSuccess)   // plane + tile sums
         return bail(e, "batch scratch");
     if ((e = cudaMemcpyAsync(b->d_sims, b->hs.data(), sizeof(BatchSim) * nsim, cudaMemcpyHostToDevice, b->stream)) != cudaSuccess ||
@@ -1043,8 +1018,6 @@ int it_batch_create(int32_t nsim, const it_sim_desc *descs, const it_params *com
     // and min(512 / (nx/4), ny) rows (one or two float4 per thread) and a
     // box of one halo row
     b->tma_ok.assign(nsim, 0);
-    b->use_tma = 1;
-    b->tma_ipt = 1;
     {
         std::vector<CUtensorMap> maps((size_t)nsim * BT_MAPS);
         std::memset(maps.data(), 0, sizeof(CUtensorMap) * maps.size());
@@ -1128,11 +1101,9 @@ int deposit_sim(it_batch *b, int sim, const double *packed, int64_t n) {
     cudaError_t e = cudaMemcpyAsync(b->d_tracks, packed, sizeof(double) * 4 * n, cudaMemcpyHostToDevice, b->stream);
     if (e != cudaSuccess) rc = cuda_fail(e, "track upload");
     v->d_tracks = b->d_tracks; v->d_wx = b->d_wx; v->d_wy = b->d_wy;
+    // packed is pageable: it has been staged when the copy returns, so nothing
+    // is waited for and the next simulation's deposit is prepared meanwhile
     if (rc == IT_OK) rc = launch_deposit(v, n, b->stream);
-    if (rc == IT_OK) {
-        e = cudaStreamSynchronize(b->stream);   // packed host memory may be freed after return
-        if (e != cudaSuccess) rc = cuda_fail(e, "deposit");
-    }
     delete v;
     return rc;
 }
@@ -1177,7 +1148,7 @@ int it_batch_retime(it_batch *b) {
     if (!b) return bfail(IT_EINVAL, "batch is NULL");
     if (b->bstep != 0) return bfail(IT_ESTATE, "the time steps can only change before the first step");
     for (int s = 0; s < b->nsim; ++s) b->active[s] = 1;
-    int rc = build_table(b);
+    int rc = rebuild(b);
     if (rc) return rc;
     const int ne = (int)b->tab.size();
     float *d_mx = nullptr;
@@ -1237,60 +1208,93 @@ int it_batch_autotune(it_batch *b, int32_t trial_steps, double *best_us) {
         cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         rc = cuda_fail(cudaGetLastError(), "batch autotune set-up");
     const long long chunk0 = b->chunk;
-    // TMA choice: 2 = the TMA kernel with two float4 per thread, 1 = with
-    // one, 0 = the register kernel
-    const int cps0 = b->vec_cps, tma0 = b->use_tma ? b->tma_ipt : 0;
-    long long best_chunk = chunk0;
-    int best_cps = cps0, best_tma = tma0;
-    double best = 1e300;
-    // the entry size only shapes the scalar kernel's entries: with no
-    // simulation on that kernel a single size is timed
-    bool any_scalar = false;
+    // the entry size only shapes the single-cell march's entries: with no
+    // simulation on it a single size is timed
+    bool any_cells = false, any_tma = false;
+    int active = 0;
     for (int s = 0; s < b->nsim; ++s)
-        if (b->active[s] && !(b->hs[s].nx % 4 == 0 && b->hs[s].nx <= 1024)) any_scalar = true;
-    const std::vector<long long> chunks = any_scalar ? std::vector<long long>{4096LL, 16384LL, 65536LL}
-                                                     : std::vector<long long>{chunk0};
-    for (int tma : {2, 1, 0})
-    for (int cps : {1, 2, 4, 8, 16, 32}) {
+        if (b->active[s]) {
+            ++active;
+            any_cells = any_cells || b->hs[s].nx % 4 != 0;
+            any_tma = any_tma || b->tma_ok[s];
+        }
+    const std::vector<long long> chunks = any_cells ? std::vector<long long>{4096LL, 16384LL, 65536LL}
+                                                    : std::vector<long long>{chunk0};
+    // candidates: the TMA kernels with z splits aiming at 1..32 CTAs per SM,
+    // each distinct split once; the direct march with the fitted chunk of
+    // planes and half of it
+    const int sms = sm_count();
+    std::vector<BatchShape> shapes;
+    if (any_tma)
+        for (int tma : {2, 1}) {
+            int seen = 0;
+            for (int cps : {1, 2, 4, 8, 16, 32}) {
+                const BatchShape sh{tma, cps};
+                const int split = tma_split(b, sh, sms);
+                if (split != seen) shapes.push_back(sh);
+                seen = split;
+            }
+        }
+    shapes.push_back({0, 1});
+    shapes.push_back({0, 2});
+    long long best_chunk = chunk0;
+    BatchShape best_shape = b->shape;
+    double best = 1e300, kind_us[3] = {1e300, 1e300, 1e300}, kind_fit[3] = {0.0, 0.0, 0.0};
+    for (const BatchShape &sh : shapes)
         for (long long chunk : chunks) {
             if (rc) break;
-            b->use_tma = tma > 0;
-            b->tma_ipt = tma == 2 ? 2 : 1;
-            b->vec_cps = cps;
+            b->shape = sh;
             b->chunk = chunk;
             rc = build_table(b);
-            for (int q = 0; q < 2 && !rc; ++q) rc = launch_batched_step(b, q & 1);
-            if (!rc && cudaEventRecord(e0, b->stream) != cudaSuccess) rc = cuda_fail(cudaGetLastError(), "event");
-            for (int q = 0; q < K && !rc; ++q) rc = launch_batched_step(b, q & 1);
-            if (!rc && cudaEventRecord(e1, b->stream) != cudaSuccess) rc = cuda_fail(cudaGetLastError(), "event");
-            float ms = 0.f;
-            if (!rc) {
-                cudaError_t e = cudaEventSynchronize(e1);
-                if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-                if (e != cudaSuccess) rc = cuda_fail(e, "batch autotune timing");
+            // two steps show a candidate that is out of the running (slower
+            // than the best by more than a twentieth); the others are timed
+            int done = 0;
+            double us = 0.0;
+            for (const int want : {std::min(2, K), K}) {
+                float ms = 0.f;
+                for (int q = 0; q < (done ? 0 : 2) && !rc; ++q) rc = launch_batched_step(b, q & 1);
+                const int n = want;
+                if (!rc && cudaEventRecord(e0, b->stream) != cudaSuccess) rc = cuda_fail(cudaGetLastError(), "event");
+                for (int q = 0; q < n && !rc; ++q) rc = launch_batched_step(b, q & 1);
+                if (!rc && cudaEventRecord(e1, b->stream) != cudaSuccess) rc = cuda_fail(cudaGetLastError(), "event");
+                if (!rc) {
+                    cudaError_t e = cudaEventSynchronize(e1);
+                    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+                    if (e != cudaSuccess) rc = cuda_fail(e, "batch autotune timing");
+                }
+                us = ms * 1e3 / n;
+                done += n;
+                if (rc || done >= K || us > 1.05 * best) break;
             }
             // the trial steps changed the state: put the deposited state back
             if (cudaMemcpyAsync(b->state[0][0], bk, bytes, cudaMemcpyDeviceToDevice, b->stream) != cudaSuccess ||
                 cudaMemcpyAsync(b->state[0][1], bk + bytes, bytes, cudaMemcpyDeviceToDevice, b->stream) != cudaSuccess)
                 rc = rc ? rc : cuda_fail(cudaGetLastError(), "batch autotune restore");
-            if (!rc && ms * 1e3 / K < best) {
-                best = ms * 1e3 / K;
+            if (rc) break;
+            if (us < kind_us[sh.tma]) {
+                kind_us[sh.tma] = us;
+                kind_fit[sh.tma] = shape_us(b, sh, sms);
+            }
+            if (done >= K && us < best) {
+                best = us;
                 best_chunk = chunk;
-                best_cps = cps;
-                best_tma = tma;
+                best_shape = sh;
             }
         }
-    }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     cudaStreamSynchronize(b->stream);
     cudaFree(backup);
     // the chosen shape; the next table build also clears the trial tallies
     b->chunk = rc ? chunk0 : best_chunk;
-    b->vec_cps = rc ? cps0 : best_cps;
-    const int tma_sel = rc ? tma0 : best_tma;
-    b->use_tma = tma_sel > 0;
-    b->tma_ipt = tma_sel == 2 ? 2 : 1;
+    if (!rc) {
+        b->tuned = true;
+        b->tuned_shape = best_shape;
+        b->tuned_active = active;
+        // the fit's error at full occupancy scales it as simulations finish
+        for (int k = 0; k < 3; ++k)
+            if (kind_fit[k] > 0.0) b->cal[k] = kind_us[k] / kind_fit[k];
+    }
     b->tab_dirty = true;
     if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
     if (rc) return rc;
@@ -1312,7 +1316,7 @@ int it_batch_run(it_batch *b, double tol, int64_t max_steps, int64_t check_every
     std::vector<double> ind;
     for (;;) {
         if (b->tab_dirty) {
-            int rc = build_table(b);
+            int rc = rebuild(b);
             if (rc) return rc;
         }
         // next pulse of a train: deposited at the start of its step
@@ -1348,7 +1352,7 @@ int it_batch_run(it_batch *b, double tol, int64_t max_steps, int64_t check_every
             }
         }
         if (changed) {
-            rc = build_table(b);
+            rc = rebuild(b);
             if (rc) return rc;
         }
         if (b->tab.empty()) break;
@@ -1369,46 +1373,36 @@ int it_batch_run(it_batch *b, double tol, int64_t max_steps, int64_t check_every
 
 int it_batch_tallies(it_batch *b, int32_t sim, it_tallies_t *t) {
     if (!b || !t || sim < 0 || sim >= b->nsim) return bfail(IT_EINVAL, "bad argument");
-    double acc[NT], rel[8];
-    IT_CK(cudaMemcpyAsync(acc, b->d_acc + (size_t)NT * sim, sizeof(acc), cudaMemcpyDeviceToHost, b->stream));
-    IT_CK(cudaMemcpyAsync(rel, b->d_rel + (size_t)8 * sim, sizeof(rel), cudaMemcpyDeviceToHost, b->stream));
-    // in-domain charge and extreme densities of this simulation's current set
+    // in-domain charge and extreme densities of this simulation's current set,
+    // then everything in one copy
     const size_t cells = (size_t)b->hs[sim].nx * b->hs[sim].ny * b->hs[sim].nz;
     const int parity = (int)(b->steps[sim] & 1);
-    constexpr int kMonBlocks = 64;
-    double *d_mon = nullptr;
-    IT_CK(cudaMalloc(&d_mon, sizeof(double) * NM * kMonBlocks));
     const double vol = b->dx[sim] * b->dx[sim] * b->dx[sim];
+    double *d_out = b->d_tal + NM * TAL_BLOCKS;
     int rc = launch_monitor_raw_f32(b->state[parity][0] + b->hs[sim].off, b->state[parity][1] + b->hs[sim].off,
-                                    cells, vol, d_mon, kMonBlocks, b->stream);
-    double mon[NM * kMonBlocks];
-    if (rc == IT_OK) {
-        cudaError_t e = cudaMemcpyAsync(mon, d_mon, sizeof(mon), cudaMemcpyDeviceToHost, b->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-        if (e != cudaSuccess) rc = cuda_fail(e, "batch tallies");
-    }
-    cudaFree(d_mon);
+                                    cells, vol, b->d_tal, TAL_BLOCKS, b->stream);
     if (rc) return rc;
+    batch_tally_kernel<<<1, TAL_OUT * 32, 0, b->stream>>>(b->d_acc + (size_t)NT * sim, b->d_rel + (size_t)8 * sim,
+                                                          b->d_tal, d_out);
+    IT_CK(cudaGetLastError());
+    double o[TAL_OUT];
+    IT_CK(cudaMemcpyAsync(o, d_out, sizeof(o), cudaMemcpyDeviceToHost, b->stream));
+    IT_CK(cudaStreamSynchronize(b->stream));
     std::memset(t, 0, sizeof(*t));
+    const double *rel = o + NT;
     for (int s = 0; s < 2; ++s) {
-        double sum = 0, mn = INFINITY, mx = -INFINITY;
-        for (int q = 0; q < kMonBlocks; ++q) {
-            sum += mon[q * NM + s];
-            mn = std::min(mn, mon[q * NM + 2 + s]);
-            mx = std::max(mx, mon[q * NM + 4 + s]);
-        }
-        t->in_domain[s] = sum;
-        t->n_min[s] = mn;
-        t->n_max[s] = mx;
+        t->released[s] = rel[s];
+        t->in_domain[s] = o[NT + 2 + s];
+        t->n_min[s] = o[NT + 4 + s];
+        t->n_max[s] = o[NT + 6 + s];
     }
-    t->recombined = acc[0];
-    t->collected_anode[0] = acc[1]; t->collected_anode[1] = acc[2];
-    t->collected_cathode[0] = acc[3]; t->collected_cathode[1] = acc[4];
-    t->lost_lateral[0] = acc[5]; t->lost_lateral[1] = acc[6];
-    t->space_charge[0] = acc[7]; t->space_charge[1] = acc[8];
-    t->released[0] = rel[0]; t->released[1] = rel[1];
+    t->recombined = o[0];
+    t->collected_anode[0] = o[1]; t->collected_anode[1] = o[2];
+    t->collected_cathode[0] = o[3]; t->collected_cathode[1] = o[4];
+    t->lost_lateral[0] = o[5]; t->lost_lateral[1] = o[6];
+    t->space_charge[0] = o[7]; t->space_charge[1] = o[8];
     const double r = rel[0] + rel[1];
-    t->f = r > 0 ? (acc[1] + acc[2] + acc[3] + acc[4]) / r : NAN;
+    t->f = r > 0 ? (o[1] + o[2] + o[3] + o[4]) / r : NAN;
     t->steps = b->steps[sim];
     t->dt_s = b->dt[sim];
     t->t_s = b->t_s[sim];
