@@ -74,6 +74,7 @@ struct ZmConf {
     int ctas_per_sm;
     long long wait_cycles;   // SM cycles a ring wait may take before it is declared lost
     int withhold;            // test hook: 1 = the first ring load is never issued
+    int pair;                // a thread's items are vertically adjacent rows in pairs
 };
 
 // Launch shape of the two-steps-per-launch z-march kernel: tiles of TY

@@ -7,7 +7,7 @@
 //
 // Layout and data movement:
 //   * a CTA owns TY full-width rows (y0 .. y0+TY-1) of one y-tile and marches
-//     up a chunk of z planes [z0, z1);
+//     up or down a chunk of z planes [z0, z1);
 //   * every plane it needs (z0-1 .. z1) arrives in a shared-memory slot by TMA
 //     (cp.async.bulk.tensor, 3-D tiles of n+ and n-): TY main rows plus one
 //     halo row above and below, wrapped when the lateral faces are periodic.
@@ -15,9 +15,10 @@
 //     electrode ghost planes z = -1 and z = nz) are filled with zeros by TMA,
 //     which is exactly the boundary condition n = 0;
 //   * an S-deep ring of slots keeps S-2 planes in flight while one plane is
-//     computed; the last warp to finish reading a slot refills it;
-//   * each thread owns float4 x-segments and keeps their k-1 and k values in
-//     registers; x and y neighbours and the k+1 plane come from shared memory;
+//     computed; a producer warp refills a slot when its readers have left it;
+//   * each thread owns float4 x-segments and keeps the last plane's and this
+//     plane's values in registers; x and y neighbours and the next plane come
+//     from shared memory;
 //     the update runs on paired FP32 instructions (two cells per instruction);
 //   * results are stored with coalesced 16-byte stores; per-thread FP32
 //     partial sums (at most 32 planes) are reduced per warp in FP64 and per
@@ -46,37 +47,60 @@ struct ZmMaps {
 constexpr int ZM_MAX_IPT = 4;                    // float4 items per thread
 constexpr int ZM_MAX_SEG = 8;                    // segments of a CTA kept in shared memory
 
-// Persistent step kernel: NW warps, all of them compute.
+// Persistent step kernel: NW warps that compute and, where PROD, one that
+// loads.
 //   The planes a CTA needs stream through an S-deep ring of shared-memory
 //   slots by TMA.  full[slot] completes when a plane's bytes have landed.
-//   There is no producer warp: every warp, after its reads of a slot, adds
-//   one to the slot's release counter, and the warp whose release completes
-//   the count (the last reader) refills the slot with the plane S further
-//   on.  So a slot is refilled the moment it is free, and all warps do the
-//   same work.
-//   Every warp marches up z, one plane per iteration, with no block-wide
-//   barrier inside the march.  The FP64 tallies live in shared memory (each
-//   warp's lane 0 adds to its own row), so the registers hold only the
-//   marching planes and offsets.
-template <bool PERIODIC, int IPT, int NW, bool SC>
-__global__ void __launch_bounds__(NW * 32, (NW <= 8 ? 2 : 1))
+//   PROD: one thread of an extra warp walks the CTA's planes, waits on
+//   empty[slot] (one arrival per computing warp) and loads the next plane.
+//   Otherwise every warp, after its reads of a slot, adds one to the slot's
+//   release counter, and the warp whose release completes the count refills
+//   the slot.  That refill is done by the warp the others wait for and adds
+//   about 1.2 us to every plane: 256x256x400, 8 rows, 2 CTAs per SM, ring of
+//   4: 73.6 us with the producer, 77 without (the loads and stores alone,
+//   with nothing computed, take 70 to 80); 512x512x256, 8 rows, 1 CTA per SM:
+//   170 against 195; 200x200x800 absorbing, 8 rows, 2 CTAs: 88 against 95.
+//   The ninth warp costs registers, though: 96 per thread instead of 128,
+//   which spills with space charge (384x320x128: 56.3 us with the producer,
+//   53.1 without), with more than two float4 per thread (32 rows of
+//   256x256x400: 142 against 83) and with two that are no pair beside
+//   absorbing faces, so those keep the refill by the last reader.
+//   Every warp marches along z, one plane per iteration, with no block-wide
+//   barrier inside the march.  DOWN: the CTA walks its planes downwards.
+//   Steps alternate between up and down, so that a step first reads the
+//   planes which the step before it wrote last and which are still in L2
+//   (256x256x400: 73.6 to 69.8 us); the update of a cell is the same
+//   operations either way.
+//   PAIR: a thread's two float4 lie one above the other, so each is the
+//   other's y neighbour: 4 shared-memory reads of 16 bytes per pair and
+//   species instead of 6.
+//   The FP64 tallies live in shared memory (each warp's lane 0 adds to its
+//   own row), so the registers hold only the marching planes and offsets.
+__host__ __device__ constexpr bool zm_prod(bool periodic, int ipt, bool sc, bool pair) {
+    return !sc && (ipt == 1 || (ipt == 2 && (periodic || pair)));
+}
+
+template <bool PERIODIC, int IPT, int NW, bool SC, bool PAIR, bool DOWN>
+__global__ void __launch_bounds__(NW * 32 + (zm_prod(PERIODIC, IPT, SC, PAIR) ? 32 : 0), (NW <= 8 ? 2 : 1))
 step_zmarch_kernel(const __grid_constant__ ZmMaps maps, float *__restrict__ outp, float *__restrict__ outm,
                    int nx, int ny, int nz, const ZmConf zc, const Coef<float> cf, double *__restrict__ slots,
                    int *__restrict__ err) {
     constexpr int NT_ = NW * 32;
+    constexpr bool PROD = zm_prod(PERIODIC, IPT, SC, PAIR);
     extern __shared__ __align__(128) unsigned char zm_smem_raw[];
     // TMA destinations need 128-byte alignment: round the base up explicitly
     unsigned char *smem_base = zm_smem_raw + ((128u - (smem_u32(zm_smem_raw) & 127u)) & 127u);
     float *ring = reinterpret_cast<float *>(smem_base);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem_base + (size_t)zc.S * zc.slot * sizeof(float));
-    uint32_t *rel = reinterpret_cast<uint32_t *>(full + zc.S);   // release counters
+    uint64_t *empty = full + zc.S;                                 // PROD: the slot's readers are done with it
+    uint32_t *rel = reinterpret_cast<uint32_t *>(full + zc.S);     // else: release counters
     uint32_t *fills = rel + zc.S;                                  // loads issued per slot
     // per-warp FP64 tallies (tally q of warp w at w*WQ+q): 7 tallies, 9 with
     // space charge; a power-of-two row keeps the index a shift
     constexpr int WQ = SC ? 16 : 8, NQ = SC ? 9 : 7;
     __shared__ double wacc[NW * WQ];
     __shared__ volatile int abort_flag;
-    __shared__ int seg_n0[ZM_MAX_SEG], seg_t[ZM_MAX_SEG], seg_za[ZM_MAX_SEG];
+    __shared__ int seg_n0[ZM_MAX_SEG], seg_t[ZM_MAX_SEG], seg_first[ZM_MAX_SEG];   // !PROD
 
     const int tid = threadIdx.x;
     const int lane = tid & 31;
@@ -88,82 +112,132 @@ step_zmarch_kernel(const __grid_constant__ ZmMaps maps, float *__restrict__ outp
     const long long g0 = total * blockIdx.x / gridDim.x;
     const long long g1 = total * (blockIdx.x + 1) / gridDim.x;
 
-    // planes this CTA loads: every segment [za, zb) loads zb - za + 2.  The
-    // first ZM_MAX_SEG segments are also kept in shared memory (first
-    // sequence number, tile, za), so that a refill finds its plane without
-    // the 64-bit divisions of the walk: a refill lies on the critical path,
-    // since the warp that issues it is the last one done with the slot
-    int nload = 0;
-    int nseg = 0;
-    {
-        Segs sg{g0, g1, nz, 0, 0, 0};
-        while (sg.next()) {
-            if (tid == 0 && nseg < ZM_MAX_SEG) {
-                seg_n0[nseg] = nload;
-                seg_t[nseg] = sg.t;
-                seg_za[nseg] = sg.za;
-            }
-            ++nseg;
-            nload += sg.zb - sg.za + 2;
-        }
-    }
-    const bool seg_cached = nseg <= ZM_MAX_SEG;
-
-    // load plane n of the sequence into its slot (one thread)
-    auto issue = [&](int n) {
-        int t = 0, p = 0;
-        if (n >= nload) return;
-        if (seg_cached) {
-            int i = 0;
-            while (i + 1 < nseg && n >= seg_n0[i + 1]) ++i;
-            t = seg_t[i];
-            p = seg_za[i] - 1 + (n - seg_n0[i]);
-        } else if (!plane_of(g0, g1, nz, n, t, p)) {
-            return;
-        }
-        const int slot = n % S;
+    // load plane p of tile t into a slot (one thread)
+    auto load = [&](int t, int p, int slot) {
         const int y0 = t * zc.TY;
         // halo rows: wrapped when periodic; rows -1 and ny otherwise, which
         // lie outside the tensor and arrive as zeros (absorbing faces hold
         // n = 0); planes -1 and nz arrive as zeros the same way
         const int ytop = PERIODIC ? (y0 > 0 ? y0 - 1 : ny - 1) : y0 - 1;
         const int ybot = PERIODIC ? (y0 + zc.TY < ny ? y0 + zc.TY : 0) : y0 + zc.TY;
-        const uint32_t tx = 2u * zc.nbx * (uint32_t)(zc.TY + 2) * zc.bx * 4u;
+        const uint32_t tx = 2u * (uint32_t)(zc.TY + 2) * zc.bx * 4u;
         float *base = ring + (size_t)slot * zc.slot;
         uint64_t *bar = &full[slot];
         fence_proxy_async();
         mbar_arrive_expect_tx(bar, tx);
+#pragma unroll
         for (int s = 0; s < 2; ++s) {
+            float *blk = base + (size_t)s * zc.blk;
             if (zc.xs > 1) {
-                // whole rows of a wide grid in one box (nbx == 1)
-                float *blk = base + (size_t)s * zc.blk;
+                // whole rows of a wide grid in one box
                 tma_load4(blk + zc.reg_main, &maps.main[s], bar, 0, 0, y0, p);
                 tma_load4(blk + zc.reg_top, &maps.halo[s], bar, 0, 0, ytop, p);
                 tma_load4(blk + zc.reg_bot, &maps.halo[s], bar, 0, 0, ybot, p);
-                continue;
-            }
-            for (int b = 0; b < zc.nbx; ++b) {
-                float *blk = base + (size_t)(s * zc.nbx + b) * zc.blk;
-                tma_load3(blk + zc.reg_main, &maps.main[s], bar, b * zc.bx, y0, p);
-                tma_load3(blk + zc.reg_top, &maps.halo[s], bar, b * zc.bx, ytop, p);
-                tma_load3(blk + zc.reg_bot, &maps.halo[s], bar, b * zc.bx, ybot, p);
+            } else {
+                tma_load3(blk + zc.reg_main, &maps.main[s], bar, 0, y0, p);
+                tma_load3(blk + zc.reg_top, &maps.halo[s], bar, 0, ytop, p);
+                tma_load3(blk + zc.reg_bot, &maps.halo[s], bar, 0, ybot, p);
             }
         }
+    };
+
+    // without a producer: planes this CTA loads (every segment [za, zb) loads
+    // zb - za + 2).  The first ZM_MAX_SEG segments are also kept in shared
+    // memory (first sequence number, tile, lowest plane, count), so that a
+    // refill finds its plane without the 64-bit divisions of the walk: a
+    // refill lies on the critical path, since the warp that issues it is the
+    // last one done with the slot
+    int nload = 0;
+    int nseg = 0;
+    if constexpr (!PROD) {
+        Segs sg{g0, g1, nz, 0, 0, 0};
+        while (sg.next()) {
+            if (tid == 0 && nseg < ZM_MAX_SEG) {
+                seg_n0[nseg] = nload;
+                seg_t[nseg] = sg.t;
+                seg_first[nseg] = DOWN ? sg.zb : sg.za - 1;
+            }
+            ++nseg;
+            nload += sg.zb - sg.za + 2;
+        }
+    }
+    // load plane n of the sequence into its slot (one thread)
+    auto issue = [&](int n) {
+        if (n >= nload) return;
+        int t = 0, p = 0;
+        if (nseg <= ZM_MAX_SEG) {
+            int i = 0;
+            while (i + 1 < nseg && n >= seg_n0[i + 1]) ++i;
+            t = seg_t[i];
+            p = DOWN ? seg_first[i] - (n - seg_n0[i]) : seg_first[i] + (n - seg_n0[i]);
+        } else {
+            Segs sg{g0, g1, nz, 0, 0, 0};
+            int m = n;   // loads of the segments from sg on
+            while (sg.next() && m >= sg.zb - sg.za + 2) m -= sg.zb - sg.za + 2;
+            t = sg.t;
+            p = DOWN ? sg.zb - m : sg.za - 1 + m;
+        }
+        const int slot = n % S;
+        load(t, p, slot);
         fills[slot] += 1;
     };
 
     if (tid == 0) {
         for (int q = 0; q < S; ++q) {
             mbar_init(&full[q], 1);
-            rel[q] = 0;
-            fills[q] = 0;
+            if (PROD) mbar_init(&empty[q], NW);
+            if (!PROD) rel[q] = fills[q] = 0;
         }
         for (int q = 0; q < NW * WQ; ++q) wacc[q] = 0.0;
         abort_flag = 0;
         fence_mbar_init();
-        for (int n = zc.withhold ? 1 : 0; n < S && n < nload; ++n) issue(n);
+        if constexpr (!PROD)
+            for (int n = zc.withhold ? 1 : 0; n < S && n < nload; ++n) issue(n);
     }
     __syncthreads();
+
+    if constexpr (PROD)
+        if (warp == NW) {
+            if (lane == 0) {
+                RingPos pos{0, 0u};
+                int n = 0;
+                Segs sg{g0, g1, nz, 0, 0, 0};
+                bool stop = false;
+                while (!stop && sg.next())
+                    for (int q = sg.za - 1; q <= sg.zb; ++q, ++n) {
+                        if (n >= S) {
+                            // the slot's readers (bounded by zc.wait_cycles)
+                            const uint32_t par = pos.phase ^ 1u;
+                            if (!mbar_try_wait(&empty[pos.slot], par)) {
+                                const long long t0 = clock64();
+                                while (!mbar_try_wait(&empty[pos.slot], par))
+                                    if (abort_flag || clock64() - t0 > zc.wait_cycles) {
+                                        stop = true;
+                                        break;
+                                    }
+                            }
+                            if (stop || abort_flag) {
+                                stop = true;
+                                abort_flag = 1;
+                                break;
+                            }
+                        }
+                        if (!(zc.withhold && n == 0)) load(sg.t, DOWN ? sg.za - 1 + sg.zb - q : q, pos.slot);
+                        pos.advance(S);
+                    }
+                if (stop) atomicExch(err, 1);
+                // no load may be in flight when the CTA exits: wait (bounded)
+                // for the last load issued into each slot
+                RingPos d{0, 0u};
+                for (int q = 0; q < n; ++q) {
+                    if (q + S >= n && !(zc.withhold && q == 0)) (void)mbar_wait_bounded(&full[d.slot], d.phase);
+                    d.advance(S);
+                }
+            }
+            __syncwarp();
+            __syncthreads();   // the computing warps' last barrier
+            return;
+        }
 
     // warp-uniform: reduce one FP32 partial per lane in FP64 (fixed shuffle
     // order) and add it to the warp's tally q
@@ -181,10 +255,12 @@ step_zmarch_kernel(const __grid_constant__ ZmMaps maps, float *__restrict__ outp
     bool valid[IPT];
 #pragma unroll
     for (int it = 0; it < IPT; ++it) {
-        const int q = tid + it * NT_;
-        valid[it] = q < nitems;
-        const int qe = valid[it] ? q : nitems - 1;
-        const int ty = qe / ncol4, c4 = qe - (qe / ncol4) * ncol4;
+        // items in raster order; as pairs: two vertically adjacent rows
+        const int q = tid + (PAIR ? it / 2 : it) * NT_;
+        const int nq = PAIR ? nitems / 2 : nitems;
+        valid[it] = q < nq;
+        const int qe = valid[it] ? q : nq - 1;
+        const int ty = PAIR ? 2 * (qe / ncol4) + (it & 1) : qe / ncol4, c4 = qe - (qe / ncol4) * ncol4;
         ty_[it] = ty;
         c4_[it] = c4;
         const int x0 = 4 * c4;
@@ -220,16 +296,21 @@ step_zmarch_kernel(const __grid_constant__ ZmMaps maps, float *__restrict__ outp
         failed = true;
         if (lane == 0) abort_flag = 1;
     };
-    // After the warp's reads of the slot: count the release; the last of the
-    // NW releases refills the slot.  A failed warp releases nothing, so no
-    // slot is refilled while its previous load may still be in flight.
+    // After the warp's reads of the slot: hand it back to the producer, or
+    // count the release, the last of NW refilling the slot.  A failed warp
+    // releases nothing, so no slot is refilled while its previous load may
+    // still be in flight.
     auto release = [&](const RingPos &u) {
         __syncwarp();
-        if (lane == 0 && !failed) {
-            const uint32_t old = atom_add_acq_rel(&rel[u.slot], 1u);
-            if (old % NW == NW - 1 && nrel + S < nload && !abort_flag) issue(nrel + S);
+        if constexpr (PROD) {
+            if (lane == 0 && !failed) mbar_arrive(&empty[u.slot]);
+        } else {
+            if (lane == 0 && !failed) {
+                const uint32_t old = atom_add_acq_rel(&rel[u.slot], 1u);
+                if (old % NW == NW - 1 && nrel + S < nload && !abort_flag) issue(nrel + S);
+            }
+            ++nrel;
         }
-        ++nrel;
     };
 
     Segs seg{g0, g1, nz, 0, 0, 0};
@@ -242,7 +323,8 @@ step_zmarch_kernel(const __grid_constant__ ZmMaps maps, float *__restrict__ outp
 #pragma unroll
         for (int it = 0; it < IPT; ++it) {
             const int yg = y0 + ty_[it];
-            off[it] = ((uint32_t)za * (uint32_t)ny + (uint32_t)yg) * (uint32_t)nx + 4u * (uint32_t)c4_[it];
+            off[it] = ((uint32_t)(DOWN ? zb - 1 : za) * (uint32_t)ny + (uint32_t)yg) * (uint32_t)nx +
+                      4u * (uint32_t)c4_[it];
             edge_u[it] = !PERIODIC && yg == 0;
             edge_d[it] = !PERIODIC && yg == ny - 1;
         }
@@ -272,54 +354,75 @@ step_zmarch_kernel(const __grid_constant__ ZmMaps maps, float *__restrict__ outp
         int nacc = 0;
         // not unrolled: an unrolled march (which would save the register
         // rotation of prev/cur) measured slower
-        for (int k = za; k < zb; ++k) {
+        for (int q = za; q < zb; ++q) {
+            const int k = DOWN ? za + zb - 1 - q : q;   // the plane computed; prev holds the one walked before it
             const bool electrode = k == 0 || k == nz - 1;
             wait_full(pos);
             const float *sk = ring + (size_t)pc.slot * zc.slot;
             const float *sn = ring + (size_t)pos.slot * zc.slot;
             float an[2] = {0.f, 0.f}, lat[2] = {0.f, 0.f};
+            // one item of one species: the update, its store and its tallies
+            auto item = [&](int it, int s, float4 n, float4 u, float4 d, float4 zn, float2 rxy, float2 rzw, float2 dxy,
+                            float2 dzw) {
+                const float *bk = sk + s * sp_ofs;
+                float l = bk[o_l[it]];
+                float r = bk[o_r[it]];
+                if (!PERIODIC) {
+                    if (c4_[it] == 0) l = 0.f;
+                    if (c4_[it] == ncol4 - 1) r = 0.f;
+                }
+                float4 v = upd7x4(n, l, r, u, d, DOWN ? zn : prev[it][s], DOWN ? prev[it][s] : zn, rxy, rzw, cf.wx[s],
+                                  cf.wzm[s], cf.wzp[s], cf.adt);
+                if (SC) {
+                    float2 pxy, pzw;
+                    v = add_sc4(v, cf.sc[s], n, dxy, dzw, pxy, pzw);
+                    if (valid[it]) (s ? ssum1 : ssum0) += (pxy.x + pxy.y) + (pzw.x + pzw.y);
+                }
+                if (valid[it]) {
+                    *reinterpret_cast<float4 *>((s ? outm : outp) + off[it]) = v;
+                    if (electrode) an[s] += (n.x + n.y) + (n.z + n.w);
+                    if (!PERIODIC) {
+                        if (c4_[it] == 0) lat[s] += n.x;
+                        if (c4_[it] == ncol4 - 1) lat[s] += n.w;
+                        if (edge_u[it]) lat[s] += (n.x + n.y) + (n.z + n.w);
+                        if (edge_d[it]) lat[s] += (n.x + n.y) + (n.z + n.w);
+                    }
+                }
+                prev[it][s] = n;
+                cur[it][s] = zn;
+            };
+            auto at = [](const float *q, int o) { return *reinterpret_cast<const float4 *>(q + o); };
 #pragma unroll
-            for (int it = 0; it < IPT; ++it) {
-                const float4 P = cur[it][0], M = cur[it][1];
-                const float2 rxy = __fmul2_rn(make_float2(P.x, P.y), make_float2(M.x, M.y));
-                const float2 rzw = __fmul2_rn(make_float2(P.z, P.w), make_float2(M.z, M.w));
-                float2 dxy, dzw;
-                if (SC) sc_diff4(P, M, dxy, dzw);
+            for (int it = 0; it < IPT; it += (PAIR ? 2 : 1)) {
+                constexpr int W = PAIR ? 2 : 1;   // items at a time
+                float2 rxy[W], rzw[W], dxy[W], dzw[W];
+#pragma unroll
+                for (int w = 0; w < W; ++w) {
+                    const float4 P = cur[it + w][0], M = cur[it + w][1];
+                    rxy[w] = __fmul2_rn(make_float2(P.x, P.y), make_float2(M.x, M.y));
+                    rzw[w] = __fmul2_rn(make_float2(P.z, P.w), make_float2(M.z, M.w));
+                    if (SC) sc_diff4(P, M, dxy[w], dzw[w]);
+                }
 #pragma unroll
                 for (int s = 0; s < 2; ++s) {
-                    const float *bk = sk + s * sp_ofs;
-                    const float4 n = cur[it][s];
-                    const float4 u = *reinterpret_cast<const float4 *>(bk + o_u[it]);
-                    const float4 d = *reinterpret_cast<const float4 *>(bk + o_d[it]);
-                    const float4 zp = *reinterpret_cast<const float4 *>(sn + s * sp_ofs + o_c[it]);
-                    float l = bk[o_l[it]];
-                    float r = bk[o_r[it]];
-                    if (!PERIODIC) {
-                        if (c4_[it] == 0) l = 0.f;
-                        if (c4_[it] == ncol4 - 1) r = 0.f;
+                    const float *bk = sk + s * sp_ofs, *bn = sn + s * sp_ofs;
+                    if constexpr (PAIR) {
+                        // the two rows are each other's y neighbours
+                        const float4 n0 = cur[it][s], n1 = cur[it + 1][s];
+                        const float4 u = at(bk, o_u[it]), d = at(bk, o_d[it + 1]);
+                        const float4 z0 = at(bn, o_c[it]), z1 = at(bn, o_c[it + 1]);
+                        item(it, s, n0, u, n1, z0, rxy[0], rzw[0], dxy[0], dzw[0]);
+                        item(it + 1, s, n1, n0, d, z1, rxy[W - 1], rzw[W - 1], dxy[W - 1], dzw[W - 1]);
+                    } else {
+                        item(it, s, cur[it][s], at(bk, o_u[it]), at(bk, o_d[it]), at(bn, o_c[it]), rxy[0], rzw[0],
+                             dxy[0], dzw[0]);
                     }
-                    float4 v = upd7x4(n, l, r, u, d, prev[it][s], zp, rxy, rzw,
-                                      cf.wx[s], cf.wzm[s], cf.wzp[s], cf.adt);
-                    if (SC) {
-                        float2 pxy, pzw;
-                        v = add_sc4(v, cf.sc[s], n, dxy, dzw, pxy, pzw);
-                        if (valid[it]) (s ? ssum1 : ssum0) += (pxy.x + pxy.y) + (pzw.x + pzw.y);
-                    }
-                    if (valid[it]) {
-                        *reinterpret_cast<float4 *>((s ? outm : outp) + off[it]) = v;
-                        if (electrode) an[s] += (n.x + n.y) + (n.z + n.w);
-                        if (!PERIODIC) {
-                            if (c4_[it] == 0) lat[s] += n.x;
-                            if (c4_[it] == ncol4 - 1) lat[s] += n.w;
-                            if (edge_u[it]) lat[s] += (n.x + n.y) + (n.z + n.w);
-                            if (edge_d[it]) lat[s] += (n.x + n.y) + (n.z + n.w);
-                        }
-                    }
-                    prev[it][s] = n;
-                    cur[it][s] = zp;
                 }
-                if (valid[it]) rsum += (rxy.x + rxy.y) + (rzw.x + rzw.y);
-                off[it] += plane;
+#pragma unroll
+                for (int w = 0; w < W; ++w) {
+                    if (valid[it + w]) rsum += (rxy[w].x + rxy[w].y) + (rzw[w].x + rzw[w].y);
+                    off[it + w] += DOWN ? 0u - plane : plane;   // modulo 2^32
+                }
             }
             // FP32 partial sums over at most 32 planes, then FP64
             if (!PERIODIC) { lsum0 += lat[0]; lsum1 += lat[1]; }
@@ -344,7 +447,7 @@ step_zmarch_kernel(const __grid_constant__ ZmMaps maps, float *__restrict__ outp
     }
     if (failed && lane == 0) atomicExch(err, 1);
     __syncthreads();
-    if (tid == 0) {
+    if (!PROD && tid == 0) {
         // no load may be in flight when the CTA exits: wait (bounded) for the
         // last load issued into each slot (already complete unless a wait
         // was lost)
@@ -479,40 +582,37 @@ static int align32f(int floats) { return (floats + 31) / 32 * 32; }   // 128-byt
 // shared by every context: raise it to the device's opt-in maximum (never
 // lower it to one context's need), so launches of other contexts with
 // larger tiles stay valid.
-template <bool P, int I, int W, bool S>
-static cudaError_t zm_set_attr(size_t smem) {
+template <bool P, int I, int W, bool S, bool R, bool D>
+static cudaError_t zm_set_attr(size_t smem, int *occ) {
+    auto *k = step_zmarch_kernel<P, I, W, S, R, D>;
     int dev = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
     cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, step_zmarch_kernel<P, I, W, S>);
+    e = cudaFuncGetAttributes(&fa, k);
     if (e != cudaSuccess) return e;
     const int max_dyn = optin - (int)fa.sharedSizeBytes;   // static shared memory counts against the limit
     if ((int)smem > max_dyn) return cudaErrorInvalidValue;
-    return cudaFuncSetAttribute(step_zmarch_kernel<P, I, W, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn);
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn);
+    int n = 0;
+    if (e == cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, W * 32 + (zm_prod(P, I, S, R) ? 32 : 0), smem) != cudaSuccess)
+        n = 0;
+    *occ = std::min(*occ, n);
+    return e;
 }
 
-template <bool P, int I, int W, bool S>
-static int zm_occupancy(size_t smem) {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_zmarch_kernel<P, I, W, S>, W * 32, smem) != cudaSuccess)
-        return 0;
-    return n;
+// both directions of the march (only the upward one with more than two float4
+// per thread: the rare shapes whose instances spill)
+template <bool P, int I, int W, bool S, bool R>
+static cudaError_t zm_prepare(size_t smem, int *occ) {
+    cudaError_t e = zm_set_attr<P, I, W, S, R, false>(smem, occ);
+    if (I <= 2 && e == cudaSuccess) e = zm_set_attr<P, I, W, S, R, I <= 2>(smem, occ);
+    return e;
 }
 
 static int ipt_of(const it_ctx *c, int TY, int nw) { return ((c->g.nx / 4) * TY + nw * 32 - 1) / (nw * 32); }
-
-// CTAs of a launch without a given grid: the largest multiple of the tile
-// count, so that every tile column is cut at the same z and adjacent tiles
-// stream in step (their halo rows are then still in L2), unless that leaves
-// more than a tenth of the resident slots empty (300 of 304 CTAs on
-// 200x200x800: 95.3 us against 100.4 with all of them; 280 on 384x320x128:
-// 53.1 against 58.0).
-static long long zmarch_grid(int ntile, long long slots) {
-    const long long g = slots / ntile * ntile;
-    return g * 10 >= slots * 9 ? g : slots;
-}
 
 static int sm_count() {
     int dev = 0, sms = 152;
@@ -521,33 +621,60 @@ static int sm_count() {
     return sms;
 }
 
-// Tile height and CTAs per SM when neither is given: the shape with the least
-// fitted time, (planes a CTA walks + 2) rounds and about 4 us to start and
-// drain; returns that time in us.  A round takes about 1.25 / 1.62 / 2.4 /
-// 3.7 us with one to four float4 per thread at two CTAs per SM and 1.3 / 1.75
-// / 2.4 / 3.5 at one (launch-shape sweeps on 256x256x400, 200x200x800,
-// 384x320x128 and 128x128x200: two CTAs per SM with two float4 per thread
-// take 76.8, 95.3, 56.5 and 19.3 us; the earlier rule, one CTA per SM with at
-// least two float4 per thread, took 81.7, 107.9, 59.0 and 22.4).
-static double zmarch_shape(const it_ctx *c, int *ty, int *cps) {
-    static const double round_us[2][4] = {{1.3, 1.75, 2.4, 3.5}, {1.25, 1.62, 2.4, 3.7}};
+// A thread's two (four) items as vertically adjacent rows?
+static bool zm_pairs(const it_ctx *c, int TY, int nw) {
+    const int ipt = ipt_of(c, TY, nw);
+    return ipt % 2 == 0 && TY % 2 == 0 && (c->g.nx / 4) * (TY / 2) <= (ipt / 2) * nw * 32;
+}
+
+// Tile height, CTAs per SM and grid when none is given: the shape with the
+// least fitted time, returned in us.  A CTA takes (planes it walks + 2) rounds
+// and about 4 us to start and drain.  A round is bound by memory or by the
+// CTA's own chain of wait, update and hand-over:
+//   * memory: 16 bytes per cell of all CTAs at 6.5 TB/s (2.46 ps per cell),
+//     times 1 + 0.75 / TY^2 when the grid is a multiple of the tile count (all
+//     tile columns are then cut at the same z and adjacent tiles stream in
+//     step, so that their halo rows come from L2), else 1 + 1 / TY (the two
+//     halo rows come from HBM);
+//   * the chain: 0.82 and 1.25 us with one and two float4 per thread and a
+//     producer, 1.7 / 2.0 / 3.2 for two to four without, 1.25 / 1.62 / 2.4 /
+//     4.3 with space charge; 10 % more at one CTA per SM without a producer,
+//     5 % more where the halo rows come from HBM.
+// Fitted to launch-shape sweeps on 18 grids, where the choice is the fastest
+// shape or within 3 % of it on all but four (within 10 %): 256x256x400 8 rows,
+// 2 CTAs per SM: 70 us (16 rows, 1 CTA: 72); 512x512x256 8 rows, 1 CTA: 170
+// (the whole 304 slots instead of a multiple of the tile count: 238);
+// 768x768x100 8 rows, 1 CTA, all 152 slots: 174 (4 rows, 2 CTAs: 207);
+// 1024x256x200 4 rows, 1 CTA: 138 (2 rows, 2 CTAs: 151); 384x320x128 with
+// space charge 8 rows, 2 CTAs: 53 (5 rows, 2 CTAs: 59).
+static double zmarch_shape(const it_ctx *c, int *ty, int *cps, long long *ctas) {
+    static const double prod_us[2] = {0.82, 1.25}, ring_us[4] = {1.25, 1.7, 2.0, 3.2}, sc_us[4] = {1.25, 1.62, 2.4, 4.3};
     const int sms = sm_count();
+    const bool sc = c->p.space_charge != 0, per = c->p.lateral_bc == IT_PERIODIC;
     double best = 1e300;
     for (int k = 2; k >= 1; --k)
         for (int t = 1; t <= std::min(c->g.ny, 255); ++t) {
             if (c->g.ny % t) continue;
-            const int ipt = ipt_of(c, t, k == 1 ? 16 : 8);
+            const int nw = k == 1 ? 16 : 8, ipt = ipt_of(c, t, nw);
             if (ipt > ZM_MAX_IPT) break;
             const size_t slot = sizeof(float) * 2 * (align32f(t * c->g.nx) + 2 * align32f(c->g.nx));
             if (3 * slot + 512 > (size_t)(220 * 1024) / k) continue;   // a ring of three slots must fit
             const int ntile = c->g.ny / t;
-            const long long tp = (long long)ntile * c->g.nz;
-            const long long grid = std::min<long long>(tp, zmarch_grid(ntile, (long long)sms * k));
-            const double us = (double)((tp + grid - 1) / grid + 2) * round_us[k - 1][ipt - 1] + 4.0;
-            if (us < 0.98 * best) {
-                best = us;
-                *ty = t;
-                *cps = k;
+            const long long tp = (long long)ntile * c->g.nz, slots = (long long)sms * k;
+            const double chain = zm_prod(per, ipt, sc, zm_pairs(c, t, nw))
+                                     ? prod_us[ipt - 1]
+                                     : (sc ? sc_us : ring_us)[ipt - 1] * (k == 1 ? 1.1 : 1.0);
+            for (int aligned = 1; aligned >= 0; --aligned) {
+                if (aligned && slots < ntile) continue;
+                const long long grid = std::min(tp, aligned ? slots / ntile * ntile : slots);
+                const double mem = 2.46e-6 * (double)(grid * t * c->g.nx) * (1.0 + (aligned ? 0.75 / t : 1.0) / t);
+                const double us = (double)((tp + grid - 1) / grid + 2) * std::max(aligned ? chain : 1.05 * chain, mem) + 4.0;
+                if (us < 0.98 * best) {
+                    best = us;
+                    *ty = t;
+                    *cps = k;
+                    *ctas = grid;
+                }
             }
         }
     return best;
@@ -569,7 +696,8 @@ int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid
         return IT_EINVAL;
     }
     int cps = want_cps > 0 ? want_cps : 1, TY = want_ty;
-    if (want_ty <= 0 && want_cps <= 0) zmarch_shape(c, &TY, &cps);
+    long long ctas = 0;
+    if (want_ty <= 0 && want_cps <= 0) zmarch_shape(c, &TY, &cps, &ctas);
     if (cps > 2) { set_error("z-march kernel runs 1 or 2 CTAs per SM"); return IT_EINVAL; }
     const int nw = cps == 1 ? 16 : 8;
     ZmConf z{};
@@ -602,24 +730,30 @@ int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid
     z.blk = z.reg_bot + align32f(z.bx);
     z.slot = 2 * z.nbx * z.blk;
     const size_t budget = (size_t)(220 * 1024) / cps;
+    const bool per = c->p.lateral_bc == IT_PERIODIC;
+    const int ipt = ipt_of(c, TY, nw);
+    const bool sc = c->p.space_charge != 0;
+    z.pair = zm_pairs(c, TY, nw);
+    // ring depth: with a producer the smallest (of 4 and more) that keeps
+    // 64 KB per SM in flight beyond the two planes in use; deeper rings only
+    // spread the CTAs' planes (256x256x400, 8 rows, 2 CTAs per SM: 71.6 / 69.8
+    // / 76.6 us with 3 / 4 / 5 slots; 200x200x800 absorbing, 10 rows: 85.2 /
+    // 90.5 with 4 / 5).  Otherwise what fits, up to 8.
     z.S = want_s > 0 ? want_s : 8;
+    if (want_s <= 0 && zm_prod(per, ipt, sc, z.pair))
+        for (z.S = 4; z.S < 8 && (size_t)(z.S - 2) * z.slot * sizeof(float) * cps < 64 * 1024;) ++z.S;
     if (z.S < 3 || z.S > 16) { set_error("z-march ring depth must be 3..16"); return IT_EINVAL; }
     for (;;) {
-        z.smem = (size_t)z.S * z.slot * sizeof(float) + 16 * z.S + 128;   // ring + barriers/counters + alignment slack
+        z.smem = (size_t)z.S * z.slot * sizeof(float) + 16 * z.S + 128;   // ring + barriers (and counters) + alignment slack
         if (z.smem <= budget || z.S == 3 || want_s > 0) break;
         --z.S;
     }
     if (z.smem > 227 * 1024) { set_error("z-march kernel: tile does not fit in shared memory"); return IT_EINVAL; }
-    const bool per = c->p.lateral_bc == IT_PERIODIC;
-    const int ipt = ipt_of(c, TY, nw);
     cudaError_t e = cudaSuccess;
-    int occ = 0;
-    const bool sc = c->p.space_charge != 0;
-#define ZM_CASE(P, I, W, S)                                        \
-    if (per == P && ipt == I && nw == W && sc == S) {              \
-        e = zm_set_attr<P, I, W, S>(z.smem);                       \
-        occ = zm_occupancy<P, I, W, S>(z.smem);                    \
-    }
+    int occ = cps;
+#define ZM_CASE(P, I, W, S)                                                                         \
+    if (per == P && ipt == I && nw == W && sc == S)                                                 \
+        e = z.pair ? zm_prepare<P, I, W, S, I % 2 == 0>(z.smem, &occ) : zm_prepare<P, I, W, S, false>(z.smem, &occ);
 #define ZM_CASES(S)                                                                          \
     ZM_CASE(true, 1, 16, S) ZM_CASE(true, 2, 16, S) ZM_CASE(true, 3, 16, S) ZM_CASE(true, 4, 16, S) \
     ZM_CASE(false, 1, 16, S) ZM_CASE(false, 2, 16, S) ZM_CASE(false, 3, 16, S) ZM_CASE(false, 4, 16, S) \
@@ -633,15 +767,16 @@ int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid
     z.ctas_per_sm = cps;
     const int sms = sm_count();
     // grid: CTAs, each taking one contiguous range of tile-planes.  0: one
-    // per resident slot (with no shape given at all, zmarch_grid's rule); -1: the largest multiple of the tile count that
-    // fits the resident slots, so every tile column is cut at the same z and
-    // vertically adjacent tiles are streamed in step (their halo rows are
-    // then still in L2); > 0: as given.
+    // per resident slot (with no shape given at all, zmarch_shape's choice);
+    // -1: the largest multiple of the tile count that fits the resident slots,
+    // so every tile column is cut at the same z and vertically adjacent tiles
+    // are streamed in step (their halo rows are then still in L2); > 0: as
+    // given.
     const long long tp = (long long)z.ntile * nz;
     long long grid = (long long)sms * cps;
     if (want_grid == -1 && grid >= z.ntile) grid = grid / z.ntile * z.ntile;
     else if (want_grid > 0) grid = want_grid;
-    else if (want_ty <= 0 && want_cps <= 0 && want_s <= 0) grid = zmarch_grid(z.ntile, grid);
+    else if (want_s <= 0 && ctas > 0) grid = ctas;
     z.nzc = (int)std::min<long long>(grid, tp);
     for (int set = 0; set < 2; ++set)
         for (int s = 0; s < 2; ++s) {
@@ -659,13 +794,14 @@ int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid
 
 // Does the march straight from L1/L2 (step_direct_kernel) beat the TMA-staged
 // one?  By the fitted times of both: it does while the state stays in L2
-// (256x256x100: 22.8 against 26.2 us per step, 128x128x200: 12.4 against
-// 19.6) and where ny has no divisor that fills a tile (224x293x119: one row
-// per tile took 154 us); from HBM it moves 1.45 times slower than a copy and
-// the ring wins (256x256x400: 86 against 77).
+// (128x128x200: 12.4 against 19.6 us per step, 256x256x100: 22.8 against a
+// fitted 24.6) and where ny has no divisor that fills a tile (224x293x119: one
+// row per tile took 154 us); from HBM it moves 1.45 times slower than a copy
+// and the ring wins (256x256x400: 86 against 70).
 bool direct_wins(const it_ctx *c) {
     int ty = 0, cps = 1;
-    return direct_us(c) < zmarch_shape(c, &ty, &cps);
+    long long ctas = 0;
+    return direct_us(c) < zmarch_shape(c, &ty, &cps, &ctas);
 }
 
 int zmarch_configure(it_ctx *c) { return zmarch_setup(c, 0, 0, 0, 0); }
@@ -687,10 +823,16 @@ int launch_step_zmarch(it_ctx *c, cudaStream_t s) {
     const int ipt = ipt_of(c, z.TY, nw);
     const int nx = c->g.nx, ny = c->g.ny, nz = c->g.nz;
     const bool sc = c->p.space_charge != 0;
-#define ZM_LAUNCH(P, I, W, S)                                                                            \
-    if (per == P && ipt == I && nw == W && sc == S)                                                      \
-        step_zmarch_kernel<P, I, W, S><<<c->zm_grid, W * 32, z.smem, s>>>(maps, op, om, nx, ny, nz, z, c->cf, \
-                                                                          c->d_slots, c->d_err);
+    const bool down = cur == 1;   // alternate steps, alternate directions
+#define ZM_LAUNCH(P, I, W, S)                                                                           \
+    if (per == P && ipt == I && nw == W && sc == S) {                                                   \
+        constexpr bool R = I % 2 == 0, D = I <= 2;                                                      \
+        auto *k = z.pair ? (down ? step_zmarch_kernel<P, I, W, S, R, D> : step_zmarch_kernel<P, I, W, S, R, false>) \
+                         : (down ? step_zmarch_kernel<P, I, W, S, false, D>                             \
+                                 : step_zmarch_kernel<P, I, W, S, false, false>);                       \
+        k<<<c->zm_grid, W * 32 + (zm_prod(P, I, S, z.pair) ? 32 : 0), z.smem, s>>>(                     \
+            maps, op, om, nx, ny, nz, z, c->cf, c->d_slots, c->d_err);                                  \
+    }
 #define ZM_LAUNCHES(S)                                                                                   \
     ZM_LAUNCH(true, 1, 16, S) ZM_LAUNCH(true, 2, 16, S) ZM_LAUNCH(true, 3, 16, S) ZM_LAUNCH(true, 4, 16, S) \
     ZM_LAUNCH(false, 1, 16, S) ZM_LAUNCH(false, 2, 16, S) ZM_LAUNCH(false, 3, 16, S) ZM_LAUNCH(false, 4, 16, S) \
