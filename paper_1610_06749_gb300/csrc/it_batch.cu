@@ -93,21 +93,26 @@ struct VecEntry {
 // and nx <= 256: the batched counterpart of the single-context step kernel.
 // A CTA owns rows [y0, y0 + rows) of one simulation (full width) and planes
 // [z0, z1).  Every plane it needs (z0 - 1 .. z1) arrives by TMA in a ring of
-// shared-memory slots: a box of bt = min(256 IPT / (nx/4), 256, ny) rows per
-// species plus one halo row above and below, wrapped when the faces are
+// shared-memory slots: a box of bt = min(IPT floor(256 / (nx/4)), 256, ny)
+// rows per species plus one halo row above and below, wrapped when the faces are
 // periodic; rows and planes outside the simulation's tensor arrive as zeros
 // (the absorbing faces and the electrode ghost planes).  Each simulation's
 // tensor maps (two sets x two species x {main box for IPT = 1, main box for
-// IPT = 2, halo row}) sit in global memory.  The last warp to release a slot
-// refills it with the plane S further on.  Thread t owns the IPT float4
-// x-segments q = t + 256 it (segment q mod (nx/4) of row q div (nx/4)),
-// keeps planes k-1 and k of them in registers and reads x/y neighbours and
-// plane k+1 from shared memory: the same per-cell operation sequence as
-// every other kernel.  IPT = 1 runs three CTAs per SM, IPT = 2 two with
-// larger rings; a plane's round through the CTA sets the time, and two
-// float4 per thread halve the rounds per cell.  Every ring wait is bounded
-// (2^32 SM cycles); a wait that runs out raises the error flag, and the CTA
-// drains the copies it issued and returns.
+// IPT = 2, halo row}) sit in global memory.  A thread owns IPT float4
+// x-segments, two of them one above the other (each is the other's y
+// neighbour), keeps planes k-1 and k of them in registers and reads x/y
+// neighbours and plane k+1 from shared memory: the same per-cell operation
+// sequence as every other kernel.  IPT = 1 runs three CTAs per SM, IPT = 2 two
+// with larger rings; a plane's round through the CTA sets the time, and two
+// float4 per thread halve the rounds per cell.  With IPT = 2 and no space
+// charge a ninth warp refills a slot as soon as its readers have left it;
+// otherwise the last warp to release a slot does (the ninth warp leaves 96
+// registers per thread).  Steps alternate between the entries' order and its
+// reverse.  256 uneven simulations of the batched workload (3.1 GB per step):
+// 577 us per step before the pairs and the producer, 503 with them (6.1 TB/s);
+// 64 of them: 183 and 158.  Every ring wait is bounded (2^32 SM cycles); a
+// wait that runs out raises the error flag, and the CTA drains the copies it
+// issued and returns.
 constexpr int BT_MAX_S = 8;
 constexpr int BT_WARPS = 8;
 // dynamic shared memory of the TMA batched kernel with one float4 per thread:
@@ -124,25 +129,33 @@ constexpr int BT_MAPS = 12;
 
 __device__ __forceinline__ int bt_align32(int f) { return (f + 31) & ~31; }
 
+__host__ __device__ constexpr bool bt_prod(bool sc, int ipt) { return !sc && ipt == 2; }
+__host__ __device__ constexpr int bt_threads(bool sc, int ipt) { return BT_WARPS * 32 + (bt_prod(sc, ipt) ? 32 : 0); }
+
 template <bool PERIODIC, bool SC, int IPT>
-__global__ void __launch_bounds__(BT_WARPS * 32, (IPT == 1 ? 3 : 2))
+__global__ void __launch_bounds__(bt_threads(SC, IPT), (IPT == 1 ? 3 : 2))
 step_batched_tma_kernel(const BatchSim *__restrict__ sims, const VecEntry *__restrict__ tab,
                         const CUtensorMap *__restrict__ maps, int parity, float *__restrict__ op_all,
                         float *__restrict__ om_all, double *__restrict__ slots, int smem_floats,
                         int *__restrict__ err) {
+    constexpr bool PROD = bt_prod(SC, IPT);
     constexpr int NW = BT_WARPS, WQ = SC ? 16 : 8, NQ = SC ? 9 : 7;
     extern __shared__ __align__(128) unsigned char bt_smem_raw[];
     unsigned char *smem_base = bt_smem_raw + ((128u - (smem_u32(bt_smem_raw) & 127u)) & 127u);
     float *ring = reinterpret_cast<float *>(smem_base);
     __shared__ double wacc[NW * WQ];
     __shared__ __align__(8) uint64_t full[BT_MAX_S];
+    __shared__ __align__(8) uint64_t empty[BT_MAX_S];   // PROD: the slot's readers are done with it
     __shared__ uint32_t rel[BT_MAX_S], fills[BT_MAX_S];
     __shared__ volatile int abort_flag;
     __shared__ BatchSim Sm;
     __shared__ VecEntry E;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // steps alternate between the entries' order and its reverse, so that a
+    // step first reads what the step before it wrote last (still in L2)
+    const unsigned ent = parity ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
     if (tid == 0) {
-        E = tab[blockIdx.x];
+        E = tab[ent];
         Sm = sims[E.sim];
     }
     __syncthreads();
@@ -153,7 +166,7 @@ step_batched_tma_kernel(const BatchSim *__restrict__ sims, const VecEntry *__res
     const float rwx[2] = {c.wx[0], c.wx[1]}, rwzm[2] = {c.wzm[0], c.wzm[1]}, rwzp[2] = {c.wzp[0], c.wzp[1]};
     const float radt = c.adt;
     const int ncol4 = nx >> 2;
-    const int bt = min(min(256 * IPT / ncol4, 256), ny);   // rows of the main box (a box dimension is <= 256)
+    const int bt = min(min(IPT * (256 / ncol4), 256), ny);   // rows of the main box (a box dimension is <= 256)
     const int rows = E.rows;                        // rows computed (<= bt)
     const int reg_main = bt_align32(nx), reg_bot = reg_main + bt_align32(bt * nx), blk = reg_bot + bt_align32(nx);
     const int slotf = 2 * blk;
@@ -186,6 +199,7 @@ step_batched_tma_kernel(const BatchSim *__restrict__ sims, const VecEntry *__res
         for (int q = 0; q < 6; ++q) fence_tensormap_acquire(&mp[q]);
         for (int q = 0; q < S; ++q) {
             mbar_init(&full[q], 1);
+            if (PROD) mbar_init(&empty[q], NW);
             rel[q] = 0;
             fills[q] = 0;
         }
@@ -195,6 +209,38 @@ step_batched_tma_kernel(const BatchSim *__restrict__ sims, const VecEntry *__res
         for (int n = 0; n < S && n < nload; ++n) issue(n);
     }
     __syncthreads();
+
+    if constexpr (PROD)
+        if (warp == NW) {
+            // the producer: refills a slot when its readers have left it
+            // (bounded wait); no load may be in flight when the CTA exits
+            if (lane == 0) {
+                RingPos pos{0, 0u};
+                for (int n = S; n < nload; ++n) {
+                    bool lost = false;
+                    if (!mbar_try_wait(&empty[pos.slot], pos.phase)) {
+                        const long long t0 = clock64();
+                        while (!mbar_try_wait(&empty[pos.slot], pos.phase))
+                            if (abort_flag || clock64() - t0 > (1LL << 32)) {
+                                lost = true;
+                                break;
+                            }
+                    }
+                    if (lost || abort_flag) {
+                        abort_flag = 1;
+                        atomicExch(err, 1);
+                        break;
+                    }
+                    issue(n);
+                    pos.advance(S);
+                }
+                for (int j = 0; j < S; ++j)
+                    if (fills[j] > 0) (void)mbar_wait_bounded(&full[j], (fills[j] - 1u) & 1u);
+            }
+            __syncwarp();
+            __syncthreads();   // the computing warps' last barrier
+            return;
+        }
 
     auto flush = [&](int q, float part) {
         double v = (double)part;
@@ -211,15 +257,19 @@ step_batched_tma_kernel(const BatchSim *__restrict__ sims, const VecEntry *__res
     const uint32_t plane = (uint32_t)nx * (uint32_t)ny;
 #pragma unroll
     for (int it = 0; it < IPT; ++it) {
-        const int q = tid + it * BT_WARPS * 32;
-        valid[it] = q < rows * ncol4;
-        const int te = valid[it] ? q : rows * ncol4 - 1;
-        const int ty = te / ncol4, c4 = te - ty * ncol4;
+        // two segments: one above the other, so that each is the other's y
+        // neighbour (below an odd last row: the halo row, not stored)
+        const int q = IPT == 2 ? tid : tid + it * BT_WARPS * 32;
+        const int nq = IPT == 2 ? (rows + 1) / 2 * ncol4 : rows * ncol4;
+        const int te = q < nq ? q : nq - 1;
+        const int tr = te / ncol4, c4 = te - tr * ncol4;
+        const int ty = IPT == 2 ? 2 * tr + it : tr;
+        valid[it] = q < nq && ty < rows;
         const int x0 = 4 * c4;
         c4_[it] = c4;
-        o_c[it] = reg_main + ty * nx + x0;
+        o_c[it] = ty < rows ? reg_main + ty * nx + x0 : reg_bot + x0;
         o_u[it] = ty == 0 ? x0 : reg_main + (ty - 1) * nx + x0;
-        o_d[it] = ty == rows - 1 ? reg_bot + x0 : reg_main + (ty + 1) * nx + x0;
+        o_d[it] = ty >= rows - 1 ? reg_bot + x0 : reg_main + (ty + 1) * nx + x0;
         o_l[it] = reg_main + ty * nx + (c4 == 0 ? nx - 1 : x0 - 1);
         o_r[it] = reg_main + ty * nx + (c4 == ncol4 - 1 ? 0 : x0 + 4);
         const int yg = y0 + ty;
@@ -247,11 +297,15 @@ step_batched_tma_kernel(const BatchSim *__restrict__ sims, const VecEntry *__res
     };
     auto release = [&](const RingPos &u) {
         __syncwarp();
-        if (lane == 0 && !failed) {
-            const uint32_t old = atom_add_acq_rel(&rel[u.slot], 1u);
-            if (old % NW == NW - 1 && nrel + S < nload && !abort_flag) issue(nrel + S);
+        if constexpr (PROD) {
+            if (lane == 0 && !failed) mbar_arrive(&empty[u.slot]);
+        } else {
+            if (lane == 0 && !failed) {
+                const uint32_t old = atom_add_acq_rel(&rel[u.slot], 1u);
+                if (old % NW == NW - 1 && nrel + S < nload && !abort_flag) issue(nrel + S);
+            }
+            ++nrel;
         }
-        ++nrel;
     };
 
     float4 prev[IPT][2], cur[IPT][2];
@@ -284,30 +338,37 @@ step_batched_tma_kernel(const BatchSim *__restrict__ sims, const VecEntry *__res
         const float *sk = ring + (size_t)pc.slot * slotf;
         const float *sn = ring + (size_t)pos.slot * slotf;
         float an[2] = {0.f, 0.f}, lat[2] = {0.f, 0.f};
+        float2 rxy[IPT], rzw[IPT], dxy[IPT], dzw[IPT];
 #pragma unroll
         for (int it = 0; it < IPT; ++it) {
             const float4 P = cur[it][0], M = cur[it][1];
-            const float2 rxy = __fmul2_rn(make_float2(P.x, P.y), make_float2(M.x, M.y));
-            const float2 rzw = __fmul2_rn(make_float2(P.z, P.w), make_float2(M.z, M.w));
-            float2 dxy, dzw;
-            if (SC) sc_diff4(P, M, dxy, dzw);
+            rxy[it] = __fmul2_rn(make_float2(P.x, P.y), make_float2(M.x, M.y));
+            rzw[it] = __fmul2_rn(make_float2(P.z, P.w), make_float2(M.z, M.w));
+            if (SC) sc_diff4(P, M, dxy[it], dzw[it]);
+        }
 #pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                const float *bk = sk + s * blk;
-                const float4 n = cur[it][s];
-                const float4 u = *reinterpret_cast<const float4 *>(bk + o_u[it]);
-                const float4 d = *reinterpret_cast<const float4 *>(bk + o_d[it]);
-                const float4 zp = *reinterpret_cast<const float4 *>(sn + s * blk + o_c[it]);
+        for (int s = 0; s < 2; ++s) {
+            const float *bk = sk + s * blk;
+            auto at = [](const float *q, int o) { return *reinterpret_cast<const float4 *>(q + o); };
+            const float4 above = at(bk, o_u[0]), below = at(bk, o_d[IPT - 1]);
+            float4 nc[IPT];
+#pragma unroll
+            for (int it = 0; it < IPT; ++it) nc[it] = cur[it][s];
+#pragma unroll
+            for (int it = 0; it < IPT; ++it) {
+                const float4 n = nc[it];
+                const float4 u = it == 0 ? above : nc[0], d = it == IPT - 1 ? below : nc[IPT - 1];
+                const float4 zp = at(sn + s * blk, o_c[it]);
                 float l = bk[o_l[it]];
                 float r = bk[o_r[it]];
                 if (!PERIODIC) {
                     if (c4_[it] == 0) l = 0.f;
                     if (c4_[it] == ncol4 - 1) r = 0.f;
                 }
-                float4 v = upd7x4(n, l, r, u, d, prev[it][s], zp, rxy, rzw, rwx[s], rwzm[s], rwzp[s], radt);
+                float4 v = upd7x4(n, l, r, u, d, prev[it][s], zp, rxy[it], rzw[it], rwx[s], rwzm[s], rwzp[s], radt);
                 if (SC) {
                     float2 pxy, pzw;
-                    v = add_sc4(v, c.sc[s], n, dxy, dzw, pxy, pzw);
+                    v = add_sc4(v, c.sc[s], n, dxy[it], dzw[it], pxy, pzw);
                     if (valid[it]) (s ? ssum1 : ssum0) += (pxy.x + pxy.y) + (pzw.x + pzw.y);
                 }
                 if (valid[it]) {
@@ -323,7 +384,10 @@ step_batched_tma_kernel(const BatchSim *__restrict__ sims, const VecEntry *__res
                 prev[it][s] = n;
                 cur[it][s] = zp;
             }
-            if (valid[it]) rsum += (rxy.x + rxy.y) + (rzw.x + rzw.y);
+        }
+#pragma unroll
+        for (int it = 0; it < IPT; ++it) {
+            if (valid[it]) rsum += (rxy[it].x + rxy[it].y) + (rzw[it].x + rzw[it].y);
             off[it] += plane;
         }
         if (!PERIODIC) { lsum0 += lat[0]; lsum1 += lat[1]; }
@@ -346,7 +410,7 @@ step_batched_tma_kernel(const BatchSim *__restrict__ sims, const VecEntry *__res
     release(pc);   // plane z1
     if (failed && lane == 0) atomicExch(err, 1);
     __syncthreads();
-    if (tid == 0) {
+    if (!PROD && tid == 0) {
         // no copy may be in flight when the CTA exits
         for (int j = 0; j < S; ++j)
             if (fills[j] > 0) (void)mbar_wait_bounded(&full[j], (fills[j] - 1u) & 1u);
@@ -358,7 +422,7 @@ step_batched_tma_kernel(const BatchSim *__restrict__ sims, const VecEntry *__res
             for (int w = 0; w < NW; ++w) v += wacc[w * WQ + q];
             acc[q] = v;
         }
-        double *sl = slots + (size_t)blockIdx.x * NT;
+        double *sl = slots + (size_t)ent * NT;
         sl[0] += acc[0] * c.rec_f;
         sl[1] += acc[1] * c.anode_f[0];
         sl[2] += acc[2] * c.anode_f[1];
@@ -560,7 +624,7 @@ int sm_count() {
     return sms;
 }
 
-int tma_rows(const BatchSim &h, int ipt) { return std::max(1, std::min(256 * ipt / (h.nx / 4), 256)); }
+int tma_rows(const BatchSim &h, int ipt) { return std::max(1, std::min(ipt * (256 / (h.nx / 4)), 256)); }
 long long march_blocks(const BatchSim &h, int v) {
     return ((long long)(h.nx / v) * h.ny + SK_THREADS - 1) / SK_THREADS;
 }
@@ -612,14 +676,16 @@ int direct_chunk(const it_batch *b, int sms, double *us) {
 }
 
 // Fitted time of a step of the active simulations in us, TMA-staged: a plane's
-// round takes 1.5 us with two float4 per thread and two CTAs per SM, 1.32 with
-// one and three, the last entries leave the chip a fifth of the longest one
-// idle, and starting takes about 6 us (256 uneven simulations of the batched
-// workload at one, two, three and six z splits: 614, 576, 579 and 602 us,
-// fitted 610, 590, 589 and 605).
+// round takes 1.3 us with two float4 per thread and two CTAs per SM (1.5 with
+// space charge, which has no producer warp), 1.32 with one and three, the last
+// entries leave the chip a fifth of the longest one idle, and starting takes
+// about 6 us (256 uneven simulations of the batched workload at one, two,
+// three and six z splits: 552, 510, 503 and 531 us, fitted 537, 519, 519 and
+// 534; 64 of them at three, five and ten: 163, 158 and 170, fitted 159, 156
+// and 160).
 double tma_us(const it_batch *b, const BatchShape &sh, int sms) {
     const int split = tma_split(b, sh, sms);
-    const double round = sh.tma == 2 ? 1.5 : 1.32;
+    const double round = sh.tma == 2 ? (b->p.space_charge ? 1.5 : 1.3) : 1.32;
     double rounds = 0.0;
     int longest = 0;
     for (int s = 0; s < b->nsim; ++s) {
@@ -794,7 +860,7 @@ int launch_batched_step(it_batch *b, int parity) {
                               : (sc ? step_batched_tma_kernel<false, true, 2> : step_batched_tma_kernel<false, false, 2>))
                        : (per ? (sc ? step_batched_tma_kernel<true, true, 1> : step_batched_tma_kernel<true, false, 1>)
                               : (sc ? step_batched_tma_kernel<false, true, 1> : step_batched_tma_kernel<false, false, 1>));
-        kt<<<nt, BT_WARPS * 32, two ? kBtSmem2 : kBtSmem, b->stream>>>(b->d_sims, b->d_vtab, b->d_maps, parity, op,
+        kt<<<nt, bt_threads(sc, two ? 2 : 1), two ? kBtSmem2 : kBtSmem, b->stream>>>(b->d_sims, b->d_vtab, b->d_maps, parity, op,
                                                                        om, b->d_slots,
                                                                        two ? kBtSmemFloats2 : kBtSmemFloats, b->d_err);
         IT_CK(cudaGetLastError());
@@ -1031,7 +1097,7 @@ int it_batch_create(int32_t nsim, const it_sim_desc *descs, const it_params *com
                     CUtensorMap *m = &maps[(size_t)s * BT_MAPS + set * 6 + sp * 3];
                     for (int ipt = 1; ipt <= 2 && rc == IT_OK; ++ipt)
                         rc = encode_map(&m[ipt - 1], base_s, h.nx, h.ny, h.nz, h.nx,
-                                        std::min(std::min(256 * ipt / (h.nx / 4), 256), h.ny));
+                                        std::min(tma_rows(h, ipt), h.ny));
                     if (rc == IT_OK) rc = encode_map(&m[2], base_s, h.nx, h.ny, h.nz, h.nx, 1);
                 }
             if (rc) { batch_free(b); return rc; }
