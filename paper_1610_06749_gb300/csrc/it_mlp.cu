@@ -453,8 +453,7 @@ layer1_fwd_kernel(const __nv_bfloat16 *__restrict__ A0, long long zA0, const __n
 // the inputs): 256 x 6 outputs, so a block owns 16 rows o and the six columns
 // of one 16 x 8 product.  Its four warps stage 256 samples at a time in shared
 // memory (dZ1 from its transposed copy), one of them walks them 16 at a step
-// (fragments straight from global memory by one warp took 11 us, this
-// 4.2).
+// (fragments straight from global memory by one warp took 11 us, this 4.2).
 constexpr int W1_K = 256;
 __global__ void __launch_bounds__(128)
 layer1_wgrad_kernel(const __nv_bfloat16 *__restrict__ dZT, long long zT, long long ldT,

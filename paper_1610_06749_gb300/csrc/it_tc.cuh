@@ -21,9 +21,9 @@
 //   * all eight warps then read the accumulator back with tcgen05.ld (warp w
 //     reaches TMEM lanes 32 (w mod 4) .., i.e. those rows of the tile, and
 //     takes columns 16 (w / 4) ..) and run the epilogue functor on their
-//     32 x 16 block, each warp with a slice
-//     of the (by then idle) stage memory to reorder its block for coalesced
-//     stores; what the epilogue reads is loaded before the wait.
+//     32 x 16 block, each warp with a slice of the (by then idle) stage memory
+//     to reorder its block for coalesced stores; what the epilogue reads is
+//     loaded before the wait.
 // Every mbarrier wait is bounded (about 2^31 SM cycles); a wait that runs
 // out raises the error flag, no further copy or MMA is issued, the copies
 // already issued are waited for, and tensor memory is freed before return.
