@@ -58,17 +58,21 @@ struct RegCoef {
 // per step of surrogate simulations (48 x 48 cells) 256 of them take 136, 64
 // 40, 16 12.1 and four 6.3 us, against 166, 60, 20.7 and 16.5 with the ring
 // (85, 21, 5.6 and 1.1 at the copy rate); the 256 larger ones of the batched
-// workload, which stream from HBM, take 624 against 576.
+// workload, which stream from HBM, take 634 against 503.  rev: the entries in
+// reverse order (a step of 256 surrogate simulations and their remainders on
+// average 62.6 to 59.5 us).
 template <bool PERIODIC, bool SC, int V>
 __global__ void __launch_bounds__(SK_THREADS, (V == 4 ? DK_BLOCKS : SK_BLOCKS_F32))
 step_batched_march_kernel(const BatchSim *__restrict__ sims, const MarchEntry *__restrict__ tab,
                           const float *__restrict__ ip_all, const float *__restrict__ im_all,
-                          float *__restrict__ op_all, float *__restrict__ om_all, double *__restrict__ slots) {
+                          float *__restrict__ op_all, float *__restrict__ om_all, int rev,
+                          double *__restrict__ slots) {
     constexpr int NV = MarchValues<PERIODIC, SC>::N;
     __shared__ double raw[5 * SK_THREADS];
     CompSum(*buf)[SK_THREADS] = reinterpret_cast<CompSum(*)[SK_THREADS]>(raw);
     __shared__ double tot[9];
-    const MarchEntry E = tab[blockIdx.x];
+    const unsigned ent = rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    const MarchEntry E = tab[ent];
     const BatchSim &S = sims[E.sim];
     const RegCoef c(S.cf);
     const long long off = S.off;
@@ -80,7 +84,7 @@ step_batched_march_kernel(const BatchSim *__restrict__ sims, const MarchEntry *_
         simple_march<float, uint32_t, PERIODIC, SC>(ip_all + off, im_all + off, op_all + off, om_all + off, S.nx, S.ny,
                                                     S.nz, E.q0, E.k0, E.k1, c, buf, tot);
     __syncthreads();
-    if (threadIdx.x < 9) sk_slot<PERIODIC, SC, NV>(tot, S.cf, slots, threadIdx.x, 1);
+    if (threadIdx.x < 9) sk_slot<PERIODIC, SC, NV>(tot, S.cf, slots + (size_t)ent * NT, threadIdx.x, 1);
 }
 
 // Entry of the TMA-staged kernel: rows [y0, y0 + rows) of one simulation,
@@ -593,6 +597,7 @@ struct it_batch {
     cudaGraphExec_t graph;
     int graph_len, graph_parity;
     bool tab_dirty;
+    double active_bytes;   // both sets of the simulations in the tables
     // pulse trains: each simulation's deposited tracks are re-deposited every
     // period_steps steps until count pulses have been released
     std::vector<std::vector<double>> pulse_tracks;   // packed [n][4]
@@ -742,6 +747,7 @@ int build_table(it_batch *b) {
     long long active_cells = 0;
     for (int s = 0; s < b->nsim; ++s)
         if (b->active[s]) active_cells += (long long)b->hs[s].nx * b->hs[s].ny * b->hs[s].nz;
+    b->active_bytes = 16.0 * (double)active_cells;
     const int sms = sm_count();
     const long long chunk = std::max(1024LL, std::min(b->chunk, active_cells / (4LL * sms)));
     const BatchShape sh = b->shape;
@@ -854,6 +860,8 @@ int launch_batched_step(it_batch *b, int parity) {
     float *op = b->state[parity ^ 1][0], *om = b->state[parity ^ 1][1];
     const bool per = b->p.lateral_bc == IT_PERIODIC;
     const bool sc = b->p.space_charge != 0;
+    // alternating order of the entries where the state streams from HBM
+    const int rev = parity && b->active_bytes > DK_ALTERNATE;
     if (nt) {
         const bool two = b->shape.tma == 2;
         auto *kt = two ? (per ? (sc ? step_batched_tma_kernel<true, true, 2> : step_batched_tma_kernel<true, false, 2>)
@@ -868,13 +876,15 @@ int launch_batched_step(it_batch *b, int parity) {
     if (nd) {
         auto *kd = per ? (sc ? step_batched_march_kernel<true, true, 4> : step_batched_march_kernel<true, false, 4>)
                        : (sc ? step_batched_march_kernel<false, true, 4> : step_batched_march_kernel<false, false, 4>);
-        kd<<<nd, SK_THREADS, 0, b->stream>>>(b->d_sims, b->d_dtab, ip, im, op, om, b->d_slots + (size_t)NT * nt);
+        kd<<<nd, SK_THREADS, 0, b->stream>>>(b->d_sims, b->d_dtab, ip, im, op, om, rev,
+                                                b->d_slots + (size_t)NT * nt);
         IT_CK(cudaGetLastError());
     }
     if (ns) {
         auto *ks = per ? (sc ? step_batched_march_kernel<true, true, 1> : step_batched_march_kernel<true, false, 1>)
                        : (sc ? step_batched_march_kernel<false, true, 1> : step_batched_march_kernel<false, false, 1>);
-        ks<<<ns, SK_THREADS, 0, b->stream>>>(b->d_sims, b->d_stab, ip, im, op, om, b->d_slots + (size_t)NT * (nt + nd));
+        ks<<<ns, SK_THREADS, 0, b->stream>>>(b->d_sims, b->d_stab, ip, im, op, om, rev,
+                                                b->d_slots + (size_t)NT * (nt + nd));
         IT_CK(cudaGetLastError());
     }
     return IT_OK;

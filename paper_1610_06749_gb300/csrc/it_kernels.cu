@@ -60,7 +60,7 @@ step_simple_kernel(const T *__restrict__ ip, const T *__restrict__ im, T *__rest
         simple_march<T, Idx, PERIODIC, SC>(ip, im, op, om, nx, ny, nz, (Idx)pb * SK_THREADS, k0, k1, c, buf, tot);
     }
     __syncthreads();
-    if (tid < 9) sk_slot<PERIODIC, SC, NV>(tot, c, slots, tid, add);
+    if (tid < 9) sk_slot<PERIODIC, SC, NV>(tot, c, slots + (size_t)blockIdx.x * NT, tid, add);
 }
 
 // Chunks per column and blocks of a launch, by the fitted time of a split.
@@ -162,12 +162,13 @@ int launch_step_simple_raw_f32(const float *ip, const float *im, float *op, floa
 // It has no ring to fill and no slot hand-back, which is what a step of a
 // small or middle-sized grid (state in L2) spends its time on with the
 // TMA-staged kernel; on grids that stream from HBM the ring wins.
-// DIRECT_MEASURED
+// 128x128x200 9.9-12.4 us per step against 19.6 with the ring, 256x256x100
+// 22.8 against a fitted 24.6; 256x256x400 86 against 70.
 template <typename Idx, bool PERIODIC, bool SC>
 __global__ void __launch_bounds__(SK_THREADS, DK_BLOCKS)
 step_direct_kernel(const float *__restrict__ ip, const float *__restrict__ im, float *__restrict__ op,
-                   float *__restrict__ om, int nx, int ny, int nz, unsigned npb, unsigned nchunk, const Coef<float> c,
-                   double *__restrict__ slots) {
+                   float *__restrict__ om, int nx, int ny, int nz, unsigned npb, unsigned nchunk, int rev,
+                   const Coef<float> c, double *__restrict__ slots) {
     constexpr int NV = MarchValues<PERIODIC, SC>::N;
     __shared__ double raw[5 * SK_THREADS];
     CompSum(*buf)[SK_THREADS] = reinterpret_cast<CompSum(*)[SK_THREADS]>(raw);
@@ -175,13 +176,14 @@ step_direct_kernel(const float *__restrict__ ip, const float *__restrict__ im, f
     const int tid = threadIdx.x;
     if (tid < 9) tot[tid] = 0.0;
     const unsigned long long units = (unsigned long long)npb * nchunk;
-    for (unsigned long long u = blockIdx.x; u < units; u += gridDim.x) {
+    for (unsigned long long q = blockIdx.x; q < units; q += gridDim.x) {
+        const unsigned long long u = rev ? units - 1 - q : q;
         const unsigned pb = (unsigned)(u % npb), ch = (unsigned)(u / npb);
         const int k0 = (int)((long long)nz * ch / nchunk), k1 = (int)((long long)nz * (ch + 1) / nchunk);
         direct_march<Idx, PERIODIC, SC>(ip, im, op, om, nx, ny, nz, (Idx)pb * SK_THREADS, k0, k1, c, buf, tot);
     }
     __syncthreads();
-    if (tid < 9) sk_slot<PERIODIC, SC, NV>(tot, c, slots, tid, 1);
+    if (tid < 9) sk_slot<PERIODIC, SC, NV>(tot, c, slots + (size_t)blockIdx.x * NT, tid, 1);
 }
 
 // Chunks and blocks, fitted as the simple kernel's are; *cycles receives the
@@ -229,9 +231,10 @@ int launch_step_direct(it_ctx *c, cudaStream_t s) {
     const int cur = c->cur, nxt = cur ^ 1;
     const int nx = c->g.nx, ny = c->g.ny, nz = c->g.nz;
     const SkShape h = dk_shape(nx, ny, nz);
+    const int rev = cur == 1 && 16.0 * (double)c->g.cells() > DK_ALTERNATE;
     const float *ip = (const float *)c->n[cur][0], *im = (const float *)c->n[cur][1];
     float *op = (float *)c->n[nxt][0], *om = (float *)c->n[nxt][1];
-    auto go = [&](auto *k) { k<<<h.grid, SK_THREADS, 0, s>>>(ip, im, op, om, nx, ny, nz, h.npb, h.nchunk, c->cf, c->d_slots); };
+    auto go = [&](auto *k) { k<<<h.grid, SK_THREADS, 0, s>>>(ip, im, op, om, nx, ny, nz, h.npb, h.nchunk, rev, c->cf, c->d_slots); };
     // 32-bit element offsets: the z-march family takes grids below 2^32 cells
     if (c->p.lateral_bc == IT_PERIODIC)
         c->cf.sc_on ? go(step_direct_kernel<uint32_t, true, true>) : go(step_direct_kernel<uint32_t, true, false>);

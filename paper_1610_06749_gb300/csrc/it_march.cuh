@@ -16,6 +16,13 @@ constexpr int SK_BLOCKS_F32 = 8, SK_BLOCKS_F64 = 6;   // resident blocks per SM
 constexpr int DK_BLOCKS = 4;                            // of the direct kernel (128 registers)
 constexpr double DK_LAT = 650.0, DK_THR = 190.0;        // its cycles per plane: alone, and per block it shares the SM with
 
+// The direct march's units run in alternating order, step by step, where both
+// sets of the state exceed this: a step then first reads what the step before
+// it wrote last and is still in L2 (320x331x120, 203 MB: 47.3 to 45.6 us,
+// 224x293x119, 125 MB: 30.0 to 29.6; smaller states stay in L2 either way and
+// lose, 256x256x100, 105 MB: 22.8 to 23.6).
+constexpr double DK_ALTERNATE = 115e6;
+
 // FP32 sum that carries the rounding error of each addition (Knuth's
 // two-sum), so a sum of some hundred terms keeps about 46 bits: as good as
 // FP64 for terms that are FP32 products.  A sum that overflows or meets a
@@ -98,8 +105,8 @@ __device__ __forceinline__ void sk_reduce(const Sum (&v)[N], Sum (*buf)[SK_THREA
     }
 }
 
-// Tally tid of a block's slot from its sums (order: rec, lateral, space
-// charge, anode from 5, cathode from 7), added or written.
+// Tally tid of a block's slot (at slots) from its sums (order: rec, lateral,
+// space charge, anode from 5, cathode from 7), added or written.
 template <bool PERIODIC, bool SC, int NV, typename T>
 __device__ __forceinline__ void sk_slot(const double *tot, const Coef<T> &c, double *slots, int tid, int add) {
     double t = 0.0;
@@ -109,7 +116,7 @@ __device__ __forceinline__ void sk_slot(const double *tot, const Coef<T> &c, dou
     // x and y weights are equal for dx = dy (latx_f == laty_f)
     else if (tid < 7) t = PERIODIC ? 0.0 : tot[1 + tid - 5] * c.latx_f[tid - 5];
     else t = SC ? tot[NV - 2 + tid - 7] * c.sc_f[tid - 7] : 0.0;
-    double *sl = slots + (size_t)blockIdx.x * NT + tid;
+    double *sl = slots + tid;
     *sl = add ? *sl + t : t;
 }
 
