@@ -1138,7 +1138,11 @@ int it_batch_create(int32_t nsim, const it_sim_desc *descs, const it_params *com
 
 namespace {
 
-// Deposit packed tracks [n][4] into simulation `sim`'s current set.
+// Deposit packed tracks [n][4] into simulation `sim`'s current set.  Nothing is
+// waited for, so that the next simulation's deposit is prepared meanwhile: the
+// host copy of pageable memory may run at any later time (a Grace host's pages
+// need no staging), so packed points into the simulation's pulse_tracks, which
+// outlive every copy.
 int deposit_sim(it_batch *b, int sim, const double *packed, int64_t n) {
     if (n <= 0) return IT_OK;
     const it_sim_desc &d = b->desc[sim];
@@ -1177,8 +1181,6 @@ int deposit_sim(it_batch *b, int sim, const double *packed, int64_t n) {
     cudaError_t e = cudaMemcpyAsync(b->d_tracks, packed, sizeof(double) * 4 * n, cudaMemcpyHostToDevice, b->stream);
     if (e != cudaSuccess) rc = cuda_fail(e, "track upload");
     v->d_tracks = b->d_tracks; v->d_wx = b->d_wx; v->d_wy = b->d_wy;
-    // packed is pageable: it has been staged when the copy returns, so nothing
-    // is waited for and the next simulation's deposit is prepared meanwhile
     if (rc == IT_OK) rc = launch_deposit(v, n, b->stream);
     delete v;
     return rc;
@@ -1198,15 +1200,22 @@ int it_batch_deposit_tracks(it_batch *b, int32_t sim, int64_t n, const double *x
         if (!std::isfinite(xy[2 * t]) || !std::isfinite(xy[2 * t + 1]) || !(let[t] >= 0) || !std::isfinite(let[t]) ||
             !(bb[t] > 0) || !std::isfinite(bb[t]))
             return bfail(IT_EINVAL, "track values must be finite with LET >= 0 and b > 0");
-    std::vector<double> packed((size_t)n * 4);
+    auto &pt = b->pulse_tracks[sim];
+    // growing the simulation's list moves it: wait for the copies out of it
+    if (!pt.empty()) IT_CK(cudaStreamSynchronize(b->stream));
+    const size_t at = pt.size();
+    pt.resize(at + (size_t)n * 4);
+    double *packed = pt.data() + at;
     for (int64_t t = 0; t < n; ++t) {
         packed[4 * t] = xy[2 * t]; packed[4 * t + 1] = xy[2 * t + 1];
         packed[4 * t + 2] = let[t]; packed[4 * t + 3] = bb[t];
     }
-    int rc = deposit_sim(b, sim, packed.data(), n);
-    if (rc) return rc;
-    auto &pt = b->pulse_tracks[sim];
-    pt.insert(pt.end(), packed.begin(), packed.end());
+    int rc = deposit_sim(b, sim, packed, n);
+    if (rc) {
+        cudaStreamSynchronize(b->stream);
+        pt.resize(at);
+        return rc;
+    }
     b->pulse_done[sim] = 1;
     return IT_OK;
 }
