@@ -648,6 +648,7 @@ struct it_mlp {
     long long pX_cap;
     cudaStream_t side[2];         // weight and bias gradients run beside the data gradients
     cudaEvent_t ev[12];
+    cudaEvent_t up[2];            // the uploads of an epoch have been read (epochs alternate)
     // training set
     float *X, *Y;
     long long n_data;
@@ -671,6 +672,8 @@ void mlp_free(it_mlp *n) {
     cudaFree(n->fhat); cudaFree(n->dz); cudaFree(n->yb); cudaFree(n->idx); cudaFree(n->loss);
     cudaFree(n->eidx); cudaFree(n->eloss); cudaFree(n->count); cudaFree(n->corr); cudaFree(n->pX);
     for (auto &e : n->ev)
+        if (e) cudaEventDestroy(e);
+    for (auto &e : n->up)
         if (e) cudaEventDestroy(e);
     for (auto &v : n->side)
         if (v) cudaStreamDestroy(v);
@@ -871,16 +874,17 @@ int adam_room(it_mlp *n, long long steps) {
 
 // The bias corrections of the next `steps` Adam steps; the counters restart:
 // the step at `first` (-1 where a gather raises it before its first use), the
-// mini-batch at 0.
-int adam_begin(it_mlp *n, long long steps, int first) {
+// mini-batch at 0.  The copy out of c is asynchronous (pageable memory is only
+// staged where it has to be, and a Grace host's pages need not): the caller
+// keeps c unchanged until the stream has passed it.
+int adam_begin(it_mlp *n, long long steps, int first, std::vector<float2> &c) {
     int rc = adam_room(n, steps);
     if (rc) return rc;
-    std::vector<float2> c((size_t)steps);
+    c.resize((size_t)steps);
     for (long long q = 0; q < steps; ++q) {
         const double t = (double)(n->adam_t + 1 + q);
         c[q] = make_float2((float)(1.0 - std::pow(0.9, t)), (float)(1.0 - std::pow(0.999, t)));
     }
-    // pageable source: staged before the call returns
     IT_CK(cudaMemcpyAsync(n->corr, c.data(), sizeof(float2) * steps, cudaMemcpyHostToDevice, n->stream));
     IT_CK(cudaMemsetAsync(n->count, first < 0 ? 0xff : 0, sizeof(int), n->stream));
     IT_CK(cudaMemsetAsync(n->count + 1, 0, sizeof(int), n->stream));
@@ -965,6 +969,8 @@ int it_mlp_create(int32_t members, int32_t max_batch, it_mlp **out) {
         (e = cudaMemsetAsync(n->count, 0, 2 * sizeof(int), n->stream)) != cudaSuccess)
         return bail("mlp step counters");
     for (auto &v : n->ev)
+        if ((e = cudaEventCreateWithFlags(&v, cudaEventDisableTiming)) != cudaSuccess) return bail("mlp events");
+    for (auto &v : n->up)
         if ((e = cudaEventCreateWithFlags(&v, cudaEventDisableTiming)) != cudaSuccess) return bail("mlp events");
     n->bpad = ((long long)max_batch + 63) / 64 * 64;
     const long long zw = (long long)members * 3 * H * H, zt = (long long)members * H * n->bpad;
@@ -1090,7 +1096,6 @@ int it_mlp_train(it_mlp *n, int32_t epochs, int32_t batch, double lr, uint64_t s
     // are enqueued without host synchronisation
     std::vector<uint64_t> st(Z);
     for (int z = 0; z < Z; ++z) st[z] = seed + 0x9E3779B97F4A7C15ULL * (uint64_t)(z + 1);
-    std::vector<int> hidx((size_t)Z * N);
     std::vector<double> lossb(Z);
     // mini-batches of an epoch: whole ones (the tail is left out), or one
     // short one when there are fewer samples than a batch
@@ -1099,6 +1104,15 @@ int it_mlp_train(it_mlp *n, int32_t epochs, int32_t batch, double lr, uint64_t s
     double *eloss = loss_per_epoch ? n->eloss : nullptr;
     int rc = adam_room(n, nb);
     if (rc) return rc;
+    // host copies of what an epoch uploads (sample orders, Adam's corrections),
+    // two of each: an epoch's are written again two epochs later, once its
+    // uploads have been read
+    std::vector<int> hidx[2];
+    std::vector<float2> hcorr[2];
+    for (int u = 0; u < std::min(epochs, 2); ++u) {
+        hidx[u].resize((size_t)Z * N);
+        hcorr[u].resize((size_t)nb);
+    }
     // the same step over and over: recorded once and replayed where the
     // recording (about 0.4 ms) pays
     cudaGraphExec_t graph = nullptr;
@@ -1108,18 +1122,22 @@ int it_mlp_train(it_mlp *n, int32_t epochs, int32_t batch, double lr, uint64_t s
     }
     cudaError_t e = cudaSuccess;
     for (int ep = 0; ep < epochs && !rc && e == cudaSuccess; ++ep) {
+        const int u = ep & 1;
+        if (ep >= 2) {
+            e = cudaEventSynchronize(n->up[u]);
+            if (e != cudaSuccess) break;
+        }
         for (int z = 0; z < Z; ++z) {
-            int *pz = hidx.data() + (size_t)z * N;
+            int *pz = hidx[u].data() + (size_t)z * N;
             for (long long i = 0; i < N; ++i) pz[i] = (int)i;
             for (long long i = N - 1; i > 0; --i) {   // Fisher-Yates with SplitMix64
                 const long long j = (long long)(splitmix_next(st[z]) % (uint64_t)(i + 1));
                 std::swap(pz[i], pz[j]);
             }
         }
-        // pageable source: the copy is staged before the call returns, so
-        // hidx may be refilled for the next epoch right away
-        e = cudaMemcpyAsync(n->eidx, hidx.data(), sizeof(int) * (size_t)Z * N, cudaMemcpyHostToDevice, n->stream);
-        if (e == cudaSuccess) rc = adam_begin(n, nb, -1);
+        e = cudaMemcpyAsync(n->eidx, hidx[u].data(), sizeof(int) * (size_t)Z * N, cudaMemcpyHostToDevice, n->stream);
+        if (e == cudaSuccess) rc = adam_begin(n, nb, -1, hcorr[u]);
+        if (e == cudaSuccess && !rc) e = cudaEventRecord(n->up[u], n->stream);
         if (e == cudaSuccess && !rc && eloss) e = cudaMemsetAsync(eloss, 0, sizeof(double) * Z, n->stream);
         for (long long q = 0; q < nb && !rc && e == cudaSuccess; ++q) {
             if (graph) e = cudaGraphLaunch(graph, n->stream);
@@ -1167,11 +1185,13 @@ int it_mlp_loss_grad(it_mlp *n, int64_t count, const double *x, const double *y,
 
 int it_mlp_adam_step(it_mlp *n, double lr) {
     if (!n || !(lr > 0)) return mfail(IT_EINVAL, "bad argument");
-    int rc = adam_begin(n, 1, 0);
+    std::vector<float2> c;
+    int rc = adam_begin(n, 1, 0, c);
     if (!rc) rc = adam_step(n, (float)lr);
+    if (!rc) n->adam_t += 1;
+    const cudaError_t e = cudaStreamSynchronize(n->stream);   // c is released on return
     if (rc) return rc;
-    n->adam_t += 1;
-    IT_CK(cudaStreamSynchronize(n->stream));
+    if (e != cudaSuccess) return cuda_fail(e, "Adam step");
     return IT_OK;
 }
 
