@@ -219,7 +219,7 @@ constexpr int kGraphSteps = 32;   // even: a segment returns to the same ping-po
 // run n steps with no deposit in between
 static int run_plain(it_ctx *c, int64_t n) {
     while (n >= kGraphSteps) {
-        if (!c->graph || c->graph_parity != c->cur) {
+        if (!c->graph || c->graph_parity != c->cur || c->graph_base != c->base) {
             if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
             const int start = c->cur;
             cudaGraph_t g = nullptr;
@@ -234,6 +234,7 @@ static int run_plain(it_ctx *c, int64_t n) {
             cudaGraphDestroy(g);
             if (e != cudaSuccess) { c->graph = nullptr; return cuda_fail(e, "cudaGraphInstantiate"); }
             c->graph_parity = start;
+            c->graph_base = c->base;
         }
         IT_CK(cudaGraphLaunch(c->graph, c->stream));
         n -= kGraphSteps;
@@ -796,6 +797,7 @@ int it_set_density(it_ctx *c, const void *plus, const void *minus, size_t bytes)
     IT_CK(cudaMemsetAsync(c->d_slots, 0, sizeof(double) * NT * c->nslots, c->stream));
     IT_CK(cudaMemsetAsync(c->d_acc, 0, sizeof(DevAcc), c->stream));
     c->steps = 0;
+    c->base = c->cur;
     c->t_s = 0.0;
     c->sched_step.clear(); c->sched_tr.clear(); c->sched_ptr = 0;
     c->log_step.assign(1, 0);
@@ -844,6 +846,7 @@ int it_reset(it_ctx *c) {
     IT_CK(cudaMemsetAsync(c->d_acc, 0, sizeof(DevAcc), c->stream));
     IT_CK(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
     c->steps = 0;
+    c->base = c->cur;
     c->t_s = 0.0;
     c->sched_step.clear(); c->sched_tr.clear(); c->sched_ptr = 0;
     // the time step stays; the log restarts from it

@@ -110,6 +110,8 @@ struct it_ctx {
     size_t esize;         // element size
     void *n[2][2];        // [set][species]
     int cur;              // current set
+    int base;             // the set of step 0 (creation, it_reset, it_set_density): odd steps, cur != base, run in the
+                          // other direction, so a rerun groups its sums as a fresh context does
     bool own_state;
     void *state_base;
     cudaStream_t stream;
@@ -145,7 +147,7 @@ struct it_ctx {
     // graph of a fixed segment of steps
     cudaGraphExec_t graph;
     int graph_len;
-    int graph_parity;
+    int graph_parity, graph_base;   // cur and base the graph was captured for
     // z-march kernel configuration (it_zmarch.cu)
     itk::ZmConf zm;
     int zm_grid;

@@ -231,7 +231,7 @@ int launch_step_direct(it_ctx *c, cudaStream_t s) {
     const int cur = c->cur, nxt = cur ^ 1;
     const int nx = c->g.nx, ny = c->g.ny, nz = c->g.nz;
     const SkShape h = dk_shape(nx, ny, nz);
-    const int rev = cur == 1 && 16.0 * (double)c->g.cells() > DK_ALTERNATE;
+    const int rev = cur != c->base && 16.0 * (double)c->g.cells() > DK_ALTERNATE;
     const float *ip = (const float *)c->n[cur][0], *im = (const float *)c->n[cur][1];
     float *op = (float *)c->n[nxt][0], *om = (float *)c->n[nxt][1];
     auto go = [&](auto *k) { k<<<h.grid, SK_THREADS, 0, s>>>(ip, im, op, om, nx, ny, nz, h.npb, h.nchunk, rev, c->cf, c->d_slots); };

@@ -823,7 +823,7 @@ int launch_step_zmarch(it_ctx *c, cudaStream_t s) {
     const int ipt = ipt_of(c, z.TY, nw);
     const int nx = c->g.nx, ny = c->g.ny, nz = c->g.nz;
     const bool sc = c->p.space_charge != 0;
-    const bool down = cur == 1;   // alternate steps, alternate directions
+    const bool down = cur != c->base;   // alternate steps, alternate directions
 #define ZM_LAUNCH(P, I, W, S)                                                                           \
     if (per == P && ipt == I && nw == W && sc == S) {                                                   \
         constexpr bool R = I % 2 == 0, D = I <= 2;                                                      \
