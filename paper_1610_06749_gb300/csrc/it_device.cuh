@@ -42,6 +42,62 @@ __device__ __forceinline__ double warp_strided_sum(const double *__restrict__ v,
     return t;
 }
 
+// FP32 sum that carries the rounding error of each addition (Knuth's
+// two-sum), so a sum of some hundred terms keeps about 46 bits: as good as
+// FP64 for terms that are FP32 products.  A sum that overflows or meets a
+// NaN is returned as it is.
+struct CompSum {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float s = __fadd_rn(hi, x);
+        const float b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+        hi = s;
+    }
+    __device__ __forceinline__ void add(const CompSum &o) {
+        const float l = o.lo;
+        add(o.hi);
+        lo = __fadd_rn(lo, l);
+    }
+    __device__ __forceinline__ void scale(float w) {   // w a small whole number
+        const float p = __fmul_rn(hi, w);
+        lo = __fmaf_rn(lo, w, __fmaf_rn(hi, w, -p));
+        hi = p;
+    }
+    __device__ __forceinline__ double value() const {
+        return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+    }
+    __device__ __forceinline__ CompSum down(int o) const {
+        CompSum r;
+        r.hi = __shfl_down_sync(0xffffffffu, hi, o);
+        r.lo = __shfl_down_sync(0xffffffffu, lo, o);
+        return r;
+    }
+};
+
+__device__ __forceinline__ void add4(CompSum &c, float4 v) { c.add(v.x); c.add(v.y); c.add(v.z); c.add(v.w); }
+
+// Two such sums side by side in paired-FP32 instructions (seven for two terms;
+// multiplications by -1 are exact, so every line is one rounding as above).
+struct CompSum2 {
+    float2 hi = make_float2(0.f, 0.f), lo = make_float2(0.f, 0.f);
+    __device__ __forceinline__ void add(float2 x) {
+        const float2 neg = make_float2(-1.f, -1.f);
+        const float2 s = __fadd2_rn(hi, x);
+        const float2 nb = __ffma2_rn(s, neg, hi);                      // hi - s
+        const float2 eh = __ffma2_rn(__fadd2_rn(s, nb), neg, hi);      // hi - (s - b)
+        lo = __fadd2_rn(lo, __fadd2_rn(eh, __fadd2_rn(x, nb)));
+        hi = s;
+    }
+    __device__ __forceinline__ CompSum total() const {
+        CompSum t;
+        t.add(hi.x);
+        t.add(hi.y);
+        t.lo = __fadd_rn(t.lo, __fadd_rn(lo.x, lo.y));
+        return t;
+    }
+};
+
 // One cell of the update as an increment in flux form:
 //   n + [wd ((l + r) + (u + d) - 4 n) + wzm (zm - n) + wzp (zp - n) - adt rr]
 // (wd = wx = wy: the cells are cubes).  Every transport term is a weight

@@ -23,40 +23,7 @@ constexpr double DK_LAT = 650.0, DK_THR = 190.0;        // its cycles per plane:
 // lose, 256x256x100, 105 MB: 22.8 to 23.6).
 constexpr double DK_ALTERNATE = 115e6;
 
-// FP32 sum that carries the rounding error of each addition (Knuth's
-// two-sum), so a sum of some hundred terms keeps about 46 bits: as good as
-// FP64 for terms that are FP32 products.  A sum that overflows or meets a
-// NaN is returned as it is.
-struct CompSum {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float x) {
-        const float s = __fadd_rn(hi, x);
-        const float b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
-        hi = s;
-    }
-    __device__ __forceinline__ void add(const CompSum &o) {
-        const float l = o.lo;
-        add(o.hi);
-        lo = __fadd_rn(lo, l);
-    }
-    __device__ __forceinline__ void scale(float w) {   // w a small whole number
-        const float p = __fmul_rn(hi, w);
-        lo = __fmaf_rn(lo, w, __fmaf_rn(hi, w, -p));
-        hi = p;
-    }
-    __device__ __forceinline__ double value() const {
-        return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
-    }
-    __device__ __forceinline__ CompSum down(int o) const {
-        CompSum r;
-        r.hi = __shfl_down_sync(0xffffffffu, hi, o);
-        r.lo = __shfl_down_sync(0xffffffffu, lo, o);
-        return r;
-    }
-};
-
-// the same for FP64 states: a plain FP64 sum
+// CompSum's counterpart for FP64 states: a plain FP64 sum
 struct PlainSum {
     double hi = 0.0;
     __device__ __forceinline__ void add(double x) { hi += x; }
@@ -119,8 +86,6 @@ __device__ __forceinline__ void sk_slot(const double *tot, const Coef<T> &c, dou
     double *sl = slots + tid;
     *sl = add ? *sl + t : t;
 }
-
-__device__ __forceinline__ float dk_sum(float4 a) { return __fadd_rn(__fadd_rn(a.x, a.y), __fadd_rn(a.z, a.w)); }
 
 // Values a unit reduces: recombination, lateral +/- (absorbing), space charge +/-.
 template <bool PERIODIC, bool SC>
@@ -219,7 +184,11 @@ __device__ __forceinline__ void simple_march(const T *__restrict__ ip, const T *
 }
 
 // The same with a float4 x-segment per thread (nx % 4 == 0), segment q0 + tid
-// (step_direct_kernel).
+// (step_direct_kernel).  Every cell's terms enter compensated sums, so the
+// tallies are as close as the simple kernel's; in paired instructions that
+// costs nothing against four cells added in FP32 first (128x128x200 9.8 us per
+// step both ways) but with space charge, where there are three such sums
+// (384x320x128: 54.3 us, 53.2 with the four cells in FP32).
 template <typename Idx, bool PERIODIC, bool SC, class C>
 __device__ __forceinline__ void direct_march(const float *__restrict__ ip, const float *__restrict__ im,
                                              float *__restrict__ op, float *__restrict__ om, int nx, int ny, int nz,
@@ -242,6 +211,7 @@ __device__ __forceinline__ void direct_march(const float *__restrict__ ip, const
     const bool el = lane == 0 || first, er = lane == 31 || last || q4 + 1 >= plane4;
     const Idx ql = first ? q + (Idx)(nx - 1) : q - 1, qr = last ? q - (Idx)(nx - 4) : q + 4;
     CompSum v[NV];
+    CompSum2 rec, spc[2];   // recombination, space charge
     Idx base = (Idx)k0 * plane;
     auto ld = [&](const float *f, Idx e) { return __ldg(reinterpret_cast<const float4 *>(f + e)); };
     float4 zm[2], n[2], zp[2];
@@ -251,7 +221,9 @@ __device__ __forceinline__ void direct_march(const float *__restrict__ ip, const
     n[1] = ld(im, base + q);
     zp[0] = k0 + 1 < nz ? ld(ip, base + plane + q) : zero4;
     zp[1] = k0 + 1 < nz ? ld(im, base + plane + q) : zero4;
-    const float an[2] = {dk_sum(n[0]), dk_sum(n[1])};   // the chunk's first plane (anode tally)
+    CompSum an[2];   // the chunk's first plane (anode tally)
+    add4(an[0], n[0]);
+    add4(an[1], n[1]);
     // y neighbours and the x neighbours a shuffle cannot give, of plane k
     float4 up[2], dn[2];
     float le[2], re[2];
@@ -266,7 +238,6 @@ __device__ __forceinline__ void direct_march(const float *__restrict__ ip, const
         }
     };
     around(base);
-    float ca[2] = {0.f, 0.f};
     for (int k = k0; k < k1; ++k, base += plane) {
         float4 z2[2];   // two planes above, for the next round
         const bool more = k + 1 < k1 && k + 2 < nz;
@@ -287,21 +258,22 @@ __device__ __forceinline__ void direct_march(const float *__restrict__ ip, const
             if constexpr (SC) {
                 float2 pxy, pzw;
                 w4[s] = add_sc4(w4[s], c.sc[s], n[s], dxy, dzw, pxy, pzw);
-                v[NV - 2 + s].add(dk_sum(make_float4(pxy.x, pxy.y, pzw.x, pzw.y)));
+                spc[s].add(pxy);
+                spc[s].add(pzw);
             }
             if constexpr (!PERIODIC) {
                 if (first) v[1 + s].add(n[s].x);
                 if (last) v[1 + s].add(n[s].w);
-                if (j == 0) v[1 + s].add(dk_sum(n[s]));
-                if (j == ny - 1) v[1 + s].add(dk_sum(n[s]));
+                if (j == 0) add4(v[1 + s], n[s]);
+                if (j == ny - 1) add4(v[1 + s], n[s]);
             }
-            if (k == nz - 1) ca[s] = dk_sum(n[s]);
         }
         if (k + 1 < k1) around(base + plane);
 #pragma unroll
         for (int s = 0; s < 2; ++s)
             if (act) *reinterpret_cast<float4 *>((s ? om : op) + base + q) = w4[s];
-        v[0].add(dk_sum(make_float4(rxy.x, rxy.y, rzw.x, rzw.y)));
+        rec.add(rxy);
+        rec.add(rzw);
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             zm[s] = n[s];
@@ -309,19 +281,21 @@ __device__ __forceinline__ void direct_march(const float *__restrict__ ip, const
             zp[s] = z2[s];
         }
     }
+    v[0] = rec.total();
+    if constexpr (SC) {
+        v[NV - 2] = spc[0].total();
+        v[NV - 1] = spc[1].total();
+    }
     if (!act) {
 #pragma unroll
         for (int t = 0; t < NV; ++t) v[t] = CompSum{};
+        an[0] = an[1] = CompSum{};
     }
     sk_reduce<NV>(v, buf, tot, 0);
-    if (k0 == 0) {
-        CompSum e[2];
-        if (act) { e[0].add(an[0]); e[1].add(an[1]); }
-        sk_reduce<2>(e, buf, tot, AN);
-    }
+    if (k0 == 0) sk_reduce<2>(an, buf, tot, AN);
     if (k1 == nz) {
         CompSum e[2];
-        if (act) { e[0].add(ca[0]); e[1].add(ca[1]); }
+        if (act) { add4(e[0], zm[0]); add4(e[1], zm[1]); }   // the last plane (cathode tally)
         sk_reduce<2>(e, buf, tot, CA);
     }
 }
