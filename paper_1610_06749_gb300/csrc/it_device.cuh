@@ -44,11 +44,23 @@ __device__ __forceinline__ double warp_strided_sum(const double *__restrict__ v,
 
 // FP32 sum that carries the rounding error of each addition (Knuth's
 // two-sum), so a sum of some hundred terms keeps about 46 bits: as good as
-// FP64 for terms that are FP32 products.  A sum that overflows or meets a
-// NaN is returned as it is.
+// FP64 for terms that are FP32 products.  Its terms are kept times 2^-32,
+// which costs nothing (the products with it are exact, in fused
+// multiply-adds), so that no sum of fewer than 2^32 finite terms overflows as
+// an FP64 one would not; terms below 2^-94 lose bits of less than 2^-117.  A
+// sum that meets an infinity or a NaN is returned as it is.
+constexpr float SUM_SCALE = 0x1p-32f;
+constexpr double SUM_UNSCALE = 0x1p32;
+
 struct CompSum {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float x) {
+    float hi = 0.f, lo = 0.f;   // times SUM_SCALE
+    __device__ __forceinline__ void term(float x) {
+        const float s = __fmaf_rn(x, SUM_SCALE, hi);
+        const float b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fmaf_rn(x, SUM_SCALE, -b)));
+        hi = s;
+    }
+    __device__ __forceinline__ void add(float x) {   // x scaled already
         const float s = __fadd_rn(hi, x);
         const float b = __fsub_rn(s, hi);
         lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
@@ -65,7 +77,7 @@ struct CompSum {
         hi = p;
     }
     __device__ __forceinline__ double value() const {
-        return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+        return (isfinite(hi) ? (double)hi + (double)lo : (double)hi) * SUM_UNSCALE;
     }
     __device__ __forceinline__ CompSum down(int o) const {
         CompSum r;
@@ -75,18 +87,18 @@ struct CompSum {
     }
 };
 
-__device__ __forceinline__ void add4(CompSum &c, float4 v) { c.add(v.x); c.add(v.y); c.add(v.z); c.add(v.w); }
+__device__ __forceinline__ void add4(CompSum &c, float4 v) { c.term(v.x); c.term(v.y); c.term(v.z); c.term(v.w); }
 
 // Two such sums side by side in paired-FP32 instructions (seven for two terms;
 // multiplications by -1 are exact, so every line is one rounding as above).
 struct CompSum2 {
     float2 hi = make_float2(0.f, 0.f), lo = make_float2(0.f, 0.f);
-    __device__ __forceinline__ void add(float2 x) {
-        const float2 neg = make_float2(-1.f, -1.f);
-        const float2 s = __fadd2_rn(hi, x);
+    __device__ __forceinline__ void term(float2 x) {
+        const float2 neg = make_float2(-1.f, -1.f), sc = make_float2(SUM_SCALE, SUM_SCALE);
+        const float2 s = __ffma2_rn(x, sc, hi);
         const float2 nb = __ffma2_rn(s, neg, hi);                      // hi - s
         const float2 eh = __ffma2_rn(__fadd2_rn(s, nb), neg, hi);      // hi - (s - b)
-        lo = __fadd2_rn(lo, __fadd2_rn(eh, __fadd2_rn(x, nb)));
+        lo = __fadd2_rn(lo, __fadd2_rn(eh, __ffma2_rn(x, sc, nb)));
         hi = s;
     }
     __device__ __forceinline__ CompSum total() const {

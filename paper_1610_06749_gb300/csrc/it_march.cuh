@@ -26,7 +26,7 @@ constexpr double DK_ALTERNATE = 115e6;
 // CompSum's counterpart for FP64 states: a plain FP64 sum
 struct PlainSum {
     double hi = 0.0;
-    __device__ __forceinline__ void add(double x) { hi += x; }
+    __device__ __forceinline__ void term(double x) { hi += x; }
     __device__ __forceinline__ void add(const PlainSum &o) { hi += o.hi; }
     __device__ __forceinline__ void scale(double w) { hi *= w; }
     __device__ __forceinline__ double value() const { return hi; }
@@ -142,13 +142,13 @@ __device__ __forceinline__ void simple_march(const T *__restrict__ ip, const T *
             if constexpr (SC) {
                 const T t = sk_mul(n[s], d);
                 w[s] = sk_fma(c.sc[s], t, w[s]);
-                v[NV - 2 + s].add(t);
+                v[NV - 2 + s].term(t);
             }
             if constexpr (!PERIODIC) {
-                if (sides > 0) v[1 + s].add(n[s]);
+                if (sides > 0) v[1 + s].term(n[s]);
             }
         }
-        v[0].add(rr);
+        v[0].term(rr);
         if (act) {
             op[base + q] = w[0];
             om[base + q] = w[1];
@@ -173,12 +173,12 @@ __device__ __forceinline__ void simple_march(const T *__restrict__ ip, const T *
     sk_reduce<NV>(v, buf, tot, 0);
     if (k0 == 0) {
         Sum e[2];
-        if (act) { e[0].add(first[0]); e[1].add(first[1]); }
+        if (act) { e[0].term(first[0]); e[1].term(first[1]); }
         sk_reduce<2>(e, buf, tot, AN);
     }
     if (k1 == nz) {
         Sum e[2];
-        if (act) { e[0].add(last[0]); e[1].add(last[1]); }
+        if (act) { e[0].term(last[0]); e[1].term(last[1]); }
         sk_reduce<2>(e, buf, tot, CA);
     }
 }
@@ -258,12 +258,12 @@ __device__ __forceinline__ void direct_march(const float *__restrict__ ip, const
             if constexpr (SC) {
                 float2 pxy, pzw;
                 w4[s] = add_sc4(w4[s], c.sc[s], n[s], dxy, dzw, pxy, pzw);
-                spc[s].add(pxy);
-                spc[s].add(pzw);
+                spc[s].term(pxy);
+                spc[s].term(pzw);
             }
             if constexpr (!PERIODIC) {
-                if (first) v[1 + s].add(n[s].x);
-                if (last) v[1 + s].add(n[s].w);
+                if (first) v[1 + s].term(n[s].x);
+                if (last) v[1 + s].term(n[s].w);
                 if (j == 0) add4(v[1 + s], n[s]);
                 if (j == ny - 1) add4(v[1 + s], n[s]);
             }
@@ -272,8 +272,8 @@ __device__ __forceinline__ void direct_march(const float *__restrict__ ip, const
 #pragma unroll
         for (int s = 0; s < 2; ++s)
             if (act) *reinterpret_cast<float4 *>((s ? om : op) + base + q) = w4[s];
-        rec.add(rxy);
-        rec.add(rzw);
+        rec.term(rxy);
+        rec.term(rzw);
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             zm[s] = n[s];

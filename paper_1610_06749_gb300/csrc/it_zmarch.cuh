@@ -98,7 +98,7 @@ struct RingSum {   // plain FP32
 template <>
 struct RingSum<true> {
     CompSum2 c;
-    __device__ __forceinline__ void add(float2 a, float2 b) { c.add(a); c.add(b); }
+    __device__ __forceinline__ void add(float2 a, float2 b) { c.term(a); c.term(b); }
     __device__ __forceinline__ double value() const { return c.total().value(); }
 };
 
@@ -340,7 +340,7 @@ step_zmarch_kernel(const __grid_constant__ ZmMaps maps, const float *__restrict_
         // the ring fills: summed in the march it holds registers and issue
         // slots that the march needs (384x320x128: 60.3 us, so 55.6)
         CompSum2 lat;   // n+ and n-
-        auto cell = [&](uint32_t e) { lat.add(make_float2(__ldg(inp + e), __ldg(inm + e))); };
+        auto cell = [&](uint32_t e) { lat.term(make_float2(__ldg(inp + e), __ldg(inm + e))); };
         Segs sg{g0, g1, nz, 0, 0, 0};
         while (sg.next()) {
             const uint32_t y0 = (uint32_t)(sg.t * zc.TY), n = (uint32_t)(sg.zb - sg.za);
@@ -365,10 +365,10 @@ step_zmarch_kernel(const __grid_constant__ ZmMaps maps, const float *__restrict_
                     }
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        lat.add(make_float2(P[u].x, M[u].x));
-                        lat.add(make_float2(P[u].y, M[u].y));
-                        lat.add(make_float2(P[u].z, M[u].z));
-                        lat.add(make_float2(P[u].w, M[u].w));
+                        lat.term(make_float2(P[u].x, M[u].x));
+                        lat.term(make_float2(P[u].y, M[u].y));
+                        lat.term(make_float2(P[u].z, M[u].z));
+                        lat.term(make_float2(P[u].w, M[u].w));
                     }
                 }
             }
