@@ -532,7 +532,8 @@ deposit_plane_kernel(const DepWindow *__restrict__ win, const double *__restrict
     __shared__ double stage[16][16];   // [track][8 column weights, 8 row weights]
     __shared__ double red[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int i0 = blockIdx.x * DEP_TILE, j0 = blockIdx.y * DEP_TILE;
+    const unsigned ntx = (unsigned)(nx + DEP_TILE - 1) / DEP_TILE;   // tiles in raster order: gridDim.y ends at 65535
+    const int i0 = (int)(blockIdx.x % ntx) * DEP_TILE, j0 = (int)(blockIdx.x / ntx) * DEP_TILE;
     const int tnx = min(DEP_TILE, nx - i0), tny = min(DEP_TILE, ny - j0);
     const bool inside = (tid % DEP_TILE) < tnx && (tid / DEP_TILE) < tny;
     const int i = i0 + (tid % DEP_TILE), j = j0 + (tid / DEP_TILE);
@@ -594,7 +595,7 @@ deposit_plane_kernel(const DepWindow *__restrict__ win, const double *__restrict
     if (inside) plane[(size_t)j * nx + i] = v;
     double r[1] = {inside ? v : 0.0};
     block_sum<1>(r, red);
-    if (tid == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = r[0];
+    if (tid == 0) part[blockIdx.x] = r[0];
 }
 
 // n += plane on every z plane.  Thread = V adjacent columns (float4 when the
@@ -669,11 +670,10 @@ int launch_deposit(it_ctx *c, int64_t n, cudaStream_t s) {
                                                                      1.0 / c->p.W_eV, c->d_wx, c->d_wy, win);
     IT_CK(cudaGetLastError());
     const long long pn = (long long)nx * ny;
-    dim3 gp((nx + DEP_TILE - 1) / DEP_TILE, (ny + DEP_TILE - 1) / DEP_TILE);
-    const size_t nparts = (size_t)gp.x * gp.y;
+    const size_t nparts = (size_t)((nx + DEP_TILE - 1) / DEP_TILE) * ((ny + DEP_TILE - 1) / DEP_TILE);
     // the tile sums go after the plane in the same scratch buffer
     double *part = c->d_plane + pn;
-    deposit_plane_kernel<<<gp, DEP_TILE * DEP_TILE, 0, s>>>(win, c->d_wx, c->d_wy, n, nx, ny, periodic ? 1 : 0,
+    deposit_plane_kernel<<<(unsigned)nparts, DEP_TILE * DEP_TILE, 0, s>>>(win, c->d_wx, c->d_wy, n, nx, ny, periodic ? 1 : 0,
                                                             1.0 / (c->dx * c->dx), c->d_plane, part);
     IT_CK(cudaGetLastError());
     const unsigned kchunks = (unsigned)((c->g.nz + DEP_KCHUNK - 1) / DEP_KCHUNK);
