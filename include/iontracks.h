@@ -328,9 +328,11 @@ int it_device_state(it_ctx *ctx, void **plus, void **minus, void **stream);
  * launch shape: rows per tile (a divisor of ny; for IT_KERNEL_ZMARCH2 it is
  * fixed at threads / (nx/4), 0 or that value), resident CTAs per SM (1: 16
  * warps, 2: 8 warps each) and ring depth (3..16); 0 leaves a value to the
- * built-in rule.  With IT_KERNEL_ZMARCH2, it_step runs steps in pairs and an
- * odd last step on the simple kernel.  Only before the first step (IT_ESTATE
- * otherwise).  IT_EINVAL if the shape does not fit the grid. */
+ * built-in rule.  With IT_KERNEL_AUTO a shape that is given is the ring's, as
+ * with IT_KERNEL_ZMARCH; with none, small grids march without a ring.  With
+ * IT_KERNEL_ZMARCH2, it_step runs steps in pairs and an odd last step on the
+ * simple kernel.  Only before the first step (IT_ESTATE otherwise).  IT_EINVAL
+ * if the shape does not fit the grid. */
 int it_set_launch(it_ctx *ctx, int kernel, int tile_rows, int ctas_per_sm, int stages);
 
 /* As it_set_launch, plus the grid of the z-march kernel: 0 = one CTA per

@@ -325,7 +325,11 @@ int set_launch(it_ctx *c, int kernel, int tile_rows, int ctas_per_sm, int stages
     } else {
         return fail(IT_EINVAL, "bad kernel");
     }
-    c->direct = c->kernel == IT_KERNEL_ZMARCH && ((kernel == IT_KERNEL_AUTO && direct_wins(c)) || tile_rows < 0);
+    // the automatic kernel may do without the ring, but not where the caller
+    // has given any of the ring's shape
+    const bool shape = tile_rows > 0 || ctas_per_sm > 0 || stages > 0 || grid != 0;
+    c->direct = c->kernel == IT_KERNEL_ZMARCH &&
+                ((kernel == IT_KERNEL_AUTO && !shape && direct_wins(c)) || tile_rows < 0);
     const int n = slots_needed(c);
     if (n != c->nslots) {
         double *ns = nullptr;
