@@ -70,6 +70,7 @@ extern "C" {
 #define IT_KERNEL_SIMPLE 1   /* one thread per column of cells, global loads (any grid and type) */
 #define IT_KERNEL_ZMARCH 2   /* marches up z, float4 segments (FP32, nx % 4 == 0): TMA-staged z-planes in
                                 shared memory, or (IT_KERNEL_AUTO, small grids) straight from L1/L2 */
+#define IT_NO_RING       (-1) /* tile_rows of IT_KERNEL_ZMARCH straight from L1/L2 (it_set_launch, it_get_launch) */
 #define IT_KERNEL_ZMARCH2 3  /* as IT_KERNEL_ZMARCH, two time steps per launch (temporal blocking
                                 of depth 2; nx/4 must divide 256 or 512 threads); densities are
                                 bitwise those of two single steps */
@@ -329,10 +330,11 @@ int it_device_state(it_ctx *ctx, void **plus, void **minus, void **stream);
  * fixed at threads / (nx/4), 0 or that value), resident CTAs per SM (1: 16
  * warps, 2: 8 warps each) and ring depth (3..16); 0 leaves a value to the
  * built-in rule.  With IT_KERNEL_AUTO a shape that is given is the ring's, as
- * with IT_KERNEL_ZMARCH; with none, small grids march without a ring.  With
- * IT_KERNEL_ZMARCH2, it_step runs steps in pairs and an odd last step on the
- * simple kernel.  Only before the first step (IT_ESTATE otherwise).  IT_EINVAL
- * if the shape does not fit the grid. */
+ * with IT_KERNEL_ZMARCH; with none, small grids march without a ring.  Rows of
+ * IT_NO_RING ask for that march by name.  With IT_KERNEL_ZMARCH2, it_step runs
+ * steps in pairs and an odd last step on the simple kernel.  Only before the
+ * first step (IT_ESTATE otherwise).  IT_EINVAL if the shape does not fit the
+ * grid. */
 int it_set_launch(it_ctx *ctx, int kernel, int tile_rows, int ctas_per_sm, int stages);
 
 /* As it_set_launch, plus the grid of the z-march kernel: 0 = one CTA per
@@ -354,7 +356,9 @@ int it_autotune(it_ctx *ctx, int trial_steps, int flags, double *best_us);
 
 /* Report the kernel in use, its launch shape and its CTA count (for
  * IT_KERNEL_ZMARCH2, the CTAs of its two-step launches; IT_KERNEL_ZMARCH
- * without a shared-memory ring reports 0 rows, 0 CTAs per SM, 0 stages). */
+ * without a shared-memory ring reports IT_NO_RING rows, 0 CTAs per SM and 0
+ * stages).  Given to it_set_launch on another context, what is reported
+ * selects the same kernel and shape. */
 int it_get_launch(it_ctx *ctx, int *kernel, int *tile_rows, int *ctas_per_sm, int *stages, int *ctas);
 
 /* ---------------------------------------------------------------------------

@@ -311,7 +311,7 @@ int set_launch(it_ctx *c, int kernel, int tile_rows, int ctas_per_sm, int stages
     if (kernel == IT_KERNEL_SIMPLE) {
         c->kernel = IT_KERNEL_SIMPLE;
     } else if (kernel == IT_KERNEL_ZMARCH2) {
-        int rc = zmarch2_setup(c, tile_rows, ctas_per_sm, stages, grid);
+        int rc = zmarch2_setup(c, std::max(tile_rows, 0), ctas_per_sm, stages, grid);
         if (rc) return rc;
         c->kernel = IT_KERNEL_ZMARCH2;
     } else if (kernel == IT_KERNEL_ZMARCH || kernel == IT_KERNEL_AUTO) {
@@ -329,7 +329,7 @@ int set_launch(it_ctx *c, int kernel, int tile_rows, int ctas_per_sm, int stages
     // has given any of the ring's shape
     const bool shape = tile_rows > 0 || ctas_per_sm > 0 || stages > 0 || grid != 0;
     c->direct = c->kernel == IT_KERNEL_ZMARCH &&
-                ((kernel == IT_KERNEL_AUTO && !shape && direct_wins(c)) || tile_rows < 0);
+                ((kernel == IT_KERNEL_AUTO && !shape && direct_wins(c)) || tile_rows == IT_NO_RING);
     const int n = slots_needed(c);
     if (n != c->nslots) {
         double *ns = nullptr;
@@ -885,7 +885,7 @@ int it_device_state(it_ctx *c, void **plus, void **minus, void **stream) {
 int it_set_launch_ex(it_ctx *c, int kernel, int tile_rows, int ctas_per_sm, int stages, int grid) {
     if (!c) return fail(IT_EINVAL, "ctx is NULL");
     if (c->steps != 0) return fail(IT_ESTATE, "launch shape can only change before the first step");
-    return set_launch(c, kernel, std::max(tile_rows, 0), ctas_per_sm, stages, grid);
+    return set_launch(c, kernel, tile_rows == IT_NO_RING ? IT_NO_RING : std::max(tile_rows, 0), ctas_per_sm, stages, grid);
 }
 
 int it_set_launch(it_ctx *c, int kernel, int tile_rows, int ctas_per_sm, int stages) {
@@ -896,7 +896,7 @@ int it_get_launch(it_ctx *c, int *kernel, int *tile_rows, int *ctas_per_sm, int 
     if (!c) return fail(IT_EINVAL, "ctx is NULL");
     const bool zm = c->kernel == IT_KERNEL_ZMARCH && !c->direct, zm2 = c->kernel == IT_KERNEL_ZMARCH2;
     if (kernel) *kernel = c->kernel;
-    if (tile_rows) *tile_rows = zm ? c->zm.TY : zm2 ? c->zm2.TY : 0;
+    if (tile_rows) *tile_rows = zm ? c->zm.TY : zm2 ? c->zm2.TY : c->direct ? IT_NO_RING : 0;
     if (ctas_per_sm) *ctas_per_sm = zm ? c->zm.ctas_per_sm : zm2 ? c->zm2.ctas_per_sm : 0;
     if (stages) *stages = zm ? c->zm.S : zm2 ? c->zm2.S : 0;
     if (ctas) *ctas = zm2 ? c->zm2.grid : zm ? c->zm_grid : c->direct ? direct_grid(c) : c->nslots;

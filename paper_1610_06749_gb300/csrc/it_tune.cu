@@ -32,7 +32,7 @@ std::vector<Shape> candidates(const it_ctx *c) {
     v.push_back({IT_KERNEL_SIMPLE, 0, 0, 0, 0});
     const int nx = c->g.nx, ny = c->g.ny;
     if (c->prec != IT_FP32 || nx % 4 != 0 || (nx > 256 && !row_piece(nx))) return v;
-    v.push_back({IT_KERNEL_ZMARCH, -1, 0, 0, 0});   // the march without the ring
+    v.push_back({IT_KERNEL_ZMARCH, IT_NO_RING, 0, 0, 0});   // the march without the ring
     const int ncol4 = nx / 4;
     for (int cps = 1; cps <= 2; ++cps) {
         const int threads = cps == 1 ? 512 : 256;
