@@ -348,10 +348,10 @@ int it_set_launch_ex(it_ctx *ctx, int kernel, int tile_rows, int ctas_per_sm, in
  * 2 untimed and trial_steps timed steps (rounded up to even, 8 if <= 0) on a
  * copy of the state, which is restored afterwards: the densities, tallies
  * and step counter are unchanged on return.  Only before the first step
- * (IT_ESTATE otherwise).  The choice is cached per grid shape, precision and
- * lateral boundary for the life of the process (flags & 1 forces a new
- * search).  *best_us (may be NULL) receives the chosen shape's time per
- * step in microseconds. */
+ * (IT_ESTATE otherwise).  The choice is cached per device, grid shape,
+ * precision, lateral boundary and space-charge term for the life of the
+ * process (flags & 1 forces a new search).  *best_us (may be NULL) receives
+ * the chosen shape's time per step in microseconds. */
 int it_autotune(it_ctx *ctx, int trial_steps, int flags, double *best_us);
 
 /* Report the kernel in use, its launch shape and its CTA count (for

@@ -23,7 +23,10 @@ struct Shape {
     int kernel, ty, cps, s, grid;
 };
 
-using Key = std::tuple<int, int, int, int, int>;
+// what selects the kernels that are timed: the device, the grid, the type, the
+// lateral faces and the space-charge term (its staged instances have no
+// producer warp and other registers)
+using Key = std::tuple<int, int, int, int, int, int, int>;
 std::map<Key, Shape> g_cache;
 std::mutex g_cache_mu;
 
@@ -116,7 +119,9 @@ extern "C" int it_autotune(it_ctx *c, int trial_steps, int flags, double *best_u
     }
     int trial = trial_steps > 0 ? trial_steps : 8;
     trial += trial & 1;
-    const Key key{c->g.nx, c->g.ny, c->g.nz, c->prec, c->p.lateral_bc};
+    int dev = 0;
+    IT_CK(cudaGetDevice(&dev));
+    const Key key{dev, c->g.nx, c->g.ny, c->g.nz, c->prec, c->p.lateral_bc, c->p.space_charge};
     if (!(flags & 1)) {
         std::lock_guard<std::mutex> lk(g_cache_mu);
         auto it = g_cache.find(key);
