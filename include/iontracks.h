@@ -476,8 +476,13 @@ int it_mlp_set_data(it_mlp *net, int64_t n, const double *x, const double *y);
 /* `epochs` passes of Adam (beta 0.9 / 0.999, eps 1e-8, rate lr) over
  * mini-batches of `batch` samples in a SplitMix64 Fisher-Yates order from
  * `seed`, a different order for every member (ensemble diversity).  loss_per_epoch (may be NULL)
- * receives the mean over batches and members of the batch loss. */
+ * receives the mean over batches and members of the batch loss.  Calls of
+ * eight or more mini-batches replay one recorded step; where it cannot be
+ * recorded, the steps are launched one by one with the same results. */
 int it_mlp_train(it_mlp *net, int32_t epochs, int32_t batch, double lr, uint64_t seed, double *loss_per_epoch);
+/* Test hook: with on = 1 it_mlp_train cannot record its step (as if memory for
+ * the graph had run out); on = 0 restores it. */
+int it_test_refuse_recording(it_mlp *net, int on);
 /* Loss and gradient of every member on n <= max_batch samples (no update):
  * grads: members x IT_MLP_PARAMS floats, loss: members doubles.  The next
  * it_mlp_adam_step applies this gradient. */

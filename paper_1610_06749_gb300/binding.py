@@ -131,6 +131,7 @@ def lib():
             "it_mlp_fit_normalization": (I, [P, I64, DP]),
             "it_mlp_set_data": (I, [P, I64, DP, DP]),
             "it_mlp_train": (I, [P, ctypes.c_int32, ctypes.c_int32, D, ctypes.c_uint64, DP]),
+            "it_test_refuse_recording": (I, [P, I]),
             "it_mlp_loss_grad": (I, [P, I64, DP, DP, ctypes.POINTER(ctypes.c_float), DP]),
             "it_mlp_adam_step": (I, [P, D]),
             "it_mlp_predict": (I, [P, I64, DP, DP, DP, DP]),
@@ -442,6 +443,10 @@ def it_mlp_train(h, epochs, batch, lr, seed):
     loss = np.zeros(max(int(epochs), 1))
     _check(lib().it_mlp_train(h, int(epochs), int(batch), float(lr), ctypes.c_uint64(seed & (2 ** 64 - 1)), _dp(loss)))
     return loss[:int(epochs)]
+
+
+def it_test_refuse_recording(h, on: bool):
+    _check(lib().it_test_refuse_recording(h, 1 if on else 0))
 
 
 def it_mlp_loss_grad(h, members, x, y):
