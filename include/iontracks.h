@@ -422,6 +422,17 @@ int it_batch_set_chunk(it_batch *b, int64_t cells_per_block);
  * shape only changes the work split, not any cell's arithmetic. */
 int it_batch_autotune(it_batch *b, int32_t trial_steps, double *best_us);
 
+/* The launch shape of the next step for the simulations still running: 2 or 1
+ * float4 per thread on the TMA-staged kernel and the CTAs per SM its z splits
+ * aim at, or 0 and 0 for the march straight from L1/L2 (either pointer may be
+ * NULL).  Simulations with nx % 4 != 0 (and, staged, nx > 256) have kernels of
+ * their own in every shape. */
+int it_batch_get_launch(it_batch *b, int *float4_per_thread, int *ctas_per_sm);
+/* Test hook: run every step in the given shape (ctas_per_sm 1 to 64; with 0
+ * float4 it divides the chunk of planes); -1 float4 per thread frees the
+ * choice again. */
+int it_test_batch_launch(it_batch *b, int float4_per_thread, int ctas_per_sm);
+
 /* Run every simulation until its in-domain charge / released < tol or it
  * has taken max_steps steps, checked every check_every steps (rounded up to
  * even).  *launches (may be NULL) receives the number of step launches.

@@ -119,6 +119,8 @@ def lib():
             "it_batch_deposit_tracks": (I, [P, ctypes.c_int32, I64, DP, DP, DP]),
             "it_batch_set_chunk": (I, [P, I64]),
             "it_batch_autotune": (I, [P, ctypes.c_int32, ctypes.POINTER(D)]),
+            "it_batch_get_launch": (I, [P, IP, IP]),
+            "it_test_batch_launch": (I, [P, I, I]),
             "it_batch_set_pulses": (I, [P, ctypes.c_int32, ctypes.c_int32, I64]),
             "it_batch_run": (I, [P, D, I64, I64, I64P]),
             "it_batch_tallies": (I, [P, ctypes.c_int32, ctypes.POINTER(it_tallies_t)]),
@@ -378,6 +380,16 @@ def it_batch_autotune(h, trial_steps=8) -> float:
     return us.value
 
 
+def it_batch_get_launch(h):
+    a, b = ctypes.c_int(), ctypes.c_int()
+    _check(lib().it_batch_get_launch(h, ctypes.byref(a), ctypes.byref(b)))
+    return {"float4_per_thread": a.value, "ctas_per_sm": b.value}
+
+
+def it_test_batch_launch(h, float4_per_thread, ctas_per_sm=1):
+    _check(lib().it_test_batch_launch(h, int(float4_per_thread), int(ctas_per_sm)))
+
+
 def it_batch_run(h, tol=1e-6, max_steps=10_000_000, check_every=64) -> int:
     n = ctypes.c_int64()
     _check(lib().it_batch_run(h, float(tol), int(max_steps), int(check_every), ctypes.byref(n)))
@@ -536,6 +548,9 @@ class Batch:
 
     def autotune(self, trial_steps=8) -> float:
         return it_batch_autotune(self.h, trial_steps)
+
+    def launch(self):
+        return it_batch_get_launch(self.h)
 
     def run(self, tol=1e-6, max_steps=10_000_000, check_every=64):
         return it_batch_run(self.h, tol, max_steps, check_every)

@@ -586,6 +586,8 @@ struct it_batch {
     bool tuned;                       // the autotuner's choice, for the simulations it was made for
     BatchShape tuned_shape;
     int tuned_active;
+    bool forced;                      // test hook: forced_shape whatever is active
+    BatchShape forced_shape;
     double cal[3];                    // measured over fitted time of the direct march and the TMA kernels
     double *d_tal;                    // one simulation's monitor blocks, then its gathered tallies
     // per simulation
@@ -722,6 +724,7 @@ BatchShape choose_shape(const it_batch *b, int sms) {
             ++active;
             any_tma = any_tma || b->tma_ok[s];
         }
+    if (b->forced) return b->forced_shape;
     if (b->tuned && active == b->tuned_active) return b->tuned_shape;
     BatchShape best{0, 1};
     double best_us = shape_us(b, best, sms) * b->cal[0];
@@ -1384,6 +1387,24 @@ int it_batch_autotune(it_batch *b, int32_t trial_steps, double *best_us) {
     if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
     if (rc) return rc;
     if (best_us) *best_us = best;
+    return IT_OK;
+}
+
+int it_batch_get_launch(it_batch *b, int *float4_per_thread, int *ctas_per_sm) {
+    if (!b) return bfail(IT_EINVAL, "batch is NULL");
+    const BatchShape sh = choose_shape(b, sm_count());
+    if (float4_per_thread) *float4_per_thread = sh.tma;
+    if (ctas_per_sm) *ctas_per_sm = sh.tma ? sh.cps : 0;
+    return IT_OK;
+}
+
+int it_test_batch_launch(it_batch *b, int float4_per_thread, int ctas_per_sm) {
+    if (!b) return bfail(IT_EINVAL, "batch is NULL");
+    if (float4_per_thread < -1 || float4_per_thread > 2 || (float4_per_thread >= 0 && (ctas_per_sm < 1 || ctas_per_sm > 64)))
+        return bfail(IT_EINVAL, "0 to 2 float4 per thread and 1 to 64 CTAs per SM (-1: the choice is free)");
+    b->forced = float4_per_thread >= 0;
+    if (b->forced) b->forced_shape = BatchShape{float4_per_thread, ctas_per_sm};
+    b->tab_dirty = true;
     return IT_OK;
 }
 
