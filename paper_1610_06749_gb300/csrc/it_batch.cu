@@ -78,7 +78,7 @@ step_batched_march_kernel(const BatchSim *__restrict__ sims, const MarchEntry *_
     const long long off = S.off;
     if (threadIdx.x < 9) tot[threadIdx.x] = 0.0;
     if constexpr (V == 4)
-        direct_march<uint32_t, PERIODIC, SC>(ip_all + off, im_all + off, op_all + off, om_all + off, S.nx, S.ny, S.nz,
+        direct_march<uint32_t, PERIODIC, SC, false>(ip_all + off, im_all + off, op_all + off, om_all + off, S.nx, S.ny, S.nz,
                                              E.q0, E.k0, E.k1, c, buf, tot);
     else
         simple_march<float, uint32_t, PERIODIC, SC>(ip_all + off, im_all + off, op_all + off, om_all + off, S.nx, S.ny,

@@ -77,6 +77,11 @@ struct ZmConf {
     int pair;                // a thread's items are vertically adjacent rows in pairs
 };
 
+// Widths whose FP32 tallies are summed as closely as FP64 would: those that
+// only the simple kernel, whose sums are that close, took before the marches
+// over float4 segments reached them.
+inline bool exact_sums(int nx) { return nx > 256 && nx % 256 != 0; }
+
 // Launch shape of the two-steps-per-launch z-march kernel: tiles of TY
 // full-width rows, one float4 item per thread of the tile (TY * nx/4 ==
 // threads); a ring slot holds TY + 4 rows of both species (two halo rows

@@ -164,7 +164,7 @@ int launch_step_simple_raw_f32(const float *ip, const float *im, float *op, floa
 // TMA-staged kernel; on grids that stream from HBM the ring wins.
 // 128x128x200 9.9-12.4 us per step against 19.6 with the ring, 256x256x100
 // 22.8 against a fitted 24.6; 256x256x400 86 against 70.
-template <typename Idx, bool PERIODIC, bool SC>
+template <typename Idx, bool PERIODIC, bool SC, bool EXACT>
 __global__ void __launch_bounds__(SK_THREADS, DK_BLOCKS)
 step_direct_kernel(const float *__restrict__ ip, const float *__restrict__ im, float *__restrict__ op,
                    float *__restrict__ om, int nx, int ny, int nz, unsigned npb, unsigned nchunk, int rev,
@@ -180,7 +180,7 @@ step_direct_kernel(const float *__restrict__ ip, const float *__restrict__ im, f
         const unsigned long long u = rev ? units - 1 - q : q;
         const unsigned pb = (unsigned)(u % npb), ch = (unsigned)(u / npb);
         const int k0 = (int)((long long)nz * ch / nchunk), k1 = (int)((long long)nz * (ch + 1) / nchunk);
-        direct_march<Idx, PERIODIC, SC>(ip, im, op, om, nx, ny, nz, (Idx)pb * SK_THREADS, k0, k1, c, buf, tot);
+        direct_march<Idx, PERIODIC, SC, EXACT>(ip, im, op, om, nx, ny, nz, (Idx)pb * SK_THREADS, k0, k1, c, buf, tot);
     }
     __syncthreads();
     if (tid < 9) sk_slot<PERIODIC, SC, NV>(tot, c, slots + (size_t)blockIdx.x * NT, tid, 1);
@@ -236,10 +236,15 @@ int launch_step_direct(it_ctx *c, cudaStream_t s) {
     float *op = (float *)c->n[nxt][0], *om = (float *)c->n[nxt][1];
     auto go = [&](auto *k) { k<<<h.grid, SK_THREADS, 0, s>>>(ip, im, op, om, nx, ny, nz, h.npb, h.nchunk, rev, c->cf, c->d_slots); };
     // 32-bit element offsets: the z-march family takes grids below 2^32 cells
+    const bool exact = exact_sums(nx);
     if (c->p.lateral_bc == IT_PERIODIC)
-        c->cf.sc_on ? go(step_direct_kernel<uint32_t, true, true>) : go(step_direct_kernel<uint32_t, true, false>);
+        !c->cf.sc_on ? go(step_direct_kernel<uint32_t, true, false, true>)
+        : exact      ? go(step_direct_kernel<uint32_t, true, true, true>)
+                     : go(step_direct_kernel<uint32_t, true, true, false>);
     else
-        c->cf.sc_on ? go(step_direct_kernel<uint32_t, false, true>) : go(step_direct_kernel<uint32_t, false, false>);
+        !c->cf.sc_on ? go(step_direct_kernel<uint32_t, false, false, true>)
+        : exact      ? go(step_direct_kernel<uint32_t, false, true, true>)
+                     : go(step_direct_kernel<uint32_t, false, true, false>);
     IT_CK(cudaGetLastError());
     c->cur = nxt;
     return IT_OK;

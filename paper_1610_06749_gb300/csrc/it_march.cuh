@@ -183,13 +183,34 @@ __device__ __forceinline__ void simple_march(const T *__restrict__ ip, const T *
     }
 }
 
+// One thread's sum of a tally over its float4 segments.
+template <bool EXACT>
+struct QuadSum {   // four cells in plain FP32, then compensated
+    CompSum c;
+    __device__ __forceinline__ void add(float2 a, float2 b) {
+        c.term(__fadd_rn(__fadd_rn(a.x, a.y), __fadd_rn(b.x, b.y)));
+    }
+    __device__ __forceinline__ CompSum total() const { return c; }
+};
+template <>
+struct QuadSum<true> {   // every cell compensated
+    CompSum2 c;
+    __device__ __forceinline__ void add(float2 a, float2 b) {
+        c.term(a);
+        c.term(b);
+    }
+    __device__ __forceinline__ CompSum total() const { return c.total(); }
+};
+
 // The same with a float4 x-segment per thread (nx % 4 == 0), segment q0 + tid
 // (step_direct_kernel).  Every cell's terms enter compensated sums, so the
 // tallies are as close as the simple kernel's; in paired instructions that
 // costs nothing against four cells added in FP32 first (128x128x200 9.8 us per
-// step both ways) but with space charge, where there are three such sums
-// (384x320x128: 54.3 us, 53.2 with the four cells in FP32).
-template <typename Idx, bool PERIODIC, bool SC, class C>
+// step both ways).  With space charge there are three such sums and it does
+// (384x320x128 54.5 us against 53.4, 128x128x200 12.2 against 11.4, 256x256x100
+// 24.6 against 23.4): there only EXACT instances sum so, for the widths whose
+// tallies the simple kernel would otherwise sum (exact_sums).
+template <typename Idx, bool PERIODIC, bool SC, bool EXACT, class C>
 __device__ __forceinline__ void direct_march(const float *__restrict__ ip, const float *__restrict__ im,
                                              float *__restrict__ op, float *__restrict__ om, int nx, int ny, int nz,
                                              Idx q0, int k0, int k1, const C &c, CompSum (*buf)[SK_THREADS],
@@ -211,7 +232,7 @@ __device__ __forceinline__ void direct_march(const float *__restrict__ ip, const
     const bool el = lane == 0 || first, er = lane == 31 || last || q4 + 1 >= plane4;
     const Idx ql = first ? q + (Idx)(nx - 1) : q - 1, qr = last ? q - (Idx)(nx - 4) : q + 4;
     CompSum v[NV];
-    CompSum2 rec, spc[2];   // recombination, space charge
+    QuadSum<!SC || EXACT> rec, spc[2];   // recombination, space charge
     Idx base = (Idx)k0 * plane;
     auto ld = [&](const float *f, Idx e) { return __ldg(reinterpret_cast<const float4 *>(f + e)); };
     float4 zm[2], n[2], zp[2];
@@ -258,8 +279,7 @@ __device__ __forceinline__ void direct_march(const float *__restrict__ ip, const
             if constexpr (SC) {
                 float2 pxy, pzw;
                 w4[s] = add_sc4(w4[s], c.sc[s], n[s], dxy, dzw, pxy, pzw);
-                spc[s].term(pxy);
-                spc[s].term(pzw);
+                spc[s].add(pxy, pzw);
             }
             if constexpr (!PERIODIC) {
                 if (first) v[1 + s].term(n[s].x);
@@ -272,8 +292,7 @@ __device__ __forceinline__ void direct_march(const float *__restrict__ ip, const
 #pragma unroll
         for (int s = 0; s < 2; ++s)
             if (act) *reinterpret_cast<float4 *>((s ? om : op) + base + q) = w4[s];
-        rec.term(rxy);
-        rec.term(rzw);
+        rec.add(rxy, rzw);
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             zm[s] = n[s];

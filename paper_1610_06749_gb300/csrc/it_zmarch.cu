@@ -110,9 +110,6 @@ int encode_bf16_sw128(CUtensorMap *m, const void *base, long long K, long long r
 
 static int align32f(int floats) { return (floats + 31) / 32 * 32; }   // 128-byte multiple of floats
 
-// widths whose tallies are summed as closely as FP64 would (EXACT)
-static bool zm_exact(int nx) { return nx > 256 && nx % 256 != 0; }
-
 static int ipt_of(const it_ctx *c, int TY, int nw) { return ((c->g.nx / 4) * TY + nw * 32 - 1) / (nw * 32); }
 
 static int sm_count() {
@@ -233,7 +230,7 @@ int zmarch_setup(it_ctx *c, int want_ty, int want_cps, int want_s, int want_grid
     const size_t budget = (size_t)(220 * 1024) / cps;
     const bool per = c->p.lateral_bc == IT_PERIODIC;
     const int ipt = ipt_of(c, TY, nw);
-    const bool sc = c->p.space_charge != 0, exact = zm_exact(nx);
+    const bool sc = c->p.space_charge != 0, exact = exact_sums(nx);
     z.pair = zm_pairs(c, TY, nw);
     // ring depth: with a producer the smallest (of 4 and more) that keeps
     // 64 KB per SM in flight beyond the two planes in use; deeper rings only
@@ -314,7 +311,7 @@ int launch_step_zmarch(it_ctx *c, cudaStream_t s) {
     const int nw = z.threads / 32;
     const int ipt = ipt_of(c, z.TY, nw);
     const int nx = c->g.nx, ny = c->g.ny, nz = c->g.nz;
-    const bool sc = c->p.space_charge != 0, exact = zm_exact(nx);
+    const bool sc = c->p.space_charge != 0, exact = exact_sums(nx);
     const bool down = cur != c->base;   // alternate steps, alternate directions
     auto *launch = exact ? zm_launch_shape<true> : zm_launch_shape<false>;
     launch(per, ipt, nw, sc, down, c->zm_grid, maps, ip, im, op, om, nx, ny, nz, z, c->cf, c->d_slots, c->d_err, s);

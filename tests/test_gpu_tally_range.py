@@ -2,7 +2,8 @@
 or a thread sums add up to more than FP32 holds (3.4e38), while every product
 and the 64-bit sum are finite.  One step's tallies against FP64 sums of the
 FP32 products, to 1e-12 of the sum of their magnitudes (as the simple kernel's
-edge test asks of ordinary states)."""
+edge test asks of ordinary states).  With space charge the march without a ring
+adds four cells of a narrow section in FP32 first, two roundings deep: 2^-23."""
 import numpy as np
 import pytest
 
@@ -41,12 +42,12 @@ def test_sums_beyond_fp32(shape, kernel, sc):
         g.set_density(n[0], n[1])
         g.step(1)
         t = g.tallies()
-    vol = dx ** 3
+    vol, tol = dx ** 3, 2.0 ** -23 if sc and kernel == B.IT_KERNEL_AUTO else 1e-12
     want = rr.astype(np.float64).sum() * float(f(ALPHA * dt)) * vol
-    assert abs(t.recombined - want) <= 1e-12 * want
+    assert abs(t.recombined - want) <= tol * want
     for s in range(2):
         if sc:
             k = float(f(-(1.0 if s == 0 else -1.0) * dt * MU[s] * Q_OVER_EPS0)) * vol
             q = (n[s] * (n[0] - n[1])).astype(np.float64)
-            assert abs(t.space_charge[s] - q.sum() * k) <= 1e-12 * np.abs(q).sum() * abs(k)
+            assert abs(t.space_charge[s] - q.sum() * k) <= tol * np.abs(q).sum() * abs(k)
         assert np.isfinite(t.in_domain[s]) and np.isfinite(t.collected_anode[s])
