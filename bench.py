@@ -101,11 +101,11 @@ def hbm_peak():
 
 
 def kernel_sha():
-    """Hash of the sources of the step kernel's device code: it_zmarch.cu,
+    """Hash of the sources of the step kernel's device code: it_zmarch.cuh,
     it_tma.cuh, it_device.cuh and the device-side types of it_internal.cuh
     (the text before the host context struct, which the kernel never sees)."""
     h = hashlib.sha256()
-    for name in ("it_zmarch.cu", "it_tma.cuh", "it_device.cuh", "it_internal.cuh"):
+    for name in ("it_zmarch.cuh", "it_tma.cuh", "it_device.cuh", "it_internal.cuh"):
         with open(os.path.join(ROOT, "paper_1610_06749_gb300", "csrc", name), "rb") as f:
             text = f.read()
         if name == "it_internal.cuh":

@@ -68,7 +68,6 @@ struct ZmConf {
     int reg_top, reg_main, reg_bot;   // float offsets of the halo/main rows in a block
     int blk;          // floats per (species, x-box) block, 128-byte multiple
     int slot;         // floats per slot = 2 * nbx * blk
-    unsigned tx_bytes;   // bytes TMA delivers per slot
     size_t smem;      // dynamic shared memory per CTA
     int threads;      // 256
     int ctas_per_sm;

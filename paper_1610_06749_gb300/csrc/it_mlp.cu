@@ -198,9 +198,6 @@ __global__ void to_bf16_kernel(const float *__restrict__ x, __nv_bfloat16 *__res
         y[i] = __float2bfloat16_rn(x[i]);
 }
 
-// normalised bf16 inputs of a batch for every member:
-// A0[z][m][j] = hi and A0[z][m][6 + j] = lo of (x[idx[z][m]][j] - mean[j]) / std[j], yb[z][m] = y[idx[z][m]]
-// (idx == NULL: sample m for every member)
 // Epilogues of the tensor-core products (it_tc.cuh), called by a whole warp
 // for its 32 x 16 block: lane holds row mw + lane, columns n0 .. n0+15.  Every
 // global access goes through the warp's shared-memory scratch, so that
@@ -591,6 +588,9 @@ adam_pack_kernel(const AdamArgs a, __nv_bfloat16 *__restrict__ w, __nv_bfloat16 
     }
 }
 
+// normalised bf16 inputs of a batch for every member:
+// A0[z][m][j] = hi and A0[z][m][6 + j] = lo of (x[idx[z][m]][j] - mean[j]) / std[j], yb[z][m] = y[idx[z][m]]
+// (idx == NULL: sample m for every member)
 __global__ void gather_inputs_kernel(const float *__restrict__ X, const float *__restrict__ Y,
                                      const int *__restrict__ idx, long long istride, int *__restrict__ count,
                                      int B, int members, int bmax, const float *__restrict__ mean, const float *__restrict__ inv_std,
@@ -629,7 +629,6 @@ struct it_mlp {
     float *dZ[2];
     __nv_bfloat16 *dZb[2];
     float *fhat, *dz, *yb;
-    int *idx;
     double *loss;
     // tensor-core operands: W2..W4 as [member][layer][out][in] and
     // [member][layer][in][out], A1..A3 transposed and the bf16 error signal
@@ -670,7 +669,7 @@ void mlp_free(it_mlp *n) {
     cudaFree(n->mean); cudaFree(n->inv_std); cudaFree(n->A0);
     for (int l = 0; l < 4; ++l) { cudaFree(n->Z[l]); cudaFree(n->Act[l]); }
     for (int q = 0; q < 2; ++q) { cudaFree(n->dZ[q]); cudaFree(n->dZb[q]); }
-    cudaFree(n->fhat); cudaFree(n->dz); cudaFree(n->yb); cudaFree(n->idx); cudaFree(n->loss);
+    cudaFree(n->fhat); cudaFree(n->dz); cudaFree(n->yb); cudaFree(n->loss);
     cudaFree(n->eidx); cudaFree(n->eloss); cudaFree(n->count); cudaFree(n->corr); cudaFree(n->pX);
     for (auto &e : n->ev)
         if (e) cudaEventDestroy(e);
@@ -961,7 +960,6 @@ int it_mlp_create(int32_t members, int32_t max_batch, it_mlp **out) {
         (e = cudaMalloc(&n->fhat, sizeof(float) * members * max_batch)) != cudaSuccess ||
         (e = cudaMalloc(&n->dz, sizeof(float) * members * max_batch)) != cudaSuccess ||
         (e = cudaMalloc(&n->yb, sizeof(float) * members * max_batch)) != cudaSuccess ||
-        (e = cudaMalloc(&n->idx, sizeof(int) * members * max_batch)) != cudaSuccess ||
         (e = cudaMalloc(&n->loss, sizeof(double) * members)) != cudaSuccess)
         return bail("mlp allocation");
     for (auto &v : n->side)
