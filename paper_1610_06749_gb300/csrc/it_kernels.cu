@@ -450,16 +450,19 @@ struct DepWindow { int x, nx, y, ny; };
 // cells from the window's start, so that a cell edge's error function is
 // evaluated once, by the lane that owns it, and the next lane takes it by
 // shuffle.  (A block per track and axis with two error functions per cell
-// took 74 us for 2000 tracks on 256x256, this takes 28.)
+// took 74 us for 2000 tracks on 256x256, this takes 28.)  Axes longer than
+// DEP_SEG cells are cut into nseg pieces, a warp each: one warp alone wrote
+// 500000 cells in 2.2 ms.
+constexpr int DEP_SEG = 31 * 32;
 __global__ void __launch_bounds__(128)
-deposit_tables_kernel(const double *__restrict__ tr, long long nt, double dx, int nx, int ny, int periodic,
+deposit_tables_kernel(const double *__restrict__ tr, long long nt, int nseg, double dx, int nx, int ny, int periodic,
                       double inv_W, double *__restrict__ wx, double *__restrict__ wy, DepWindow *__restrict__ win) {
     const long long unit = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    if (unit >= 2 * nt) return;
-    const long long t = unit >> 1;
-    const int axis = (int)(unit & 1);
-    const int n = axis ? ny : nx;
+    if (unit >= 2 * nt * nseg) return;
+    const long long t = unit / (2 * nseg);
+    const int rest = (int)(unit - t * (2 * nseg)), axis = rest & 1, seg = (rest >> 1) * DEP_SEG;
+    const int n = axis ? ny : nx, end = min(n, seg + DEP_SEG);   // cells [seg, end) of the walk
     const double ctr = tr[t * 4 + axis];
     const double b = tr[t * 4 + 3];
     const double f = axis ? 1.0 : tr[t * 4 + 2] * 1e7 * inv_W;   // ions per cm, on the x table
@@ -476,13 +479,13 @@ deposit_tables_kernel(const double *__restrict__ tr, long long nt, double dx, in
         start = c1 >= c0 ? (int)c0 : 0;
         count = c1 >= c0 ? (int)(c1 - c0 + 1) : 0;
     }
-    if (lane == 0) {
+    if (lane == 0 && seg == 0) {
         int *o = reinterpret_cast<int *>(win + t) + 2 * axis;
         o[0] = start;
         o[1] = count;
     }
     if (periodic && 2 * w + 1 > n) {   // a cell has several images: sum them, lowest first
-        for (int i = lane; i < n; i += 32) {
+        for (int i = seg + lane; i < end; i += 32) {
             double sum = 0.0;
             long long ii = i + n * (-floor_div(-(lo - i), n));   // first image >= lo
             for (; ii <= hi; ii += n)
@@ -494,7 +497,7 @@ deposit_tables_kernel(const double *__restrict__ tr, long long nt, double dx, in
     // cell m of the walk is cell (start + m) mod n; its unwrapped index is
     // first + m, and 31 cells a round share 32 edges
     const long long first = periodic ? lo : start;
-    for (int m0 = 0; m0 < n; m0 += 31) {
+    for (int m0 = seg; m0 < end; m0 += 31) {
         const int m = m0 + lane;
         double e = 0.0;
         if (m0 < count) e = m <= count ? erf(((double)(first + m) * dx - ctr) / b) : 0.0;
@@ -517,88 +520,98 @@ __device__ __forceinline__ bool window_hits(int start, int count, int t0, int tn
 
 constexpr int DEP_TILE = 8;       // 8 x 8 cells per CTA
 constexpr int DEP_LIST = 512;     // tracks gathered per pass
+constexpr size_t DEP_BLOCKS = 152 * 32 * 4;   // four rounds of resident blocks; fixed, so the sums are deterministic
 
 // plane[j][i] = sum_t N0_t wx[t][i] wy[t][j] / dx^2, tracks in index order.
 // Each CTA first lists (in index order) the tracks whose window reaches its
 // tile, then every cell sums over that list; tracks that miss the tile only
 // contribute zeros, so the per-cell sum is the same as over all tracks.
-// part[blockIdx] receives the tile's sum of the plane (FP64).  Bound by the
-// chain of additions per cell and by the scan; small tiles keep the lists
+// part[blockIdx] receives the sum of the plane over the block's tiles (FP64);
+// a block takes tiles blockIdx.x, blockIdx.x + gridDim.x, ... (one, up to
+// DEP_BLOCKS tiles; with a block each a single track on 4096x4096 took 770 us,
+// 192 so, most of it for 262144 FP64 reductions and the sum of the parts).
+// Bound by the chain of additions per cell and by the scan; small tiles keep the lists
 // short and give a 48x48 section 36 CTAs (16x16 tiles with 64-bit window
 // arithmetic in every scan: 93 us on 256x256 with 2000 tracks and 120 us on
 // 48x48 with up to 500; this: 23 and 30).
 __global__ void __launch_bounds__(DEP_TILE *DEP_TILE)
 deposit_plane_kernel(const DepWindow *__restrict__ win, const double *__restrict__ wx, const double *__restrict__ wy,
-                     long long nt, int nx, int ny, int periodic, double inv_dx2, double *__restrict__ plane,
-                     double *__restrict__ part) {
+                     long long nt, int nx, int ny, unsigned ntiles, int periodic, double inv_dx2,
+                     double *__restrict__ plane, double *__restrict__ part) {
     constexpr int NTH = DEP_TILE * DEP_TILE, NWARP = NTH / 32;
     __shared__ int list[DEP_LIST];
     __shared__ int wcount[NWARP];
     __shared__ double stage[16][16];   // [track][8 column weights, 8 row weights]
     __shared__ double red[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned ntx = (unsigned)(nx + DEP_TILE - 1) / DEP_TILE;   // tiles in raster order: gridDim.y ends at 65535
-    const int i0 = (int)(blockIdx.x % ntx) * DEP_TILE, j0 = (int)(blockIdx.x / ntx) * DEP_TILE;
-    const int tnx = min(DEP_TILE, nx - i0), tny = min(DEP_TILE, ny - j0);
-    const bool inside = (tid % DEP_TILE) < tnx && (tid / DEP_TILE) < tny;
-    const int i = i0 + (tid % DEP_TILE), j = j0 + (tid / DEP_TILE);
-    double sum = 0.0;
-    for (long long base = 0; base < nt;) {
-        // gather up to DEP_LIST candidates in index order, NTH tracks per round
-        int n = 0;
-        long long t0 = base;
-        for (; t0 < nt && n + NTH <= DEP_LIST; t0 += NTH) {
-            const long long t = t0 + tid;
-            bool hit = false;
-            if (t < nt) {
-                const DepWindow w = win[t];
-                hit = window_hits(w.x, w.nx, i0, tnx, nx, periodic != 0) &&
-                      window_hits(w.y, w.ny, j0, tny, ny, periodic != 0);
-            }
-            const unsigned bal = __ballot_sync(0xffffffffu, hit);
-            if (lane == 0) wcount[warp] = __popc(bal);
-            __syncthreads();
-            int before = 0, total = 0;
-#pragma unroll
-            for (int q = 0; q < NWARP; ++q) {
-                if (q < warp) before += wcount[q];
-                total += wcount[q];
-            }
-            if (hit) list[n + before + __popc(bal & ((1u << lane) - 1u))] = (int)t;
-            n += total;
-            __syncthreads();
-        }
-        // the listed tracks' weights on the tile's columns and rows, 16 tracks
-        // at a time through shared memory (the next 16 are loaded while these
-        // are added, in order)
-        double r[4];
-        auto fetch = [&](int q0) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int idx = tid + NTH * e, q = q0 + (idx >> 4), w = idx & 15;
-                r[e] = 0.0;
-                if (q < n) {
-                    const long long t = list[q];
-                    r[e] = w < DEP_TILE ? wx[t * nx + min(i0 + w, nx - 1)] : wy[t * ny + min(j0 + w - DEP_TILE, ny - 1)];
+    const unsigned ntx = (unsigned)(nx + DEP_TILE - 1) / DEP_TILE;   // tiles in raster order
+    double all = 0.0;   // this thread's cells of all the block's tiles
+    for (unsigned tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int i0 = (int)(tile % ntx) * DEP_TILE, j0 = (int)(tile / ntx) * DEP_TILE;
+        const int tnx = min(DEP_TILE, nx - i0), tny = min(DEP_TILE, ny - j0);
+        const bool inside = (tid % DEP_TILE) < tnx && (tid / DEP_TILE) < tny;
+        const int i = i0 + (tid % DEP_TILE), j = j0 + (tid / DEP_TILE);
+        double sum = 0.0;
+        for (long long base = 0; base < nt;) {
+            // gather up to DEP_LIST candidates in index order, NTH tracks per round
+            int n = 0;
+            long long t0 = base;
+            for (; t0 < nt && n + NTH <= DEP_LIST; t0 += NTH) {
+                const long long t = t0 + tid;
+                bool hit = false;
+                if (t < nt) {
+                    const DepWindow w = win[t];
+                    hit = window_hits(w.x, w.nx, i0, tnx, nx, periodic != 0) &&
+                          window_hits(w.y, w.ny, j0, tny, ny, periodic != 0);
                 }
+                const unsigned bal = __ballot_sync(0xffffffffu, hit);
+                if (lane == 0) wcount[warp] = __popc(bal);
+                __syncthreads();
+                int before = 0, total = 0;
+#pragma unroll
+                for (int q = 0; q < NWARP; ++q) {
+                    if (q < warp) before += wcount[q];
+                    total += wcount[q];
+                }
+                if (hit) list[n + before + __popc(bal & ((1u << lane) - 1u))] = (int)t;
+                n += total;
+                __syncthreads();
             }
-        };
-        fetch(0);
-        for (int q0 = 0; q0 < n; q0 += 16) {
-            __syncthreads();
+            // the listed tracks' weights on the tile's columns and rows, 16 tracks
+            // at a time through shared memory (the next 16 are loaded while these
+            // are added, in order)
+            double r[4];
+            auto fetch = [&](int q0) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) stage[(tid + NTH * e) >> 4][(tid + NTH * e) & 15] = r[e];
-            __syncthreads();
-            if (q0 + 16 < n) fetch(q0 + 16);
+                for (int e = 0; e < 4; ++e) {
+                    const int idx = tid + NTH * e, q = q0 + (idx >> 4), w = idx & 15;
+                    r[e] = 0.0;
+                    if (q < n) {
+                        const long long t = list[q];
+                        r[e] = w < DEP_TILE ? wx[t * nx + min(i0 + w, nx - 1)] : wy[t * ny + min(j0 + w - DEP_TILE, ny - 1)];
+                    }
+                }
+            };
+            fetch(0);
+            for (int q0 = 0; q0 < n; q0 += 16) {
+                __syncthreads();
 #pragma unroll
-            for (int t = 0; t < 16; ++t) sum = fma(stage[t][tid % DEP_TILE], stage[t][DEP_TILE + tid / DEP_TILE], sum);
+                for (int e = 0; e < 4; ++e) stage[(tid + NTH * e) >> 4][(tid + NTH * e) & 15] = r[e];
+                __syncthreads();
+                if (q0 + 16 < n) fetch(q0 + 16);
+#pragma unroll
+                for (int t = 0; t < 16; ++t) sum = fma(stage[t][tid % DEP_TILE], stage[t][DEP_TILE + tid / DEP_TILE], sum);
+            }
+            base = t0;
+            __syncthreads();
         }
-        base = t0;
-        __syncthreads();
+        const double v = sum * inv_dx2;
+        if (inside) {
+            plane[(size_t)j * nx + i] = v;
+            all += v;
+        }
     }
-    const double v = sum * inv_dx2;
-    if (inside) plane[(size_t)j * nx + i] = v;
-    double r[1] = {inside ? v : 0.0};
+    double r[1] = {all};
     block_sum<1>(r, red);
     if (tid == 0) part[blockIdx.x] = r[0];
 }
@@ -671,15 +684,17 @@ int launch_deposit(it_ctx *c, int64_t n, cudaStream_t s) {
     const int nx = c->g.nx, ny = c->g.ny;
     const bool periodic = c->p.lateral_bc == IT_PERIODIC;
     DepWindow *win = reinterpret_cast<DepWindow *>(c->d_tracks + 4 * n);   // after the track records
-    deposit_tables_kernel<<<(unsigned)((2 * n + 3) / 4), 128, 0, s>>>(c->d_tracks, n, c->dx, nx, ny, periodic,
-                                                                     1.0 / c->p.W_eV, c->d_wx, c->d_wy, win);
+    const int nseg = (std::max(nx, ny) + DEP_SEG - 1) / DEP_SEG;
+    deposit_tables_kernel<<<(unsigned)((2 * n * nseg + 3) / 4), 128, 0, s>>>(c->d_tracks, n, nseg, c->dx, nx, ny, periodic,
+                                                                            1.0 / c->p.W_eV, c->d_wx, c->d_wy, win);
     IT_CK(cudaGetLastError());
     const long long pn = (long long)nx * ny;
-    const size_t nparts = (size_t)((nx + DEP_TILE - 1) / DEP_TILE) * ((ny + DEP_TILE - 1) / DEP_TILE);
+    const size_t ntiles = (size_t)((nx + DEP_TILE - 1) / DEP_TILE) * ((ny + DEP_TILE - 1) / DEP_TILE);
+    const size_t nparts = std::min(ntiles, DEP_BLOCKS);
     // the tile sums go after the plane in the same scratch buffer
     double *part = c->d_plane + pn;
-    deposit_plane_kernel<<<(unsigned)nparts, DEP_TILE * DEP_TILE, 0, s>>>(win, c->d_wx, c->d_wy, n, nx, ny, periodic ? 1 : 0,
-                                                            1.0 / (c->dx * c->dx), c->d_plane, part);
+    deposit_plane_kernel<<<(unsigned)nparts, DEP_TILE * DEP_TILE, 0, s>>>(
+        win, c->d_wx, c->d_wy, n, nx, ny, (unsigned)ntiles, periodic ? 1 : 0, 1.0 / (c->dx * c->dx), c->d_plane, part);
     IT_CK(cudaGetLastError());
     const unsigned kchunks = (unsigned)((c->g.nz + DEP_KCHUNK - 1) / DEP_KCHUNK);
     if (c->prec == IT_FP32 && nx % 4 == 0)
