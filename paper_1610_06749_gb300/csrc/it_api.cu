@@ -578,8 +578,9 @@ int it_deposit_tracks_angled(it_ctx *c, int64_t n, const double *xy, const doubl
     IT_CK(cudaMemcpyAsync(c->d_angled, h.data(), sizeof(double) * 5 * n, cudaMemcpyHostToDevice, c->stream));
     rc = launch_deposit_angled(c, c->d_angled, n, c->d_angled + 5 * n, kBlocks,
                                tab > 0 ? c->d_angled + 5 * n + kBlocks : nullptr, c->stream);
+    const cudaError_t done = cudaStreamSynchronize(c->stream);   // the host records are released on return, failed or not
     if (rc) return rc;
-    IT_CK(cudaStreamSynchronize(c->stream));   // the host records are released on return
+    if (done != cudaSuccess) return cuda_fail(done, "cudaStreamSynchronize(tilted tracks)");
     return IT_OK;
 }
 

@@ -1070,9 +1070,12 @@ int it_mlp_set_data(it_mlp *n, int64_t count, const double *x, const double *y) 
     for (long long i = 0; i < count; ++i) hy[i] = (float)y[i];
     IT_CK(cudaMalloc(&n->X, sizeof(float) * hx.size()));
     IT_CK(cudaMalloc(&n->Y, sizeof(float) * hy.size()));
-    IT_CK(cudaMemcpyAsync(n->X, hx.data(), sizeof(float) * hx.size(), cudaMemcpyHostToDevice, n->stream));
-    IT_CK(cudaMemcpyAsync(n->Y, hy.data(), sizeof(float) * hy.size(), cudaMemcpyHostToDevice, n->stream));
-    IT_CK(cudaStreamSynchronize(n->stream));
+    cudaError_t e = cudaMemcpyAsync(n->X, hx.data(), sizeof(float) * hx.size(), cudaMemcpyHostToDevice, n->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(n->Y, hy.data(), sizeof(float) * hy.size(), cudaMemcpyHostToDevice, n->stream);
+    const cudaError_t done = cudaStreamSynchronize(n->stream);   // hx and hy are released on return, failed or not
+    if (e == cudaSuccess) e = done;
+    if (e != cudaSuccess) return cuda_fail(e, "training data");
     n->n_data = count;
     return IT_OK;
 }
